@@ -218,6 +218,9 @@ sinet_status sinet_compile_prefix_table(const uint32_t *h_net, const uint8_t *h_
  * bits, intervals, most toggle blocks of one bucket, and whether each form
  * fits shared memory. *bytes receives the image size; image (capacity bytes,
  * may be NULL to query the size) receives the image.
+ * The image ends in four words that locate the leaf form the kernels stage
+ * where it fits (leaves offset, leaf descriptors offset, descriptor bits, words
+ * a leaf; words 0 = the toggle form is staged).
  */
 sinet_status sinet_prefix_table_image(const uint32_t *h_net, const uint8_t *h_len, uint32_t n,
                                       uint8_t *image, size_t capacity, uint32_t *layout,

@@ -144,8 +144,9 @@ sinet_status zero_outputs(const sinet_hist_params *p, const sinet_hist_out *o, c
     return SINET_OK;
 }
 
-// Lookup form for a table: the staged interval form when it fits shared
-// memory, the per-length form on request, else global-memory intervals.
+// Lookup form for a table: the staged leaf form (or the toggle form, where
+// that is smaller) when it fits shared memory, the per-length form on request,
+// else global-memory intervals.
 int pick_lookup(const sinet_prefix_table *t, int32_t lookup, sinet_status *err) {
     *err = SINET_OK;
     if (lookup == SINET_LOOKUP_PML) {
@@ -153,12 +154,28 @@ int pick_lookup(const sinet_prefix_table *t, int32_t lookup, sinet_status *err) 
         return LK_PML;
     }
     if (!t->img.iv_fits_smem) return LK_INTERVAL_GLOBAL;
-    return t->host.toggle_form == 1 ? LK_TOGGLE1 : t->host.toggle_form == 2 ? LK_TOGGLE2 : LK_INTERVAL;
+    return staged_lookup(t);
+}
+
+int staged_lookup(const sinet_prefix_table *t) {
+    if (t->host.leaf_words) return t->host.leaf_words == 2 ? LK_LEAF2 : LK_LEAF4;
+    return toggle_lookup(t);
+}
+
+int toggle_lookup(const sinet_prefix_table *t) {
+    // a table in one block per bucket always has a leaf form no larger
+    return t->host.toggle_form == 2 ? LK_TOGGLE2 : LK_INTERVAL;
+}
+
+bool toggle_is_smaller(const sinet_prefix_table *t, int lk) {
+    return (lk == LK_LEAF2 || lk == LK_LEAF4) && t->host.toggle_form != 1 &&
+           t->img.iv_bytes + 16 < t->img.leaf_bytes;
 }
 
 static uint32_t table_smem(const sinet_prefix_table *t, int lk) {
     if (!t) return 0;
-    if (lk == LK_INTERVAL || lk == LK_TOGGLE1 || lk == LK_TOGGLE2) return t->img.iv_bytes;
+    if (lk == LK_LEAF2 || lk == LK_LEAF4) return t->img.leaf_bytes;
+    if (lk == LK_INTERVAL || lk == LK_TOGGLE2) return t->img.iv_bytes;
     if (lk == LK_PML) return t->img.pml_bytes;
     return 0;
 }
@@ -175,7 +192,8 @@ static const uint32_t kCacheSetBits = 9;
 // Bins per direction that fit a shared-memory tile (8 bytes per bin and
 // direction) after the staged table and the kernel's static shared memory.
 static uint32_t tile_capacity(const DeviceState *ds, uint32_t tsm) {
-    const size_t reserve = 1024;
+    // (the leaf form may be one 16-byte block larger than the toggle form)
+    const size_t reserve = 1008;
     const size_t used = ((tsm + 15u) & ~15u) + reserve;
     if (ds->smem_optin <= used) return 0;
     return (uint32_t)((ds->smem_optin - used) / 16) & ~3u;
@@ -325,7 +343,7 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
     c.status = ds->status;
     c.sm_count = ds->sm_count;
     const uint32_t tsm = table_smem(t, lk);
-    const uint32_t cap = tile_capacity(ds, tsm);
+    uint32_t cap = tile_capacity(ds, tsm);
 
     int strat = p->strategy;
     const TableArgs *watch = p->watch ? &p->watch->args : nullptr;
@@ -370,6 +388,11 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
         ct.block = p->block_threads ? (int)p->block_threads : 512;
         if (strat == SINET_STRAT_SMEM_FULL) {
             ta.tile_bins = (uint32_t)((p->n_bins + 3) & ~3ull);  // whole histogram
+            if (ta.tile_bins > cap && t && toggle_is_smaller(t, lk)) {
+                // fits beside the table's smaller form only
+                lk = toggle_lookup(t);
+                cap = tile_capacity(ds, table_smem(t, lk));
+            }
             if (ta.tile_bins > cap) return SINET_ERR_UNSUPPORTED;
             ta.full = 1;
             ta.margin = 0;
@@ -597,7 +620,10 @@ sinet_status sinet_build_prefix_table(const uint32_t *h_net, const uint8_t *h_le
     a.off_blocks = t->img.off_blocks;
     a.off_desc = t->img.off_desc;
     a.desc_bits = t->host.desc_bits;
-    a.toggle_form = t->host.toggle_form;
+    a.leaf_bytes = t->img.leaf_bytes;
+    a.off_leaves = t->img.off_leaves;
+    a.off_leaf_desc = t->img.off_leaf_desc;
+    a.leaf_bits = t->host.leaf_bits;
     a.off_lo = t->img.off_lo;
     a.off_hi = t->img.off_hi;
     a.off_idx32 = t->img.off_idx32;
@@ -646,8 +672,9 @@ sinet_status sinet_discriminate(const sinet_prefix_table *t, const uint32_t *d_s
     r.src = d_src;
     r.dst = d_dst;
     r.cls_out = d_class;
-    r.g = make_geom(n, {{d_src, 4}, {d_dst, 4}, {d_class, 1}});
+    r.g = make_geom(n, {{d_src, 4}, {d_dst, 4}});  // the class bytes follow in stores of their own width
     LaunchCfg c;
+    c.block = 512;
     c.stream = stream;
     c.status = ds->status;
     c.sm_count = ds->sm_count;

@@ -59,6 +59,11 @@ sinet_status check_params(const sinet_hist_params *p);
 sinet_status check_out(const sinet_hist_out *o);
 HistArgs make_hist(const sinet_hist_params *p, const sinet_hist_out *o);
 sinet_status zero_outputs(const sinet_hist_params *p, const sinet_hist_out *o, cudaStream_t s);
+// The shared-memory form of a table that has one: its leaf form, else its toggle form.
+int staged_lookup(const sinet_prefix_table *t);
+int toggle_lookup(const sinet_prefix_table *t);
+// The table's toggle form takes less shared memory than the form `lk`.
+bool toggle_is_smaller(const sinet_prefix_table *t, int lk);
 int pick_lookup(const sinet_prefix_table *t, int32_t lookup, sinet_status *err);
 
 }  // namespace sinet

@@ -17,7 +17,7 @@ uint32_t batch_smem(const DeviceState *ds) {
     // kernel's static shared memory (descriptor copy, slice starts, counters)
     // stays below 5 KB
     const size_t per_cta = ds->smem_per_sm / 2;
-    size_t v = per_cta > 6144 ? per_cta - 6144 : 0;
+    size_t v = per_cta > 6128 ? per_cta - 6128 : 0;
     v = std::min(v, ds->smem_optin);
     return (uint32_t)(v & ~(size_t)15);
 }
@@ -85,13 +85,24 @@ sinet_status plan_slice(const sinet_batch_slice &u, const DeviceState *ds, uint3
     d.h.status = ds->status;
     // the toggle form is staged when it leaves room for the hot-key cache
     uint32_t staged = 0;
-    if (t->img.iv_fits_smem && round16(t->img.iv_bytes) + kBatchCacheBytes <= smem) {
+    const uint32_t form_bytes = t->host.leaf_words ? t->img.leaf_bytes : t->img.iv_bytes;
+    if (t->img.iv_fits_smem && round16(form_bytes) + kBatchCacheBytes <= smem) {
+        staged = round16(form_bytes);
+        d.lk = (uint32_t)staged_lookup(t);
+    } else if (t->img.iv_fits_smem && toggle_is_smaller(t, staged_lookup(t)) &&
+               round16(t->img.iv_bytes) + kBatchCacheBytes <= smem) {
         staged = round16(t->img.iv_bytes);
-        d.lk = t->host.toggle_form == 1 ? LK_TOGGLE1 : t->host.toggle_form == 2 ? LK_TOGGLE2 : LK_INTERVAL;
+        d.lk = (uint32_t)toggle_lookup(t);
     } else {
         d.lk = LK_INTERVAL_GLOBAL;
     }
     const uint64_t T = (u.params.n_bins + 3) & ~3ull;
+    if (staged && staged + 16 * T > smem && toggle_is_smaller(t, (int)d.lk) &&
+        round16(t->img.iv_bytes) + 16 * T <= smem) {
+        // the whole-histogram tile fits beside the table's smaller form only
+        staged = round16(t->img.iv_bytes);
+        d.lk = (uint32_t)toggle_lookup(t);
+    }
     d.tile_bins = (uint32_t)std::min<uint64_t>(T, 0xFFFFFFFFull);
     ps.tile_fits = staged + 16 * T <= smem;
     d.zero = u.params.accumulate ? 0u : 1u;

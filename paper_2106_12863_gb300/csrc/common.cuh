@@ -212,15 +212,13 @@ struct PmlView {
 // Toggle form (shared memory). For the bucket of the top `bits` address bits,
 // desc gives the membership of the bucket's first address (bit 31) and the
 // blocks holding the ascending offsets t at which membership flips, stored as
-// t - 1 (< 2^24; padded with 0x7FFFFFFF): NB = 1, one block (bits 0-14);
-// NB = 2, two blocks (bits 0-14, 15-29; the second may be the all-padding
+// t - 1 (< 2^24; padded with 0x7FFFFFFF): NB = 2, two blocks (bits 0-14, 15-29; the second may be the all-padding
 // block 0); NB = 0, consecutive blocks (bits 0-23 first, 24-27 count). A
 // toggle lies at or below the address's offset `off` exactly when
 // (t - 1) - off is negative as a 32-bit signed value, so the XOR of the four
 // differences (and of desc, for the start state) carries the membership in
-// bit 31. Pure buckets use block 0, so for NB = 1, 2 every lookup is the same
-// branch-free sequence of loads and integer operations.
-template <int NB>  // 1 or 2 blocks per bucket, loaded unconditionally; 0: as counted
+// bit 31. Serves the tables whose leaf form (below) would take more room.
+template <int NB>  // 2 blocks per bucket; 0: as counted
 struct ToggleView {
     const uint4 *blocks;
     const uint32_t *desc;
@@ -254,13 +252,49 @@ struct ToggleView {
                 x = d[i];
                 const uint32_t b1 = d[i] & 0x7FFFu;
                 if (b1) x ^= parity_bits(blocks[b1], off);
-                if (NB == 2) {
-                    const uint32_t b2 = (d[i] >> 15) & 0x7FFFu;
-                    if (b2) x ^= parity_bits(blocks[b2], off);
-                }
+                const uint32_t b2 = (d[i] >> 15) & 0x7FFFu;
+                if (b2) x ^= parity_bits(blocks[b2], off);
             }
             in[i] = x >> 31;
         }
+    }
+};
+
+// Leaf form (shared memory, [leaves | descriptors], see table_host.h): every
+// address takes one descriptor and one leaf of W words, two dependent loads
+// and no branch, where the toggle form's second block and its skipped loads
+// cost branches and up to two 16-byte loads. On 200 M records against the
+// paper-shaped 2,000-prefix list the classification alone went from 563 to
+// 355 us with it (and is now bound by the shared-memory wavefronts of the
+// two divergent loads, about eight a warp and address).
+template <int W>
+struct LeafView {
+    static_assert(W == 2 || W == 4, "leaf words");
+    const uint8_t *leaves;
+    const uint32_t *desc;
+    uint32_t shift;     // 32 - bits
+    uint32_t off_mask;  // (1 << shift) - 1
+
+    // bit 31 of the result is the membership of the address in the leaf that d names
+    __device__ __forceinline__ uint32_t sign(uint32_t d, uint32_t a) const {
+        const uint32_t off = a & off_mask;
+        const uint32_t leaf = __funnelshift_r(off, 0u, d);  // off >> (d & 31)
+        const uint8_t *p = leaves + (d >> 8) + leaf * (4 * W);
+        if (W == 2) {
+            const uint2 w = *reinterpret_cast<const uint2 *>(p);
+            return (w.x - off) ^ (w.y - off);
+        }
+        const uint4 w = *reinterpret_cast<const uint4 *>(p);
+        return (w.x - off) ^ (w.y - off) ^ (w.z - off) ^ (w.w - off);
+    }
+
+    template <int N>
+    __device__ __forceinline__ void signs_n(const uint32_t (&a)[N], uint32_t (&in)[N]) const {
+        uint32_t d[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) d[i] = desc[a[i] >> shift];
+#pragma unroll
+        for (int i = 0; i < N; ++i) in[i] = sign(d[i], a[i]);
     }
 };
 
@@ -268,7 +302,9 @@ struct ToggleView {
 struct TableArgs {
     const uint8_t *image;     // device image base
     uint32_t iv_bytes;        // [blocks | desc] staged for the toggle form
-    uint32_t off_blocks, off_desc, desc_bits, toggle_form;
+    uint32_t off_blocks, off_desc, desc_bits;
+    uint32_t leaf_bytes;      // [leaves | descriptors] staged for the leaf form
+    uint32_t off_leaves, off_leaf_desc, leaf_bits;
     uint32_t off_lo, off_hi, off_idx32;  // global-memory interval form
     uint32_t n_iv, index_bits;
     uint32_t off_nets, off_groups, pml_bytes, n_groups;

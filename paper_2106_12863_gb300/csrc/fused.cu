@@ -10,37 +10,75 @@
 namespace sinet {
 
 // ---------------------------------------------------------------------------
-// Algorithm 1 only.
+// Algorithm 1 only. Each thread takes quads of records; a quad's eight
+// memberships stay sign bits until they are packed into its four class bytes
+// (byte permutes that replicate the sign), and the classes are counted by
+// population counts of those bytes. `align`: log2 of the alignment of the class
+// bytes of a full quad (2: one 32-bit store; 1, 0: smaller stores, when the
+// class array starts at another offset than the addresses).
+__device__ __forceinline__ uint32_t signs4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    uint32_t lo, hi, w;  // 0xFF per byte whose word has bit 31 set
+    asm("prmt.b32 %0, %1, %2, 0xFB;" : "=r"(lo) : "r"(a), "r"(b));
+    asm("prmt.b32 %0, %1, %2, 0xFB;" : "=r"(hi) : "r"(c), "r"(d));
+    asm("prmt.b32 %0, %1, %2, 0x5410;" : "=r"(w) : "r"(lo), "r"(hi));
+    return w;
+}
+
 template <int LK>
-__global__ void __launch_bounds__(256) k_discriminate(RecArgs r, TableArgs t, uint64_t *counts,
-                                                      uint32_t *status) {
+__global__ void __launch_bounds__(512, LK == LK_INTERVAL ? 2 : 3) k_discriminate(RecArgs r, TableArgs t, uint32_t align, uint64_t *counts,
+                                                         uint32_t *status) {
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ uint64_t bar;
     Classifier<LK> C;
     if (!C.init(t, smem, &bar, status)) return;  // table not staged: the status word says so
     const uint64_t pol = policy_evict_first();
-    uint32_t cc[4] = {0, 0, 0, 0}, oor[2] = {0, 0};
+    uint32_t n_rec = 0, n_src = 0, n_dst = 0, n_both = 0;  // 8 x the thread's records of each kind
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; q < r.g.quads; q += stride) {
         Quad Q;
         load_quad<false, true, false, false>(r, q, pol, Q);
-        classify_quad<LK>(C, Q);
+        uint32_t s[4], d[4];
+        C.template sign_n<4>(Q.src, s);
+        C.template sign_n<4>(Q.dst, d);
+        uint32_t S = signs4(s[0], s[1], s[2], s[3]), D = signs4(d[0], d[1], d[2], d[3]);
+        const int64_t base = quad_base(r.g, q);
+        if (Q.valid == 0xFu) {
+            if (r.cls_out) {
+                const uint32_t w = (S & 0x01010101u) | (D & 0x02020202u);
+                uint8_t *p = r.cls_out + base;
+                if (align == 2) {
+                    *reinterpret_cast<uint32_t *>(p) = w;
+                } else if (align == 1) {
+                    *reinterpret_cast<uint16_t *>(p) = (uint16_t)w;
+                    *reinterpret_cast<uint16_t *>(p + 2) = (uint16_t)(w >> 16);
+                } else {
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (Q.valid >> j & 1u) bump_class(cc, Q.cls[j]);
-        if (r.cls_out) {
-            const int64_t base = quad_base(r.g, q);
-            if (Q.valid == 0xFu && quad_full(r.g, base)) {
-                uint32_t w = Q.cls[0] | Q.cls[1] << 8 | Q.cls[2] << 16 | Q.cls[3] << 24;
-                *reinterpret_cast<uint32_t *>(r.cls_out + base) = w;
-            } else {
+                    for (int j = 0; j < 4; ++j) p[j] = (uint8_t)(w >> (8 * j));
+                }
+            }
+        } else {
+            const uint32_t m = signs4(Q.valid << 31, Q.valid << 30, Q.valid << 29, Q.valid << 28);
+            S &= m;
+            D &= m;
+            if (r.cls_out) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    if (Q.valid >> j & 1u) r.cls_out[base + j] = (uint8_t)Q.cls[j];
+                    if (Q.valid >> j & 1u) r.cls_out[base + j] = (uint8_t)(((S >> (8 * j)) & 1u) | ((D >> (8 * j)) & 2u));
             }
         }
+        n_rec += 8 * __popc(Q.valid);
+        n_src += __popc(S);
+        n_dst += __popc(D);
+        n_both += __popc(S & D);
     }
-    flush_counters(counts, cc, oor, false);
+    // at most 2^40 records over at least one 512-thread CTA per SM: a thread's counts stay below 2^28
+    const uint32_t v[4] = {n_rec - n_src - n_dst + n_both, n_src - n_both, n_dst - n_both, n_both};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t sum = __reduce_add_sync(kFull, v[k] / 8);
+        if ((threadIdx.x & 31) == 0 && sum)
+            atomicAdd(reinterpret_cast<unsigned long long *>(counts + k), (unsigned long long)sum);
+    }
 }
 
 // Watch list (the blocklist views of Section 6, as a filter): a record whose
@@ -349,16 +387,20 @@ cudaError_t run_discriminate(int lk, const RecArgs &r, const TableArgs &t, uint6
                              const LaunchCfg &c) {
     int grid = 0;
     cudaError_t e;
+    // full quads start 4-record aligned in the addresses, not always in the class array
+    const uintptr_t at = (uintptr_t)r.cls_out + (uintptr_t)(intptr_t)r.g.shift;
+    const uint32_t align = at % 4 == 0 ? 2u : at % 2 == 0 ? 1u : 0u;
     switch (lk) {
 #define SINET_DISC(L)                                                                           \
     case L: {                                                                                   \
         size_t smem = Classifier<L>::smem_bytes(t);                                             \
         if ((e = launch(k_discriminate<L>, smem, c, grid)) != cudaSuccess) return e;            \
-        k_discriminate<L><<<grid, c.block, smem, c.stream>>>(r, t, counts, c.status);           \
+        k_discriminate<L><<<grid, c.block, smem, c.stream>>>(r, t, align, counts, c.status);    \
         break;                                                                                  \
     }
         SINET_DISC(LK_INTERVAL)
-        SINET_DISC(LK_TOGGLE1)
+        SINET_DISC(LK_LEAF2)
+        SINET_DISC(LK_LEAF4)
         SINET_DISC(LK_TOGGLE2)
         SINET_DISC(LK_PML)
         SINET_DISC(LK_INTERVAL_GLOBAL)
@@ -386,13 +428,15 @@ cudaError_t run_fused_atomic(int lk, bool agg, const RecArgs &r, const TableArgs
     }
 #define SINET_ATOM2(L, WA) SINET_ATOM(L, true, WA) SINET_ATOM(L, false, WA)
     SINET_ATOM2(LK_INTERVAL, false)
-    SINET_ATOM2(LK_TOGGLE1, false)
+    SINET_ATOM2(LK_LEAF2, false)
+    SINET_ATOM2(LK_LEAF4, false)
     SINET_ATOM2(LK_TOGGLE2, false)
     SINET_ATOM2(LK_PML, false)
     SINET_ATOM2(LK_INTERVAL_GLOBAL, false)
     SINET_ATOM2(LK_CLASS_IN, false)
     SINET_ATOM2(LK_INTERVAL, true)
-    SINET_ATOM2(LK_TOGGLE1, true)
+    SINET_ATOM2(LK_LEAF2, true)
+    SINET_ATOM2(LK_LEAF4, true)
     SINET_ATOM2(LK_TOGGLE2, true)
     SINET_ATOM2(LK_INTERVAL_GLOBAL, true)
 #undef SINET_ATOM2
@@ -414,8 +458,10 @@ cudaError_t run_fused_tile(int lk, const RecArgs &r, const TableArgs &t, const H
     }
     SINET_TILE(LK_INTERVAL, true)
     SINET_TILE(LK_INTERVAL, false)
-    SINET_TILE(LK_TOGGLE1, true)
-    SINET_TILE(LK_TOGGLE1, false)
+    SINET_TILE(LK_LEAF2, true)
+    SINET_TILE(LK_LEAF2, false)
+    SINET_TILE(LK_LEAF4, true)
+    SINET_TILE(LK_LEAF4, false)
     SINET_TILE(LK_TOGGLE2, true)
     SINET_TILE(LK_TOGGLE2, false)
     SINET_TILE(LK_PML, true)

@@ -63,7 +63,7 @@ struct BatchSlice {
     RecArgs r;
     TableArgs t;
     HistArgs h;
-    uint32_t lk;         // LK_TOGGLE1, LK_TOGGLE2, LK_INTERVAL or LK_INTERVAL_GLOBAL
+    uint32_t lk;         // LK_LEAF2, LK_LEAF4, LK_TOGGLE2, LK_INTERVAL or LK_INTERVAL_GLOBAL
     uint32_t strat;      // BS_*
     uint32_t tile_bins;  // BS_TILE: bins per direction of the tile (>= n_bins, multiple of 4)
     uint32_t zero;       // 1: the outputs are zeroed by the launch (not accumulated into)

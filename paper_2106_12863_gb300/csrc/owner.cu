@@ -485,8 +485,10 @@ static cudaError_t launch_owner_pair(const RecArgs &r, const TableArgs &t, const
 #define SINET_OWN_FORMS(X)        \
     X(LK_INTERVAL, true)          \
     X(LK_INTERVAL, false)         \
-    X(LK_TOGGLE1, true)           \
-    X(LK_TOGGLE1, false)          \
+    X(LK_LEAF2, true)             \
+    X(LK_LEAF2, false)            \
+    X(LK_LEAF4, true)             \
+    X(LK_LEAF4, false)            \
     X(LK_TOGGLE2, true)           \
     X(LK_TOGGLE2, false)          \
     X(LK_PML, true)               \

@@ -1253,7 +1253,8 @@ cudaError_t run_partition(int lk, const RecArgs &r, const TableArgs &t, const Hi
     if ((e = cudaMemsetAsync(d.page_fill, 0, 4ull * d.dyn_base, c.stream)) != cudaSuccess) return e;
     switch (lk) {
         case LK_INTERVAL: e = launch_lk<LK_INTERVAL>(r, t, h, P, c); break;
-        case LK_TOGGLE1: e = launch_lk<LK_TOGGLE1>(r, t, h, P, c); break;
+        case LK_LEAF2: e = launch_lk<LK_LEAF2>(r, t, h, P, c); break;
+        case LK_LEAF4: e = launch_lk<LK_LEAF4>(r, t, h, P, c); break;
         case LK_TOGGLE2: e = launch_lk<LK_TOGGLE2>(r, t, h, P, c); break;
         case LK_PML: e = launch_lk<LK_PML>(r, t, h, P, c); break;
         case LK_INTERVAL_GLOBAL: e = launch_lk<LK_INTERVAL_GLOBAL>(r, t, h, P, c); break;

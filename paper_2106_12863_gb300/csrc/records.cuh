@@ -6,10 +6,11 @@
 
 namespace sinet {
 
-// Lookup kinds: LK_INTERVAL / LK_TOGGLE1 / LK_TOGGLE2 are the shared-memory
-// toggle form with a variable / one / two blocks per bucket.
-enum : int { LK_INTERVAL = 0, LK_PML = 1, LK_INTERVAL_GLOBAL = 2, LK_CLASS_IN = 3, LK_TOGGLE1 = 4,
-             LK_TOGGLE2 = 5 };
+// Lookup kinds: LK_LEAF2 / LK_LEAF4 are the shared-memory leaf form with two /
+// four words a leaf; LK_TOGGLE2 / LK_INTERVAL the toggle form with two / a
+// variable number of blocks per bucket, for tables without a leaf form.
+enum : int { LK_INTERVAL = 0, LK_PML = 1, LK_INTERVAL_GLOBAL = 2, LK_CLASS_IN = 3, LK_LEAF2 = 4,
+             LK_TOGGLE2 = 5, LK_LEAF4 = 6 };
 
 struct RecArgs {
     const uint64_t *ts;
@@ -67,6 +68,13 @@ struct ToggleClassifier {
     __device__ __forceinline__ void in_n(const uint32_t (&a)[N], uint32_t (&r)[N]) const {
         v.template contains_n<N>(a, r);
     }
+    // membership in bit 31
+    template <int N>
+    __device__ __forceinline__ void sign_n(const uint32_t (&a)[N], uint32_t (&r)[N]) const {
+        in_n<N>(a, r);
+#pragma unroll
+        for (int i = 0; i < N; ++i) r[i] <<= 31;
+    }
     // in_n for a whole converged warp: when no lane's address falls in a
     // bucket with blocks (the common case: most buckets are pure), the
     // descriptors' parity bits are the answers and one vote replaces the
@@ -77,7 +85,7 @@ struct ToggleClassifier {
             v.template contains_n<N>(a, r);
             return;
         }
-        constexpr uint32_t kBlocks = NB == 2 ? 0x3FFFFFFFu : 0x7FFFu;
+        constexpr uint32_t kBlocks = 0x3FFFFFFFu;
         uint32_t d[N], any = 0;
 #pragma unroll
         for (int i = 0; i < N; ++i) {
@@ -95,9 +103,59 @@ struct ToggleClassifier {
 template <>
 struct Classifier<LK_INTERVAL> : ToggleClassifier<0> {};
 template <>
-struct Classifier<LK_TOGGLE1> : ToggleClassifier<1> {};
-template <>
 struct Classifier<LK_TOGGLE2> : ToggleClassifier<2> {};
+
+template <int W>
+struct LeafClassifier {
+    LeafView<W> v;
+    __device__ __forceinline__ bool init(const TableArgs &t, uint8_t *smem, uint64_t *bar,
+                                         uint32_t *status) {
+        const bool ok = stage_to_smem(smem, t.image + t.off_leaves, t.leaf_bytes, bar, status);
+        attach(t, smem);
+        return ok;
+    }
+    __device__ __forceinline__ void attach(const TableArgs &t, const uint8_t *smem) {
+        v.leaves = smem;
+        v.desc = reinterpret_cast<const uint32_t *>(smem + (t.off_leaf_desc - t.off_leaves));
+        v.shift = 32 - t.leaf_bits;
+        v.off_mask = (1u << v.shift) - 1u;
+    }
+    static __host__ __device__ uint32_t smem_bytes(const TableArgs &t) { return t.leaf_bytes; }
+    template <int N>
+    __device__ __forceinline__ void sign_n(const uint32_t (&a)[N], uint32_t (&r)[N]) const {
+        v.template signs_n<N>(a, r);
+    }
+    template <int N>
+    __device__ __forceinline__ void in_n(const uint32_t (&a)[N], uint32_t (&r)[N]) const {
+        v.template signs_n<N>(a, r);
+#pragma unroll
+        for (int i = 0; i < N; ++i) r[i] >>= 31;
+    }
+    // for a whole converged warp: when every lane's buckets are pure, the
+    // descriptors name one of the two pure leaves and one vote replaces the
+    // leaf loads
+    template <int N>
+    __device__ __forceinline__ void in_n_warp(const uint32_t (&a)[N], uint32_t (&r)[N]) const {
+        constexpr uint32_t kIn = 4u * W << 8, kMixed = ~(2 * kIn - 1);
+        uint32_t d[N], any = 0;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            d[i] = v.desc[a[i] >> v.shift];
+            any |= d[i];
+        }
+        if (__any_sync(kFull, any & kMixed)) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) r[i] = v.sign(d[i], a[i]) >> 31;
+            return;
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i) r[i] = (d[i] & kIn) ? 1u : 0u;
+    }
+};
+template <>
+struct Classifier<LK_LEAF2> : LeafClassifier<2> {};
+template <>
+struct Classifier<LK_LEAF4> : LeafClassifier<4> {};
 
 template <>
 struct Classifier<LK_PML> {
@@ -115,6 +173,13 @@ struct Classifier<LK_PML> {
     __device__ __forceinline__ void in_n(const uint32_t (&a)[N], uint32_t (&r)[N]) const {
 #pragma unroll
         for (int i = 0; i < N; ++i) r[i] = v.contains(a[i]);
+    }
+    // membership in bit 31
+    template <int N>
+    __device__ __forceinline__ void sign_n(const uint32_t (&a)[N], uint32_t (&r)[N]) const {
+        in_n<N>(a, r);
+#pragma unroll
+        for (int i = 0; i < N; ++i) r[i] <<= 31;
     }
     template <int N>
     __device__ __forceinline__ void in_n_warp(const uint32_t (&a)[N], uint32_t (&r)[N]) const {
@@ -141,6 +206,13 @@ struct Classifier<LK_INTERVAL_GLOBAL> {
     __device__ __forceinline__ void in_n(const uint32_t (&a)[N], uint32_t (&r)[N]) const {
 #pragma unroll
         for (int i = 0; i < N; ++i) r[i] = v.contains(a[i]);
+    }
+    // membership in bit 31
+    template <int N>
+    __device__ __forceinline__ void sign_n(const uint32_t (&a)[N], uint32_t (&r)[N]) const {
+        in_n<N>(a, r);
+#pragma unroll
+        for (int i = 0; i < N; ++i) r[i] <<= 31;
     }
     template <int N>
     __device__ __forceinline__ void in_n_warp(const uint32_t (&a)[N], uint32_t (&r)[N]) const {

@@ -469,9 +469,10 @@ cudaError_t run_sort_reduce(int lk, const RecArgs &r, const TableArgs &t, const 
     if (e != cudaSuccess) return e;
     if (r.g.quads == 0) return cudaSuccess;
 
-    const uint32_t tsm = (lk == LK_INTERVAL || lk == LK_TOGGLE1 || lk == LK_TOGGLE2 ? Classifier<LK_INTERVAL>::smem_bytes(t)
-                          : lk == LK_PML    ? Classifier<LK_PML>::smem_bytes(t)
-                                            : 0u);
+    const uint32_t tsm = (lk == LK_INTERVAL || lk == LK_TOGGLE2 ? Classifier<LK_INTERVAL>::smem_bytes(t)
+                          : lk == LK_LEAF2 || lk == LK_LEAF4 ? Classifier<LK_LEAF2>::smem_bytes(t)
+                          : lk == LK_PML ? Classifier<LK_PML>::smem_bytes(t)
+                                         : 0u);
     const size_t smem = ((tsm + 15u) & ~15u) + 8ull * kEmitRecords * (h.two_dir ? 2 : 1);
     switch (lk) {
 #define SINET_EMIT(L)                                                                          \
@@ -482,7 +483,8 @@ cudaError_t run_sort_reduce(int lk, const RecArgs &r, const TableArgs &t, const 
                                                                               plan.emit_tiles, c.status); \
         break;
         SINET_EMIT(LK_INTERVAL)
-        SINET_EMIT(LK_TOGGLE1)
+        SINET_EMIT(LK_LEAF2)
+        SINET_EMIT(LK_LEAF4)
         SINET_EMIT(LK_TOGGLE2)
         SINET_EMIT(LK_PML)
         SINET_EMIT(LK_INTERVAL_GLOBAL)

@@ -26,6 +26,86 @@ static uint32_t iv_image_bytes(uint32_t n_iv, uint32_t k) {
     return pad16(4 * n_iv) * 2 + pad16(2 * ((1u << k) + 1));
 }
 
+// Fills the leaf form (table_host.h) if it fits `budget` bytes: two words a
+// leaf where that fits, else four; within a width, the bucket bits that take
+// the least room. The budget is never below the toggle form's size plus one
+// block, so a one-block toggle table always has a four-word leaf form (its
+// buckets need no cut, and the second pure leaf is the extra block).
+static void build_leaves(TableHost &t, size_t budget) {
+    // toggles in (0, 2^32): where membership flips
+    std::vector<uint32_t> tog;
+    for (size_t i = 0; i < t.lo.size(); i++) {
+        if (t.lo[i]) tog.push_back(t.lo[i]);
+        if (t.hi[i] != 0xFFFFFFFFu) tog.push_back(t.hi[i] + 1);
+    }
+    const bool first_in = !t.lo.empty() && t.lo[0] == 0;
+    const size_t n = tog.size();
+    t.leaf_words = 0;
+    for (uint32_t words : {2u, 4u}) {
+        // a leaf of 2^s addresses holds tog[i] .. tog[i + words] strictly inside
+        // (a toggle on its first address is the start state instead) exactly
+        // when tog[i] - 1 and tog[i + words] agree above bit s: it must be cut
+        // to the highest bit in which they differ
+        std::vector<uint8_t> cut(n > words ? n - words : 0);
+        for (size_t i = 0; i < cut.size(); i++) {
+            uint32_t d = (tog[i] - 1) ^ tog[i + words], s = 31;
+            while (!(d >> s)) s--;
+            cut[i] = (uint8_t)s;
+        }
+        uint32_t best_bits = 0;
+        size_t best = budget + 1;
+        std::vector<uint8_t> size_log2, best_log2;  // per bucket: leaf size, or 0xFF when pure
+        for (uint32_t kb = 6; kb <= 14; kb++) {
+            const uint32_t sh = 32 - kb, m = (1u << sh) - 1;
+            size_log2.assign(1u << kb, 0xFF);
+            for (uint32_t v : tog)
+                if (v & m) size_log2[v >> sh] = (uint8_t)sh;
+            for (size_t i = 0; i < cut.size(); i++)
+                if (cut[i] < sh) {
+                    uint8_t &s = size_log2[tog[i + words] >> sh];
+                    s = std::min(s, cut[i]);
+                }
+            size_t leaves = 2;
+            for (uint8_t s : size_log2)
+                if (s != 0xFF) leaves += (size_t)1 << (sh - s);
+            const size_t bytes = ((4 * words * leaves + 15) & ~(size_t)15) + (4ull << kb);
+            if (bytes < best) {
+                best = bytes;
+                best_bits = kb;
+                best_log2 = size_log2;
+            }
+        }
+        if (!best_bits) continue;
+        const uint32_t sh = 32 - best_bits;
+        t.leaf_bits = best_bits;
+        t.leaf_words = words;
+        t.leaf_desc.assign(1u << best_bits, 0);
+        t.leaves.assign(2 * words, 0x7FFFFFFFu);
+        t.leaves[words] = 0xFFFFFFFFu;  // the pure leaf that is inside
+        size_t j = 0;  // toggles at or below the current leaf's first address
+        for (uint32_t b = 0; b < (1u << best_bits); b++) {
+            const uint64_t start = (uint64_t)b << sh, end = start + (1ull << sh);
+            while (j < n && tog[j] <= start) j++;
+            if (best_log2[b] == 0xFF) {
+                t.leaf_desc[b] = (((j & 1) != 0) != first_in ? 4 * words : 0u) << 8 | sh;
+                continue;
+            }
+            const uint32_t s = best_log2[b];
+            t.leaf_desc[b] = (uint32_t)(4 * t.leaves.size()) << 8 | s;
+            for (uint64_t a = start; a < end; a += 1ull << s) {
+                while (j < n && tog[j] <= a) j++;
+                const uint32_t in = ((j & 1) != 0) != first_in;
+                for (uint32_t k = 0; k < words; k++) {
+                    const bool here = j + k < n && tog[j + k] < a + (1ull << s);
+                    const uint32_t w = here ? (uint32_t)(tog[j + k] - start - 1) : 0x7FFFFFFFu;
+                    t.leaves.push_back(w ^ (k == 0 ? in << 31 : 0u));
+                }
+            }
+        }
+        return;
+    }
+}
+
 int compile_table(const uint32_t *net, const uint8_t *len, uint32_t n, uint32_t index_bits,
                   TableHost &t) {
     if (n > (1u << 24)) return SINET_ERR_TABLE_TOO_LARGE;
@@ -187,6 +267,8 @@ int compile_table(const uint32_t *net, const uint8_t *len, uint32_t n, uint32_t 
         form = 0;
     }
     build_toggles(kb, form, true);
+    const size_t toggle_bytes = pad16(4 * (uint32_t)t.blocks.size()) + pad16(4 * (uint32_t)t.desc.size());
+    if (t.max_blocks <= 15 && toggle_bytes <= kSmemTableBudget) build_leaves(t, std::max<size_t>(kLeafBudget, toggle_bytes + 16));
     return SINET_OK;
 }
 
@@ -214,6 +296,16 @@ std::vector<uint8_t> serialise(const TableHost &t, TableImage &img) {
     off += pad16(4 * n_pairs);
     img.off_idx32 = off;
     off += pad16(4 * nb1);
+    // the leaf form, and after it a trailer of four words saying where it is:
+    // {off_leaves, off_leaf_desc, leaf_bits, leaf_words}
+    if (t.leaf_words) {
+        img.off_leaves = off;
+        off += pad16(4 * (uint32_t)t.leaves.size());
+        img.off_leaf_desc = off;
+        off += pad16(4 * (uint32_t)t.leaf_desc.size());
+        img.leaf_bytes = off - img.off_leaves;
+    }
+    off += 16;
     img.total = off;
 
     std::vector<uint8_t> buf(img.total, 0);
@@ -237,6 +329,12 @@ std::vector<uint8_t> serialise(const TableHost &t, TableImage &img) {
         g[4 * i + 3] = 0;
     }
     std::memcpy(buf.data() + img.off_idx32, t.index.data(), 4 * nb1);
+    if (t.leaf_words) {
+        std::memcpy(buf.data() + img.off_leaves, t.leaves.data(), 4 * t.leaves.size());
+        std::memcpy(buf.data() + img.off_leaf_desc, t.leaf_desc.data(), 4 * t.leaf_desc.size());
+    }
+    const uint32_t trailer[4] = {img.off_leaves, img.off_leaf_desc, t.leaf_bits, t.leaf_words};
+    std::memcpy(buf.data() + img.total - 16, trailer, 16);
     return buf;
 }
 
