@@ -83,28 +83,27 @@ typedef enum {
                                       ordered: 8 bytes per range, 4 per CTA, 32 per queued item
                                       (at most one per range plus one per 32,767 records). At most
                                       512 threads per block. */
-    SINET_STRAT_PARTITION = 8      /* hot/cold partition, for unsorted input over histograms far
-                                      larger than L2 (Section 5's map-reduce with the reduction
-                                      kept on chip): a strided sample of about n / 4,096 records
-                                      ranks the bins; the most sampled ones (up to 16,384 slots,
-                                      as shared memory allows) are summed in shared memory by
-                                      every CTA; every other routed update is appended as an
-                                      8-byte (bin, direction, bytes) entry to a page of its
-                                      bin range, and a cooperative second kernel sorts the pages
-                                      by owner CTA in place and has each CTA sum its own bins in
-                                      shared memory and store each of them once. The outputs
-                                      need no zeroing and see no read-modify-write. tile_bins, a
-                                      power of two, sets the bins per range (default 2^19; raised
-                                      until there are at most 256 ranges; at most 2^20).
+    SINET_STRAT_PARTITION = 8      /* hot/cold partition, for unsorted input over histograms too
+                                      large for shared memory (Section 5's map-reduce with the
+                                      reduction kept on chip): a strided sample of about n / 4,096
+                                      records ranks the bins; the most sampled ones (up to 16,384
+                                      slots, as shared memory allows) are summed in shared memory
+                                      by every CTA; every other routed update is appended as an
+                                      8-byte (bin, direction, bytes) entry to the CTA's run of its
+                                      bin range, large histograms' runs are split by tile of bins,
+                                      and each tile is summed in shared memory and every bin of it
+                                      stored once. The outputs need no zeroing and see no
+                                      read-modify-write. tile_bins, a power of two of at most 2^20,
+                                      asks for that many bins per range (taken to the nearest size
+                                      the cold pass sums without a split: one to eight tiles of at
+                                      most 2^13 bins; default: as measured best).
                                       sinet_discriminate_histogram only, no watch list; at most
                                       2^32 - 4,096 routed updates and 2^28 bins. Scratch, stream-
-                                      ordered: 16 KB pages of 2,048 entries, namely a region
-                                      per CTA and range (pages for an even share of 30 % of the
-                                      routed updates, plus one, at most 16) and a shared pool for
-                                      every routed update (8 bytes each) plus two pages per CTA
-                                      and range; about 320 bytes of bookkeeping per page, and
-                                      64 MB at most for the sample. The second kernel is a
-                                      cooperative launch (one CTA per SM, all resident). */
+                                      ordered: the runs' room (8 bytes for 1.125 entries per routed
+                                      update, up to 2.125 for small inputs, and 512 bytes per CTA
+                                      and range), as much again for the tiles of a split (a call
+                                      that cannot have it runs without the split), an overflow list
+                                      of a sixteenth, and at most 64 MB for the sample. */
 } sinet_strategy;
 
 /* How membership is looked up. Both are exact. */
@@ -533,7 +532,8 @@ sinet_status sinet_histogram_sparse(const sinet_hist_out *in, uint64_t n_bins, u
  * partition for unsorted input over a histogram of 256 MB or more with at
  * least one record per four bins (the 32-byte cells where the partition's
  * limits are exceeded, or where its scratch does not fit the free device
- * memory at the call), warp combining otherwise). No kernel runs.
+ * memory at the call) or of 64 MB or more with at least 6 M records, warp
+ * combining otherwise). No kernel runs.
  */
 sinet_status sinet_auto_strategy(const sinet_prefix_table *t, uint64_t n, const sinet_hist_params *p,
                                  int32_t *strategy);

@@ -184,6 +184,8 @@ static uint32_t table_smem(const sinet_prefix_table *t, int lk) {
 // scratch when the input is not time-sorted: well beyond L2, unsorted updates
 // miss, and one sector per update instead of two halves the DRAM traffic.
 static const uint64_t kCellMinHistBytes = 256ull << 20;
+// Smaller ones take the partition from these sizes on (see auto_rule).
+static const uint64_t kPartMinHistBytes = 64ull << 20, kPartMinRecords = 6000000;
 
 // Hot-key cache of the warp-aggregated atomic kernel: 2^9 sets x 4 ways
 // (32 KB of shared memory per CTA).
@@ -232,14 +234,19 @@ static int auto_rule(const sinet_hist_params *p, const RecArgs &r, uint32_t cap,
     // the tile strategy: measured faster than OWNER on the paper-shaped day
     // (about 4.6 records per ms bin, +-500 ms disorder)
     if (p->hints & SINET_HINT_TIME_SORTED) return SINET_STRAT_PRIV_TILE;
-    // unsorted input over a histogram far beyond L2: the hot/cold partition
-    // (measured 1.9x faster than the cells on the Zipf-skewed heavy day),
-    // else the cells
-    if (24 * p->n_bins >= kCellMinHistBytes && r.g.n >= p->n_bins / 4) {
+    // unsorted input over a histogram that global reductions do not find in L2:
+    // the hot/cold partition, else (far beyond L2) the cells. Measured, us, the
+    // partition against the faster of combining and plain reductions: 20 M
+    // records over 3.6 M bins 283 / 411, over 21.6 M 455 / 1,074; skewed, over
+    // 8.6 M bins 286 / 352; 100 M over 86.4 M 1,588 / 6,054, skewed 1,044 / 2,163.
+    // Its fixed costs (about 80 us) lose below some 5 M records (3 M over 3.6 M
+    // bins: 127 / 106), and to warp combining where bins outnumber records
+    const bool large = 24 * p->n_bins >= kCellMinHistBytes;
+    if (large ? r.g.n >= p->n_bins / 4 : 24 * p->n_bins >= kPartMinHistBytes && r.g.n >= kPartMinRecords) {
         PartPlan probe{};
-        if (plan_partition(lk, tsm, r, h, 0, ds->sm_count, ds->smem_optin, &probe) == cudaSuccess)
+        if (plan_partition(lk, tsm, r, h, 0, ds->sm_count, ds->smem_optin, false, &probe) == cudaSuccess)
             return SINET_STRAT_PARTITION;
-        return SINET_STRAT_ATOMIC_CELL;
+        if (large) return SINET_STRAT_ATOMIC_CELL;
     }
     return SINET_STRAT_GLOBAL_ATOMIC;
 }
@@ -261,7 +268,7 @@ static int auto_candidates(const sinet_hist_params *p, const RecArgs &r, uint32_
     if (24 * p->n_bins >= kCellMinHistBytes) out[k++] = SINET_STRAT_ATOMIC_CELL;
     PartPlan probe{};
     if (k < 4 && !(p->hints & SINET_HINT_TIME_SORTED) &&
-        plan_partition(lk, tsm, r, h, 0, ds->sm_count, ds->smem_optin, &probe) == cudaSuccess)
+        plan_partition(lk, tsm, r, h, 0, ds->sm_count, ds->smem_optin, false, &probe) == cudaSuccess)
         out[k++] = SINET_STRAT_PARTITION;
     return k;
 }
@@ -418,15 +425,15 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
     if (strat == SINET_STRAT_SORT_REDUCE && r.g.n * (h.two_dir ? 2ull : 1ull) >= 0xFFFFFFF0ull)
         return SINET_ERR_UNSUPPORTED;
     PartPlan pplan{};
+    uint32_t pbits = 0;  // log2 of the caller's bins per range
     if (strat == SINET_STRAT_PARTITION) {
         if (watch) return SINET_ERR_UNSUPPORTED;
-        uint32_t bb = 0;
         if (p->tile_bins) {
             if (p->tile_bins & (p->tile_bins - 1)) return SINET_ERR_INVALID_ARG;
-            while ((1u << bb) < p->tile_bins) ++bb;
-            if (bb > 20) return SINET_ERR_UNSUPPORTED;
+            while ((1u << pbits) < p->tile_bins) ++pbits;
+            if (pbits > 20) return SINET_ERR_UNSUPPORTED;
         }
-        if (plan_partition(lk, tsm, r, h, bb, ds->sm_count, ds->smem_optin, &pplan) != cudaSuccess)
+        if (plan_partition(lk, tsm, r, h, pbits, ds->sm_count, ds->smem_optin, false, &pplan) != cudaSuccess)
             return SINET_ERR_UNSUPPORTED;
     }
     OwnerPlan oplan{};
@@ -487,6 +494,15 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
         case SINET_STRAT_PARTITION: {
             void *scratch = nullptr;
             e = cudaMallocAsync(&scratch, pplan.scratch_bytes, s);
+            if (e != cudaSuccess && pplan.d.split) {
+                // without the split's room: slower, and a little over half the scratch
+                cudaGetLastError();
+                PartPlan lean{};
+                if (plan_partition(lk, tsm, r, h, pbits, ds->sm_count, ds->smem_optin, true, &lean) == cudaSuccess) {
+                    pplan = lean;
+                    e = cudaMallocAsync(&scratch, pplan.scratch_bytes, s);
+                }
+            }
             if (e != cudaSuccess && p->strategy == SINET_STRAT_AUTO) {
                 // AUTO's choice does not fit the free memory: the cells need
                 // far less scratch and zero the same outputs (none)
