@@ -61,7 +61,11 @@ typedef enum {
 /* How the histogram update is carried out. All give identical results. */
 typedef enum {
     SINET_STRAT_AUTO = 0,          /* autotuner / heuristics choose */
-    SINET_STRAT_GLOBAL_ATOMIC = 1, /* warp match + reduce, then global atomics */
+    SINET_STRAT_GLOBAL_ATOMIC = 1, /* warp match + reduce (while that saves updates), then global
+                                      atomics; not accumulating, outside a capture, from 1 M
+                                      records and with up to 3.9 M bins (six a record at most)
+                                      they go to stream-ordered scratch of 16 bytes a bin, then
+                                      expanded (straight to the outputs when it cannot be had) */
     SINET_STRAT_PRIV_TILE = 2,     /* shared-memory bin tile per chunk (time-sorted input) */
     SINET_STRAT_SORT_REDUCE = 3,   /* plain path: discriminate, radix sort, reduce by key */
     SINET_STRAT_SMEM_FULL = 4,     /* whole histogram privatised in shared memory (small n_bins) */
@@ -532,7 +536,7 @@ sinet_status sinet_histogram_sparse(const sinet_hist_out *in, uint64_t n_bins, u
  * partition for unsorted input over a histogram of 256 MB or more with at
  * least one record per four bins (the 32-byte cells where the partition's
  * limits are exceeded, or where its scratch does not fit the free device
- * memory at the call) or of 64 MB or more with at least 6 M records, warp
+ * memory at the call) or of 90 MB or more with at least 6 M records, warp
  * combining otherwise). No kernel runs.
  */
 sinet_status sinet_auto_strategy(const sinet_prefix_table *t, uint64_t n, const sinet_hist_params *p,

@@ -185,7 +185,7 @@ static uint32_t table_smem(const sinet_prefix_table *t, int lk) {
 // miss, and one sector per update instead of two halves the DRAM traffic.
 static const uint64_t kCellMinHistBytes = 256ull << 20;
 // Smaller ones take the partition from these sizes on (see auto_rule).
-static const uint64_t kPartMinHistBytes = 64ull << 20, kPartMinRecords = 6000000;
+static const uint64_t kPartMinHistBytes = 90ull << 20, kPartMinRecords = 6000000;
 
 // Hot-key cache of the warp-aggregated atomic kernel: 2^9 sets x 4 ways
 // (32 KB of shared memory per CTA).
@@ -228,21 +228,64 @@ static cudaError_t run_cells(int lk, const RecArgs &r, const TableArgs &ta_tab, 
     return e == cudaSuccess ? e2 : e;
 }
 
+// Warp combining through packed cells (one reduction an update instead of two,
+// see HistArgs::packed) while the cells stay in L2, which keeps about 60 MB for
+// one set of accesses (3.6 M bins: 58 MB of cells stay, 86 MB of output arrays
+// did not): 16 bytes a bin are zeroed and read besides the outputs' 24 written.
+// 20 M uniform records over 3.6 M bins 411 -> 186 us, 10 M over 100 K 159 -> 98,
+// 1 M over 3.6 M 87 -> 78. Below a record per six bins or 1 M records the
+// expansion costs more than the reductions it saves (100 K over 3.6 M: 59 us,
+// straight into the outputs 42).
+static bool packed_pays(uint64_t n_bins, uint64_t n) {
+    return 16 * n_bins <= (60ull << 20) && n >= 1000000 && n >= n_bins / 6;
+}
+// Not beyond 2^32 records, up to which the totals that check the cells cannot
+// wrap, and not while the stream is captured: a graph with an allocation of its
+// own can be instantiated only once at a time.
+static bool use_packed(const sinet_hist_params *p, uint64_t n, bool capturing) {
+    return !p->accumulate && !capturing && packed_pays(p->n_bins, n) && n < (1ull << 32);
+}
+
+static bool is_capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();  // the legacy stream while another one is captured
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+static cudaError_t run_packed(int lk, const RecArgs &r, const TableArgs &tab, HistArgs h, const LaunchCfg &c,
+                              cudaStream_t s, const TableArgs *watch) {
+    void *scratch = nullptr;
+    const size_t bytes = 64 + 16 * (size_t)h.n_bins;
+    cudaError_t e = cudaMallocAsync(&scratch, bytes, s);
+    if (e != cudaSuccess) return e;
+    h.pack_sums = static_cast<uint64_t *>(scratch);
+    h.packed = h.pack_sums + 8;
+    e = cudaMemsetAsync(scratch, 0, bytes, s);
+    if (e == cudaSuccess) e = run_fused_atomic(lk, true, r, tab, h, kCacheSetBits, c, watch);
+    if (e == cudaSuccess) e = run_pack_finish(lk, r, tab, h, c, watch);
+    const cudaError_t e2 = cudaFreeAsync(scratch, s);
+    return e == cudaSuccess ? e2 : e;
+}
+
 static int auto_rule(const sinet_hist_params *p, const RecArgs &r, uint32_t cap, int lk, uint32_t tsm,
-                     const HistArgs &h, const DeviceState *ds) {
+                     const HistArgs &h, const DeviceState *ds, bool capturing) {
     if (2ull * p->n_bins <= 8192 && p->n_bins <= cap) return SINET_STRAT_SMEM_FULL;
     // the tile strategy: measured faster than OWNER on the paper-shaped day
     // (about 4.6 records per ms bin, +-500 ms disorder)
     if (p->hints & SINET_HINT_TIME_SORTED) return SINET_STRAT_PRIV_TILE;
-    // unsorted input over a histogram that global reductions do not find in L2:
-    // the hot/cold partition, else (far beyond L2) the cells. Measured, us, the
-    // partition against the faster of combining and plain reductions: 20 M
-    // records over 3.6 M bins 283 / 411, over 21.6 M 455 / 1,074; skewed, over
-    // 8.6 M bins 286 / 352; 100 M over 86.4 M 1,588 / 6,054, skewed 1,044 / 2,163.
-    // Its fixed costs (about 80 us) lose below some 5 M records (3 M over 3.6 M
-    // bins: 127 / 106), and to warp combining where bins outnumber records
+    // unsorted input over a histogram whose packed cells do not stay in L2 (see
+    // packed_pays): the hot/cold partition, else (far beyond L2) the cells.
+    // Measured, us, the partition against the faster of combining and plain
+    // reductions: 20 M records over 21.6 M bins 455 / 1,074; skewed, over 8.6 M
+    // bins 286 / 352; 100 M over 86.4 M 1,588 / 6,054, skewed 1,044 / 2,163. Its
+    // fixed costs (about 80 us) lose below some 5 M records, and to warp
+    // combining where bins outnumber records
     const bool large = 24 * p->n_bins >= kCellMinHistBytes;
-    if (large ? r.g.n >= p->n_bins / 4 : 24 * p->n_bins >= kPartMinHistBytes && r.g.n >= kPartMinRecords) {
+    if (large ? r.g.n >= p->n_bins / 4
+              : !capturing && 24 * p->n_bins >= kPartMinHistBytes && r.g.n >= kPartMinRecords) {
         PartPlan probe{};
         if (plan_partition(lk, tsm, r, h, 0, ds->sm_count, ds->smem_optin, false, &probe) == cudaSuccess)
             return SINET_STRAT_PARTITION;
@@ -352,6 +395,7 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
     const uint32_t tsm = table_smem(t, lk);
     uint32_t cap = tile_capacity(ds, tsm);
 
+    const bool capturing = is_capturing(s);
     int strat = p->strategy;
     const TableArgs *watch = p->watch ? &p->watch->args : nullptr;
     if (watch && (lk == LK_PML || lk == LK_CLASS_IN)) return SINET_ERR_UNSUPPORTED;
@@ -361,7 +405,7 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
     // a watch list keeps few records (a blocklist): the plain combining kernel
     if (strat == SINET_STRAT_AUTO && watch) strat = SINET_STRAT_GLOBAL_ATOMIC;
     if (strat == SINET_STRAT_AUTO) {
-        strat = auto_rule(p, r, cap, lk, tsm, h, ds);
+        strat = auto_rule(p, r, cap, lk, tsm, h, ds, capturing);
         int dev = 0;
         cudaGetDevice(&dev);
         const std::string key = auto_key(dev, lk, p, r, h);
@@ -452,7 +496,8 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
         oplan = plan_owner(r.g.n, h.n_bins, S, (uint32_t)g);
     }
 
-    if ((strat == SINET_STRAT_ATOMIC_CELL || strat == SINET_STRAT_OWNER || strat == SINET_STRAT_PARTITION) &&
+    const bool packed = strat == SINET_STRAT_GLOBAL_ATOMIC && use_packed(p, r.g.n, capturing);
+    if ((strat == SINET_STRAT_ATOMIC_CELL || strat == SINET_STRAT_OWNER || strat == SINET_STRAT_PARTITION || packed) &&
         !p->accumulate && r.g.n > 0) {
         // the expansion (cells), the owners or the cold pass write every bin;
         // only the counters start at zero
@@ -467,6 +512,16 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
     cudaError_t e = cudaSuccess;
     switch (strat) {
         case SINET_STRAT_GLOBAL_ATOMIC:
+            if (packed) {
+                e = run_packed(lk, r, ta_tab, h, c, s, watch);
+                if (e == cudaErrorMemoryAllocation) {  // no room for the cells: straight into the outputs
+                    cudaGetLastError();
+                    st = zero_outputs(p, o, s);
+                    if (st != SINET_OK) return st;
+                    e = run_fused_atomic(lk, true, r, ta_tab, h, kCacheSetBits, c, watch);
+                }
+                break;
+            }
             e = run_fused_atomic(lk, true, r, ta_tab, h, kCacheSetBits, c, watch);
             break;
         case SINET_STRAT_ATOMIC_NOAGG:
@@ -786,7 +841,7 @@ sinet_status sinet_auto_strategy(const sinet_prefix_table *t, uint64_t n, const 
     sinet_hist_out o{};
     HistArgs h = make_hist(p, &o);
     const uint32_t tsm = table_smem(t, lk);
-    *strategy = auto_rule(p, r, tile_capacity(ds, tsm), lk, tsm, h, ds);
+    *strategy = auto_rule(p, r, tile_capacity(ds, tsm), lk, tsm, h, ds, false);
     int dev = 0;
     cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lk_(g_auto_mu);

@@ -59,9 +59,12 @@ struct HotCache {
 // leader that adds the group's count (popc of the peer mask) and byte sum.
 // Byte sums are reduced as two 16-bit halves so 32 values of up to 2^32 - 1
 // cannot overflow the 32-bit warp reduction; they are recombined in 64 bits.
-__device__ __forceinline__ void update_agg(const HistArgs &h, HotCache &hc, uint32_t key, uint32_t b) {
+// CACHED: the group's sum goes to the hot-key cache if it takes the key.
+// Returns (in the leader) the global updates this saved against one per lane.
+template <bool CACHED>
+__device__ __forceinline__ uint32_t update_agg(const HistArgs &h, HotCache &hc, uint32_t key, uint32_t b) {
     const uint32_t peers = __match_any_sync(kFull, key);
-    if (key == kNoKey) return;
+    if (key == kNoKey) return 0u;
     const uint32_t c = __popc(peers);
     uint64_t s = b;
     if (c > 1) {
@@ -69,9 +72,10 @@ __device__ __forceinline__ void update_agg(const HistArgs &h, HotCache &hc, uint
         const uint32_t hi = __reduce_add_sync(peers, b >> 16);
         s = (uint64_t)lo + ((uint64_t)hi << 16);
     }
-    if ((threadIdx.x & 31) == (uint32_t)(__ffs(peers) - 1)) {
-        if (!hc.add(key, c, s)) gadd(h, key & 1u, key >> 1, c, s);
-    }
+    if ((threadIdx.x & 31) != (uint32_t)(__ffs(peers) - 1)) return 0u;
+    if (CACHED && hc.add(key, c, s)) return c;
+    gadd(h, key & 1u, key >> 1, c, s);
+    return c - 1;
 }
 
 // Walk a quad's records in order; consecutive records with the same (bin,

@@ -4,6 +4,8 @@
 // thread, Algorithm 1 against the shared-memory-staged table, routing by the
 // class policy, millisecond binning, and the histogram update of Section 5
 // (a merge-scatter with the associative, commutative integer +).
+#include <algorithm>
+
 #include "combine.cuh"
 #include "launch.h"
 
@@ -108,7 +110,35 @@ __device__ __forceinline__ void flush_filtered(uint64_t *stats, uint32_t flt) {
     if ((threadIdx.x & 31) == 0 && v) atomicAdd(reinterpret_cast<unsigned long long *>(stats + 6), (unsigned long long)v);
 }
 
-template <int LK, bool AGG, bool WATCH>
+// The warp's totals of updates and of their bytes added to `to` (lane 0).
+__device__ __forceinline__ void flush_totals(uint64_t *to, uint64_t updates, uint64_t bytes) {
+#pragma unroll
+    for (int d = 16; d; d >>= 1) {
+        updates += __shfl_down_sync(kFull, updates, d);
+        bytes += __shfl_down_sync(kFull, bytes, d);
+    }
+    if ((threadIdx.x & 31) == 0 && updates) {
+        red_add_u64(to, updates);
+        red_add_u64(to + 1, bytes);
+    }
+}
+
+// With AGG a warp combines its lanes' equal keys only while that saves global
+// updates: combining costs about twice the instructions of a plain reduction,
+// which uniform records over many bins would pay for nothing, and without it
+// the hottest bin of skewed records serialises its reductions. Every kRecheck-th
+// quad of a warp that goes without is combined all the same, and decides anew.
+//   AGG 1: hot keys are kept in a shared-memory cache; fewer than a quarter of a
+//          quad's updates saved, and the warp goes without. (10 M records over
+//          100 K bins, packed cells: uniform 97 us, Zipf 157; always combining,
+//          into the output arrays, 159 and 199.)
+//   AGG 2: no cache, for inputs too small to fill one (an hour of 1 M records
+//          over 3.6 M bins: 75 us, with the cache 95); none saved, and it goes
+//          without (a hot bin's warps all save some).
+enum : int { AGG_NONE = 0, AGG_CACHE = 1, AGG_WARP = 2 };
+constexpr uint32_t kRecheck = 16;
+
+template <int LK, int AGG, bool WATCH>
 __global__ void __launch_bounds__(256, 3) k_fused_atomic(RecArgs r, TableArgs t, HistArgs h,
                                                          uint32_t cache_set_bits, TableArgs wt, uint32_t *status) {
     extern __shared__ __align__(16) uint8_t smem[];
@@ -121,7 +151,7 @@ __global__ void __launch_bounds__(256, 3) k_fused_atomic(RecArgs r, TableArgs t,
     uint32_t cc[4] = {0, 0, 0, 0}, oor[2] = {0, 0}, flt = 0;
     const uint32_t lane = threadIdx.x & 31;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    if (!AGG) {
+    if (AGG == AGG_NONE) {
         for (uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; q < r.g.quads; q += stride) {
             Quad Q;
             load_quad<true, LK != LK_CLASS_IN, true, LK == LK_CLASS_IN>(r, q, pol, Q);
@@ -144,20 +174,44 @@ __global__ void __launch_bounds__(256, 3) k_fused_atomic(RecArgs r, TableArgs t,
     hc.lo = hc.cnt + slots;
     hc.hi = hc.lo + slots;
     hc.set_bits = cache_set_bits;
-    for (uint32_t i = threadIdx.x; i < slots; i += blockDim.x) {
-        hc.keys[i] = kNoKey;
-        hc.cnt[i] = 0;
-        hc.lo[i] = 0;
-        hc.hi[i] = 0;
+    if (AGG == AGG_CACHE) {
+        for (uint32_t i = threadIdx.x; i < slots; i += blockDim.x) {
+            hc.keys[i] = kNoKey;
+            hc.cnt[i] = 0;
+            hc.lo[i] = 0;
+            hc.hi[i] = 0;
+        }
+        __syncthreads();
     }
-    __syncthreads();
+    uint64_t sum = 0;  // bytes of the thread's updates, for the check of packed cells
+    uint32_t plain = 0;  // quads the warp takes next without combining
     // warp-uniform trip count: every lane reaches the warp-synchronous updates
     for (uint64_t q0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) - lane; q0 < r.g.quads;
          q0 += stride) {
+        // a loop of its own: with both ways in one body Zipf-skewed records,
+        // which never take this one, took a fifth longer
+        for (; plain && q0 < r.g.quads; --plain, q0 += stride) {
+            Quad Q;
+            load_quad<true, LK != LK_CLASS_IN, true, LK == LK_CLASS_IN>(r, q0 + lane, pol, Q);
+            watch_filter<WATCH>(W, Q, flt);
+            classify_quad<LK>(C, Q);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (!(Q.valid >> j & 1u)) continue;
+                bump_class(cc, Q.cls[j]);
+                uint32_t bin;
+                const uint32_t dirs = route(h, Q.cls[j], Q.ts[j], bin, oor);
+                if (h.packed) sum += (uint64_t)__popc(dirs) * Q.by[j];
+                if (dirs & 1u) gadd(h, 0u, bin, 1u, Q.by[j]);
+                if (dirs & 2u) gadd(h, 1u, bin, 1u, Q.by[j]);
+            }
+        }
+        if (q0 >= r.g.quads) break;
         Quad Q;
         load_quad<true, LK != LK_CLASS_IN, true, LK == LK_CLASS_IN>(r, q0 + lane, pol, Q);
         watch_filter<WATCH>(W, Q, flt);
         classify_quad<LK>(C, Q);
+        uint32_t saved = 0;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const bool v = Q.valid >> j & 1u;
@@ -166,18 +220,29 @@ __global__ void __launch_bounds__(256, 3) k_fused_atomic(RecArgs r, TableArgs t,
                 bump_class(cc, Q.cls[j]);
                 dirs = route(h, Q.cls[j], Q.ts[j], bin, oor);
             }
+            if (h.packed) sum += (uint64_t)__popc(dirs) * Q.by[j];
             const uint32_t key = dirs ? (bin << 1 | (dirs & 1u ? 0u : 1u)) : kNoKey;
-            update_agg(h, hc, key, Q.by[j]);
+            saved += update_agg<AGG == AGG_CACHE>(h, hc, key, Q.by[j]);
             if (h.two_dir) {
                 const bool both = dirs == 3u;
-                if (__any_sync(kFull, both)) update_agg(h, hc, both ? (bin << 1 | 1u) : kNoKey, Q.by[j]);
+                if (__any_sync(kFull, both))
+                    update_agg<AGG == AGG_CACHE>(h, hc, both ? (bin << 1 | 1u) : kNoKey, Q.by[j]);
             }
         }
+        if (__reduce_add_sync(kFull, saved) < (AGG == AGG_CACHE ? 32u : 1u)) plain = kRecheck - 1;
     }
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < slots; i += blockDim.x) {
-        const uint32_t c = hc.cnt[i];
-        if (c) gadd(h, hc.keys[i] & 1u, hc.keys[i] >> 1, c, (uint64_t)hc.hi[i] << 32 | hc.lo[i]);
+    if (h.packed) {
+        uint64_t updates = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) updates += (uint64_t)cc[k] * __popc((h.policy >> (8 * k)) & 3u);
+        flush_totals(h.pack_sums, updates - oor[0] - oor[1], sum);
+    }
+    if (AGG == AGG_CACHE) {
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < slots; i += blockDim.x) {
+            const uint32_t c = hc.cnt[i];
+            if (c) gadd(h, hc.keys[i] & 1u, hc.keys[i] >> 1, c, (uint64_t)hc.hi[i] << 32 | hc.lo[i]);
+        }
     }
     flush_counters(h.stats, cc, oor, true);
     if (WATCH) flush_filtered(h.stats, flt);
@@ -353,6 +418,127 @@ __global__ void __launch_bounds__(256) k_cells_expand(HistArgs h, uint32_t accum
 }
 
 // ---------------------------------------------------------------------------
+// Packed cells (HistArgs::packed): expansion into the output arrays, and the
+// totals of what it wrote.
+// VEC: four bins a thread in 16-byte loads and stores (every array 16-byte
+// aligned and n_bins a multiple of four); else one, four rows in flight.
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_pack_expand(HistArgs h) {
+    uint64_t updates = 0, bytes = 0;
+    constexpr uint64_t kMask = (1ull << kPackBits) - 1;
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, first = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (VEC) {
+        for (uint64_t q = first; q < h.n_bins / 4; q += stride) {
+            ulonglong2 x[2][2];
+#pragma unroll
+            for (int d = 0; d < 2; ++d) {
+                const ulonglong2 *p = reinterpret_cast<const ulonglong2 *>(h.packed + (uint64_t)d * h.n_bins) + 2 * q;
+                x[d][0] = __ldcs(p);
+                x[d][1] = __ldcs(p + 1);
+            }
+#pragma unroll
+            for (int d = 0; d < 2; ++d) {
+                const uint64_t v[4] = {x[d][0].x, x[d][0].y, x[d][1].x, x[d][1].y};
+                uint32_t c[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    c[k] = (uint32_t)(v[k] >> kPackBits);
+                    updates += c[k];
+                    bytes += v[k] & kMask;
+                }
+                reinterpret_cast<uint4 *>(h.cnt[d])[q] = make_uint4(c[0], c[1], c[2], c[3]);
+                ulonglong2 *o = reinterpret_cast<ulonglong2 *>(h.byt[d]) + 2 * q;
+                o[0] = make_ulonglong2(v[0] & kMask, v[1] & kMask);
+                o[1] = make_ulonglong2(v[2] & kMask, v[3] & kMask);
+            }
+        }
+    } else {
+        for (uint64_t b0 = first; b0 < h.n_bins; b0 += 4 * stride) {
+            uint64_t x[4][2];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int d = 0; d < 2; ++d) {
+                    const uint64_t b = b0 + k * stride;
+                    x[k][d] = b < h.n_bins ? h.packed[(uint64_t)d * h.n_bins + b] : 0ull;
+                }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint64_t b = b0 + k * stride;
+                if (b >= h.n_bins) break;
+#pragma unroll
+                for (int d = 0; d < 2; ++d) {
+                    const uint32_t c = (uint32_t)(x[k][d] >> kPackBits);
+                    h.cnt[d][b] = c;
+                    h.byt[d][b] = x[k][d] & kMask;
+                    updates += c;
+                    bytes += x[k][d] & kMask;
+                }
+            }
+        }
+    }
+    flush_totals(h.pack_sums + 2, updates, bytes);
+}
+
+__device__ __forceinline__ bool pack_right(const uint64_t *s) {
+    return s[0] == s[2] && s[1] == s[3];
+}
+
+// What follows when the totals disagree, in a cooperative launch: the outputs
+// are zeroed, and once every CTA has done its share (a bounded wait) every
+// record is added to them with plain reductions (the class and window counters
+// stand). Otherwise it returns at once.
+template <int LK, bool WATCH>
+__global__ void __launch_bounds__(256) k_pack_redo(RecArgs r, TableArgs t, HistArgs h, TableArgs wt, uint32_t *status) {
+    extern __shared__ __align__(16) uint8_t smem[];
+    __shared__ uint64_t bar;
+    if (pack_right(h.pack_sums)) return;
+    for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; b < h.n_bins;
+         b += (uint64_t)gridDim.x * blockDim.x)
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+            h.cnt[d][b] = 0;
+            h.byt[d][b] = 0;
+        }
+    __threadfence();
+    __syncthreads();
+    __shared__ bool s_zeroed;
+    if (threadIdx.x == 0) {
+        uint32_t *arrived = reinterpret_cast<uint32_t *>(h.pack_sums + 4);
+        atomicAdd(arrived, 1u);
+        bool ok = false;
+        for (uint32_t k = 0; k < kSpinLimit && !ok; ++k)
+            ok = *reinterpret_cast<volatile uint32_t *>(arrived) == gridDim.x;
+        if (!ok) latch_status(status, SINET_ERR_TIMEOUT);
+        s_zeroed = ok;
+    }
+    __syncthreads();
+    if (!s_zeroed) return;
+    h.packed = nullptr;
+    Classifier<LK> C;
+    if (!C.init(t, smem, &bar, status)) return;  // table not staged: the status word says so
+    Classifier<LK_INTERVAL_GLOBAL> W;
+    if (WATCH) W.attach(wt, nullptr);
+    const uint64_t pol = policy_evict_first();
+    uint32_t oor[2] = {0, 0}, flt = 0;
+    for (uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; q < r.g.quads;
+         q += (uint64_t)gridDim.x * blockDim.x) {
+        Quad Q;
+        load_quad<true, LK != LK_CLASS_IN, true, LK == LK_CLASS_IN>(r, q, pol, Q);
+        watch_filter<WATCH>(W, Q, flt);
+        classify_quad<LK>(C, Q);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (!(Q.valid >> j & 1u)) continue;
+            uint32_t bin;
+            const uint32_t dirs = route(h, Q.cls[j], Q.ts[j], bin, oor);
+            if (dirs & 1u) gadd(h, 0u, bin, 1u, Q.by[j]);
+            if (dirs & 2u) gadd(h, 1u, bin, 1u, Q.by[j]);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Host launchers.
 
 size_t smem_optin_limit() {
@@ -381,6 +567,45 @@ cudaError_t run_cells_expand(const HistArgs &h, bool accumulate, const LaunchCfg
     const int grid = 8 * c.sm_count;
     k_cells_expand<<<grid, 256, 0, c.stream>>>(h, accumulate ? 1u : 0u);
     return cudaGetLastError();
+}
+
+cudaError_t run_pack_finish(int lk, const RecArgs &r, const TableArgs &t, const HistArgs &h, const LaunchCfg &c,
+                            const TableArgs *watch) {
+    const int grid = (int)std::min<uint64_t>(8ull * c.sm_count, ((uint64_t)h.n_bins + 1023) / 1024);
+    const uintptr_t all = (uintptr_t)h.cnt[0] | (uintptr_t)h.cnt[1] | (uintptr_t)h.byt[0] | (uintptr_t)h.byt[1];
+    if (all % 16 == 0 && h.n_bins % 4 == 0)
+        k_pack_expand<true><<<grid, 256, 0, c.stream>>>(h);
+    else
+        k_pack_expand<false><<<grid, 256, 0, c.stream>>>(h);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    RecArgs ra = r;
+    TableArgs ta = t, wa = watch ? *watch : TableArgs{};
+    HistArgs ha = h;
+    uint32_t *status = c.status;
+    void *args[] = {&ra, &ta, &ha, &wa, &status};
+#define SINET_REDO(L, WA)                                                                                     \
+    if (lk == L && (watch != nullptr) == WA) {                                                                \
+        const size_t smem = Classifier<L>::smem_bytes(t);                                                     \
+        const void *f = (const void *)k_pack_redo<L, WA>;                                                     \
+        e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);                  \
+        if (e != cudaSuccess) return e;                                                                       \
+        return cudaLaunchCooperativeKernel(f, dim3(c.sm_count), dim3(256), args, smem, c.stream);             \
+    }
+    SINET_REDO(LK_INTERVAL, false)
+    SINET_REDO(LK_LEAF2, false)
+    SINET_REDO(LK_LEAF4, false)
+    SINET_REDO(LK_TOGGLE2, false)
+    SINET_REDO(LK_PML, false)
+    SINET_REDO(LK_INTERVAL_GLOBAL, false)
+    SINET_REDO(LK_CLASS_IN, false)
+    SINET_REDO(LK_INTERVAL, true)
+    SINET_REDO(LK_LEAF2, true)
+    SINET_REDO(LK_LEAF4, true)
+    SINET_REDO(LK_TOGGLE2, true)
+    SINET_REDO(LK_INTERVAL_GLOBAL, true)
+#undef SINET_REDO
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t run_discriminate(int lk, const RecArgs &r, const TableArgs &t, uint64_t *counts,
@@ -417,16 +642,19 @@ cudaError_t run_fused_atomic(int lk, bool agg, const RecArgs &r, const TableArgs
     int grid = 0;
     cudaError_t e;
     const TableArgs none{};
+    // below about 17 records a thread (the kernel's grid is three CTAs an SM) a
+    // cache costs more to fill and flush than it saves
+    const int mode = !agg ? AGG_NONE : r.g.n < 13000ull * (uint64_t)c.sm_count ? AGG_WARP : AGG_CACHE;
 #define SINET_ATOM(L, A, WA)                                                                    \
-    if (lk == L && agg == A && (watch != nullptr) == WA) {                                      \
+    if (lk == L && mode == A && (watch != nullptr) == WA) {                                     \
         size_t smem = ((Classifier<L>::smem_bytes(t) + 15u) & ~15u) +                           \
-                      (A ? (size_t)HotCache::kSlotBytes * (HotCache::kWays << cache_set_bits) : 0ull);                 \
+                      (A == AGG_CACHE ? (size_t)HotCache::kSlotBytes * (HotCache::kWays << cache_set_bits) : 0ull); \
         if ((e = launch(k_fused_atomic<L, A, WA>, smem, c, grid)) != cudaSuccess) return e;     \
         k_fused_atomic<L, A, WA><<<grid, c.block, smem, c.stream>>>(r, t, h, cache_set_bits,     \
                                                                    WA ? *watch : none, c.status); \
         return cudaGetLastError();                                                              \
     }
-#define SINET_ATOM2(L, WA) SINET_ATOM(L, true, WA) SINET_ATOM(L, false, WA)
+#define SINET_ATOM2(L, WA) SINET_ATOM(L, AGG_CACHE, WA) SINET_ATOM(L, AGG_WARP, WA) SINET_ATOM(L, AGG_NONE, WA)
     SINET_ATOM2(LK_INTERVAL, false)
     SINET_ATOM2(LK_LEAF2, false)
     SINET_ATOM2(LK_LEAF4, false)

@@ -44,6 +44,12 @@ cudaError_t run_fused_tile(int lk, const RecArgs &r, const TableArgs &t, const H
 // adding to them when accumulate is set.
 cudaError_t run_cells_expand(const HistArgs &h, bool accumulate, const LaunchCfg &c);
 
+// After the atomic kernel into packed cells (see HistArgs::packed): expand them
+// into the output arrays of h, and redo the call without cells if the totals
+// show that one overflowed.
+cudaError_t run_pack_finish(int lk, const RecArgs &r, const TableArgs &t, const HistArgs &h, const LaunchCfg &c,
+                            const TableArgs *watch);
+
 // Largest dynamic shared memory a CTA may use on this device.
 size_t smem_optin_limit();
 

@@ -38,7 +38,19 @@ struct HistArgs {
     // output arrays: u64 byte sums of directions 0 and 1, then their u32
     // counts (one DRAM sector per update where the arrays would touch two).
     uint64_t *cells;
+    // When set, updates go to one 64-bit cell per (direction, bin) instead:
+    // count << kPackBits | byte sum, one reduction where the arrays take two.
+    // The fields can overflow into one another, so the routed totals are kept
+    // beside: pack_sums = {updates, their bytes} as the records give them,
+    // then the same as the expanded cells give them. A
+    // cell whose byte sum reaches 2^kPackBits decodes to less than it holds, and
+    // then one whose count alone overflows does, and nothing ever decodes to
+    // more: the totals agree exactly when every cell is right (and where they
+    // do not, the call is redone without cells).
+    uint64_t *packed;
+    uint64_t *pack_sums;
 };
+constexpr uint32_t kPackBits = 40;
 
 // ---------------------------------------------------------------------------
 // Classifier: stages the table image into shared memory (interval or
@@ -419,6 +431,10 @@ __device__ __forceinline__ void flush_counters(uint64_t *stats, const uint32_t c
 }
 
 __device__ __forceinline__ void gadd(const HistArgs &h, uint32_t d, uint32_t bin, uint32_t c, uint64_t s) {
+    if (h.packed) {
+        red_add_u64(h.packed + (uint64_t)d * h.n_bins + bin, ((uint64_t)c << kPackBits) + s);
+        return;
+    }
     if (h.cells) {
         uint64_t *cell = h.cells + 4 * (uint64_t)bin;
         red_add_u64(cell + d, s);
