@@ -41,11 +41,118 @@ __global__ void __launch_bounds__(256) k_batch_zero(BatchArgs b) {
         const HistArgs &h = b.slices[s].h;
         const uint32_t b0 = (z - b.zero_start[s]) * kZeroBins;
         const uint32_t nb = min(kZeroBins, h.n_bins - b0);
+        if (b0 == 0 && threadIdx.x < 8) h.stats[threadIdx.x] = 0;
+        if (h.packed) {  // the expansion stores every bin of the outputs
+            zero_words(reinterpret_cast<uint32_t *>(h.packed + b0), 2 * nb);
+            zero_words(reinterpret_cast<uint32_t *>(h.packed + h.n_bins + b0), 2 * nb);
+            if (b0 == 0 && threadIdx.x < 8) h.pack_sums[threadIdx.x] = 0;
+            continue;
+        }
         zero_words(h.cnt[0] + b0, nb);
         zero_words(h.cnt[1] + b0, nb);
         zero_words(reinterpret_cast<uint32_t *>(h.byt[0] + b0), 2 * nb);
         zero_words(reinterpret_cast<uint32_t *>(h.byt[1] + b0), 2 * nb);
-        if (b0 == 0 && threadIdx.x < 8) h.stats[threadIdx.x] = 0;
+    }
+}
+
+// Packed cells (HistArgs::packed) of the slices that use them into their
+// outputs, in the zeroing items' shares, with the totals of what was stored.
+__global__ void __launch_bounds__(256) k_batch_expand(BatchArgs b) {
+    const uint32_t total = b.hdr->total_zero, n = b.hdr->n_slices;
+    for (uint32_t z = blockIdx.x; z < total; z += gridDim.x) {
+        const uint32_t s = find_slice(b.zero_start, n, z);
+        const HistArgs &h = b.slices[s].h;
+        if (!h.packed) continue;
+        const uint32_t b0 = (z - b.zero_start[s]) * kZeroBins;
+        const uint32_t b1 = b0 + min(kZeroBins, h.n_bins - b0);
+        uint64_t updates = 0, bytes = 0;
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+            const uint64_t *cells = h.packed + (uint64_t)d * h.n_bins;
+            uint32_t *cnt = h.cnt[d];
+            uint64_t *byt = h.byt[d];
+            for (uint32_t i = b0 + threadIdx.x; i < b1; i += 8 * blockDim.x) {
+                uint64_t x[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const uint32_t at = i + k * blockDim.x;
+                    x[k] = at < b1 ? __ldcs(reinterpret_cast<const unsigned long long *>(cells + at)) : 0ull;
+                }
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const uint32_t at = i + k * blockDim.x;
+                    if (at >= b1) break;
+                    const uint32_t c = (uint32_t)(x[k] >> kPackBits);
+                    const uint64_t sum = x[k] & ((1ull << kPackBits) - 1);
+                    cnt[at] = c;
+                    byt[at] = sum;
+                    updates += c;
+                    bytes += sum;
+                }
+            }
+        }
+        flush_totals(h.pack_sums + 2, updates, bytes);
+    }
+}
+
+// Slices one of whose cells overflowed (the totals disagree): the outputs are
+// zeroed by all CTAs of this cooperative launch, and once every one has done its
+// share (a bounded wait) every record is added to them. Usually none is.
+__global__ void __launch_bounds__(256) k_batch_redo(BatchArgs b, uint32_t *status) {
+    __shared__ bool s_zeroed;
+    const uint32_t n = b.hdr->n_slices;
+    const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x, threads = gridDim.x * blockDim.x;
+    for (uint32_t s0 = 0; s0 < n; s0 += blockDim.x) {
+        // one slice a thread; few are ever left
+        const uint32_t mine = s0 + threadIdx.x;
+        bool wrong = false;
+        if (mine < n && b.slices[mine].h.packed) {
+            const uint64_t *t = b.slices[mine].h.pack_sums;
+            wrong = t[0] != t[2] || t[1] != t[3];
+        }
+        if (!__syncthreads_or(wrong)) continue;
+        for (uint32_t s = s0; s < min(s0 + blockDim.x, n); ++s) {
+            const BatchSlice &S = b.slices[s];
+            HistArgs h = S.h;
+            if (!h.packed || (h.pack_sums[0] == h.pack_sums[2] && h.pack_sums[1] == h.pack_sums[3])) continue;
+            for (uint32_t i = tid; i < h.n_bins; i += threads)
+#pragma unroll
+                for (int d = 0; d < 2; ++d) {
+                    h.cnt[d][i] = 0;
+                    h.byt[d][i] = 0;
+                }
+            __threadfence();
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                uint32_t *arrived = reinterpret_cast<uint32_t *>(h.pack_sums + 4);
+                atomicAdd(arrived, 1u);
+                bool ok = false;
+                for (uint32_t k = 0; k < kSpinLimit && !ok; ++k)
+                    ok = *reinterpret_cast<volatile uint32_t *>(arrived) == gridDim.x;
+                if (!ok) latch_status(status, SINET_ERR_TIMEOUT);
+                s_zeroed = ok;
+            }
+            __syncthreads();
+            if (!s_zeroed) return;
+            h.packed = nullptr;
+            Classifier<LK_INTERVAL_GLOBAL> C;
+            C.attach(S.t, nullptr);
+            const uint64_t pol = policy_evict_first();
+            uint32_t oor[2] = {0, 0};
+            for (uint64_t q = tid; q < S.r.g.quads; q += threads) {
+                Quad Q;
+                load_quad<true, true, true, false>(S.r, q, pol, Q);
+                classify_quad<LK_INTERVAL_GLOBAL>(C, Q);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (!(Q.valid >> j & 1u)) continue;
+                    uint32_t bin;
+                    const uint32_t dirs = route(h, Q.cls[j], Q.ts[j], bin, oor);
+                    if (dirs & 1u) gadd(h, 0u, bin, 1u, Q.by[j]);
+                    if (dirs & 2u) gadd(h, 1u, bin, 1u, Q.by[j]);
+                }
+            }
+        }
     }
 }
 
@@ -169,8 +276,12 @@ __device__ __forceinline__ uint32_t bdirs(uint32_t policy, uint32_t cls, bool in
     return dirs;
 }
 
-// Add (c, s) to bin `bin` of direction d of the current slice's outputs.
+// Add (c, s) to bin `bin` of direction d of the current slice's outputs (or packed cells).
 __device__ __forceinline__ void bgadd(uint32_t d, uint32_t bin, uint32_t c, uint64_t s) {
+    if (uint64_t *cells = vld(g_desc.h.packed)) {
+        red_add_u64(cells + (uint64_t)d * vld(g_desc.h.n_bins) + bin, ((uint64_t)c << kPackBits) + s);
+        return;
+    }
     red_add_u32(vld(g_desc.h.cnt[d]) + bin, c);
     red_add_u64(vld(g_desc.h.byt[d]) + bin, s);
 }
@@ -210,8 +321,8 @@ __device__ __forceinline__ void item_agg(const Classifier<LK> &C, uint64_t q0, u
         hc.hi[i] = 0;
     }
     __syncthreads();
-    uint64_t ccp = 0;
-    uint32_t oorp = 0;
+    uint64_t ccp = 0, sum = 0;
+    uint32_t oorp = 0, updates = 0;
     const uint32_t lane = threadIdx.x & 31;
     // warp-uniform trip count: every lane reaches the warp-synchronous updates
     for (uint64_t qb = q0 + threadIdx.x - lane; qb < q1; qb += blockDim.x) {
@@ -229,6 +340,8 @@ __device__ __forceinline__ void item_agg(const Classifier<LK> &C, uint64_t q0, u
                 bump_class_packed(ccp, Q.cls[j]);
                 dirs = bdirs(policy, Q.cls[j], inr >> j & 1u, oorp);
             }
+            updates += __popc(dirs);
+            sum += (uint64_t)__popc(dirs) * Q.by[j];
             const uint32_t key = dirs ? (bins[j] << 1 | (dirs & 1u ? 0u : 1u)) : kNoKey;
             bupdate_agg(hc, key, Q.by[j]);
             if (two) {
@@ -238,6 +351,7 @@ __device__ __forceinline__ void item_agg(const Classifier<LK> &C, uint64_t q0, u
         }
     }
     drain_packed(ccp, oorp, s_cnt);
+    if (vld(g_desc.h.packed)) flush_totals(vld(g_desc.h.pack_sums), updates, sum);
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < slots; i += blockDim.x) {
         const uint32_t c = hc.cnt[i];
@@ -249,8 +363,8 @@ __device__ __forceinline__ void item_agg(const Classifier<LK> &C, uint64_t q0, u
 template <int LK>
 __device__ __forceinline__ void item_noagg(const Classifier<LK> &C, uint64_t q0, uint64_t q1, uint64_t pol,
                                            unsigned long long *s_cnt) {
-    uint64_t ccp = 0;
-    uint32_t oorp = 0;
+    uint64_t ccp = 0, sum = 0;
+    uint32_t oorp = 0, updates = 0;
     for (uint64_t q = q0 + threadIdx.x; q < q1; q += blockDim.x) {
         Quad Q;
         bload(q, q1, pol, Q);
@@ -266,6 +380,8 @@ __device__ __forceinline__ void item_noagg(const Classifier<LK> &C, uint64_t q0,
             bump_class_packed(ccp, Q.cls[j]);
             const uint32_t dirs = bdirs(policy, Q.cls[j], inr >> j & 1u, oorp);
             if (!dirs) continue;
+            updates += __popc(dirs);
+            sum += (uint64_t)__popc(dirs) * Q.by[j];
             const uint32_t key = bins[j] << 1 | (dirs & 1u ? 0u : 1u);
             if (key == pk) {
                 pc++;
@@ -280,7 +396,9 @@ __device__ __forceinline__ void item_noagg(const Classifier<LK> &C, uint64_t q0,
         }
         if (pk != kNoKey) bgadd(pk & 1u, pk >> 1, pc, ps);
     }
+    __syncwarp();
     drain_packed(ccp, oorp, s_cnt);
+    if (vld(g_desc.h.packed)) flush_totals(vld(g_desc.h.pack_sums), updates, sum);
 }
 
 // Quads [q0, q1) into a shared-memory tile holding the slice's whole
@@ -501,6 +619,15 @@ __global__ void __launch_bounds__(kBatchBlock, 2) k_batch(BatchArgs b, uint32_t 
 cudaError_t run_batch_zero(const BatchArgs &b, int grid, cudaStream_t s) {
     k_batch_zero<<<grid, 256, 0, s>>>(b);
     return cudaGetLastError();
+}
+
+cudaError_t run_batch_expand(const BatchArgs &b, int grid, int sm_count, cudaStream_t s, uint32_t *status) {
+    k_batch_expand<<<grid, 256, 0, s>>>(b);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    BatchArgs ba = b;
+    void *args[] = {&ba, &status};
+    return cudaLaunchCooperativeKernel((const void *)k_batch_redo, dim3(sm_count), dim3(256), args, 0, s);
 }
 
 cudaError_t batch_occupancy(uint32_t smem, int *per_sm) {

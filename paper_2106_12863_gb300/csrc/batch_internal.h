@@ -46,6 +46,10 @@ sinet_status plan_slice(const sinet_batch_slice &u, const DeviceState *ds, uint3
 // candidates (tune), or by the fixed rule.
 sinet_status resolve_strategies(std::vector<PlannedSlice> &v, bool tune, const DeviceState *ds,
                                 uint32_t smem, cudaStream_t s);
+// Whether a slice's reductions go to packed cells (HistArgs::packed), and the
+// bytes of its cells and their totals.
+bool slice_packed(const PlannedSlice &ps);
+size_t packed_bytes(uint32_t n_bins);
 // Map a public strategy to the batch kernel's update scheme.
 uint32_t batch_scheme(int32_t strategy);
 
@@ -78,10 +82,14 @@ struct BatchEngine {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     std::vector<SortJob> sorts;  // slices run by the plain path, after the batch kernel
+    void *cells = nullptr;       // packed cells of the slices that use them
+    bool packed = false;         // the graph expands cells
 
     sinet_status init(uint32_t capacity, const DeviceState *ds, uint32_t smem_bytes);
     // host image (header, starts, descriptors) of `v` in descriptor order
     void image(const std::vector<PlannedSlice> &v, std::vector<uint8_t> &buf) const;
+    // packed cells for the slices of v that gain by them (before image and capture)
+    void plan_packed(std::vector<PlannedSlice> &v);
     // scratch for the slices of v run by the plain path (before capture)
     sinet_status plan_sorts(const std::vector<PlannedSlice> &v, const DeviceState *ds);
     sinet_status capture(uint32_t *status);  // capture zero + batch kernels (+ plain chains) as a graph

@@ -110,19 +110,6 @@ __device__ __forceinline__ void flush_filtered(uint64_t *stats, uint32_t flt) {
     if ((threadIdx.x & 31) == 0 && v) atomicAdd(reinterpret_cast<unsigned long long *>(stats + 6), (unsigned long long)v);
 }
 
-// The warp's totals of updates and of their bytes added to `to` (lane 0).
-__device__ __forceinline__ void flush_totals(uint64_t *to, uint64_t updates, uint64_t bytes) {
-#pragma unroll
-    for (int d = 16; d; d >>= 1) {
-        updates += __shfl_down_sync(kFull, updates, d);
-        bytes += __shfl_down_sync(kFull, bytes, d);
-    }
-    if ((threadIdx.x & 31) == 0 && updates) {
-        red_add_u64(to, updates);
-        red_add_u64(to + 1, bytes);
-    }
-}
-
 // With AGG a warp combines its lanes' equal keys only while that saves global
 // updates: combining costs about twice the instructions of a plain reduction,
 // which uniform records over many bins would pay for nothing, and without it

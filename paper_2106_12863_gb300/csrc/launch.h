@@ -113,6 +113,10 @@ cudaError_t run_batch_zero(const BatchArgs &b, int grid, cudaStream_t s);
 // The persistent batch kernel with `smem` bytes of dynamic shared memory per
 // CTA (table region + work region of any slice must fit).
 cudaError_t run_batch(const BatchArgs &b, uint32_t smem, int grid, cudaStream_t s, uint32_t *status);
+// After it, where slices use packed cells (HistArgs::packed): their expansion
+// into the outputs (with the zeroing kernel's grid), and the slices redone whose
+// totals show that a cell overflowed.
+cudaError_t run_batch_expand(const BatchArgs &b, int grid, int sm_count, cudaStream_t s, uint32_t *status);
 // Set the batch kernel's dynamic shared memory limit; returns CTAs per SM.
 cudaError_t batch_occupancy(uint32_t smem, int *per_sm);
 

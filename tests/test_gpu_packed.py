@@ -73,3 +73,34 @@ def test_warps_change_their_mind(orc, order):
            "alternating": np.arange(n) // 100_000 % 2 == 0}[order]
     ts = np.where(hot, rng.integers(0, 8, n), rng.integers(0, n_bins, n))
     _check(orc, _records(ts, rng.integers(0, 1 << 20, n), 6), n_bins)
+
+
+def test_batch_slices(orc):
+    """Slices with packed cells in one batch, one of which overflows a cell; replayed, since the cells are kept."""
+    import torch
+
+    table = sinet.PrefixTable(*NET)
+    slices, want = [], []
+    for i, (strategy, n_bins, big) in enumerate([("atomic_noagg", 10_001, False), ("atomic_noagg", 10_000, True),
+                                                 ("global_atomic", 70_000, False), ("global_atomic", 20_000, True),
+                                                 ("atomic_noagg", 140_000, False)]):
+        rng = np.random.default_rng(i)
+        rec = _records(rng.integers(0, n_bins + 1, 60_000), rng.integers(0, 1 << 30, 60_000), i)
+        if big:
+            rec["ts"][:600], rec["bytes"][:600] = 77, 0xFFFFFFFF
+        d = to_dev(rec, offsets={k: i for k in ("ts", "src", "dst", "bytes")})
+        out = sinet.Histogram(n_bins)
+        slices.append((table, d["ts"], d["src"], d["dst"], d["bytes"],
+                       sinet.HistParams(0, 1, n_bins, strategy=strategy), out))
+        want.append(orc.discriminate_histogram(*NET, rec, 0, 1, n_bins))
+    batch = sinet.Batch(slices)
+    for _ in range(3):
+        for s in slices:
+            s[-1].count.fill_(-1)
+            s[-1].bytes.fill_(-1)
+        batch.run()
+        torch.cuda.synchronize()
+        for i, (s, ref) in enumerate(zip(slices, want)):
+            assert_hist_equal(s[-1].to_numpy(), ref, f"slice {i}")
+    assert sinet.sinet_device_status() == 0
+    batch.close()
