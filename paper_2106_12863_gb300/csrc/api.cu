@@ -64,6 +64,27 @@ Divider make_divider(uint64_t w) {
     return d;
 }
 
+// The same for 32-bit numerators, 1 <= w < 2^32.
+static Divider32 make_divider32(uint64_t w) {
+    Divider32 d{};
+    uint32_t l = 0;
+    while (l < 32 && (1ull << l) < w) l++;
+    d.m = (uint32_t)((((1ull << l) - w) << 32) / w + 1);
+    d.sh1 = l < 1 ? l : 1;
+    d.sh2 = l >= 1 ? l - 1 : 0;
+    return d;
+}
+
+// The window and bin width of a histogram's arguments.
+static void set_window(HistArgs &h, uint64_t t0, uint64_t w, uint64_t n_bins) {
+    h.t0 = t0;
+    h.span = n_bins * w;
+    h.div = make_divider(w);
+    h.w_is_one = w == 1;
+    h.small = h.span < (1ull << 32);  // and w with it
+    if (h.small) h.div32 = make_divider32(w);
+}
+
 // Quad geometry: pick the first record index (<= 0) at which every stream is
 // 16-byte aligned (4-byte for byte streams), or fall back to scalar loads.
 QuadGeom make_geom(uint64_t n, std::initializer_list<Stream> streams) {
@@ -120,10 +141,7 @@ HistArgs make_hist(const sinet_hist_params *p, const sinet_hist_out *o) {
     h.byt[0] = o->bytes[0];
     h.byt[1] = o->bytes[1];
     h.stats = o->stats;
-    h.t0 = p->t0_ms;
-    h.span = p->n_bins * p->bin_width_ms;
-    h.div = make_divider(p->bin_width_ms);
-    h.w_is_one = p->bin_width_ms == 1;
+    set_window(h, p->t0_ms, p->bin_width_ms, p->n_bins);
     h.policy = 0;
     h.two_dir = 0;
     for (int c = 0; c < 4; ++c) {
@@ -447,7 +465,7 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
             if (ta.tile_bins > cap) return SINET_ERR_UNSUPPORTED;
             ta.full = 1;
             ta.margin = 0;
-            ta.iters = (uint32_t)(2048 / ct.block);
+            ta.iters = (uint32_t)(65535 / (4 * ct.block));  // as few flushes of the whole tile as its counts allow
         } else {
             // default: as many bins as let two CTAs share an SM (at most
             // 4,096), and chunks of about three records per tile bin (fewer,
@@ -465,6 +483,16 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
         // a chunk stays within 65,535 records: a tile entry counts in 16 bits
         while ((uint64_t)ct.block * 4 * ta.iters > 65535 && ta.iters > 1) ta.iters--;
         if (ta.iters == 0) ta.iters = 1;
+        // no chunk longer than lets every CTA (two an SM) have one, and the whole
+        // histogram's chunks of a length that gives every CTA as many
+        const uint64_t round = 2ull * ds->sm_count * ct.block;  // quads that the grid takes at once
+        const uint64_t all = std::max<uint64_t>(1, (r.g.quads + round - 1) / round);
+        if (ta.full) {
+            const uint64_t rounds = (all + ta.iters - 1) / ta.iters;
+            ta.iters = (uint32_t)((all + rounds - 1) / rounds);
+        } else {
+            ta.iters = (uint32_t)std::min<uint64_t>(ta.iters, all);
+        }
     }
     if (strat == SINET_STRAT_SORT_REDUCE && r.g.n * (h.two_dir ? 2ull : 1ull) >= 0xFFFFFFF0ull)
         return SINET_ERR_UNSUPPORTED;
@@ -766,9 +794,7 @@ sinet_status sinet_bin(const uint64_t *d_ts, uint64_t n, uint64_t t0_ms, uint64_
     DeviceState *ds = nullptr;
     if ((st = device_state(&ds)) != SINET_OK) return st;
     HistArgs h{};
-    h.t0 = t0_ms;
-    h.span = n_bins * bin_width_ms;
-    h.div = make_divider(bin_width_ms);
+    set_window(h, t0_ms, bin_width_ms, n_bins);
     LaunchCfg c;
     c.stream = stream;
     c.sm_count = ds->sm_count;

@@ -250,6 +250,18 @@ __device__ __forceinline__ uint32_t bbin(const Quad &Q, uint32_t bins[4]) {
             bins[j] = in ? (uint32_t)rel : 0u;
             inr |= (uint32_t)in << j;
         }
+    } else if (vld(h.small)) {
+        Divider32 dv;
+        dv.m = vld(h.div32.m);
+        dv.sh1 = vld(h.div32.sh1);
+        dv.sh2 = vld(h.div32.sh2);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint64_t rel = Q.ts[j] - t0;
+            const bool in = rel < span;
+            bins[j] = in ? divide((uint32_t)rel, dv) : 0u;
+            inr |= (uint32_t)in << j;
+        }
     } else {
         Divider dv;
         dv.m = vld(h.div.m);

@@ -37,6 +37,17 @@ __device__ __forceinline__ uint64_t divide(uint64_t n, const Divider &d) {
     return (t1 + ((n - t1) >> d.sh1)) >> d.sh2;
 }
 
+// The same for 32-bit numerators (N = 32): one multiply where the 64-bit form
+// takes a 64 x 64-bit product of them, about 20 instructions a record.
+struct Divider32 {
+    uint32_t m, sh1, sh2;
+};
+
+__device__ __forceinline__ uint32_t divide(uint32_t n, const Divider32 &d) {
+    const uint32_t t1 = __umulhi(d.m, n);
+    return (t1 + ((n - t1) >> d.sh1)) >> d.sh2;
+}
+
 // ---------------------------------------------------------------------------
 // Cache-hinted loads: records are streamed once (evict-first in L2 so the
 // histogram lines stay resident; no L1 allocation for the 32-bit streams).

@@ -410,7 +410,7 @@ __device__ __forceinline__ void part_record(const HistArgs &h, const PartDev &p,
     bump_class_packed(ccp, cls);
     const uint64_t rel = ts - h.t0;
     const bool inw = rel < h.span;
-    const uint32_t bin = inw ? (W1 ? (uint32_t)rel : (uint32_t)divide(rel, h.div)) : 0u;
+    const uint32_t bin = inw ? (W1 ? (uint32_t)rel : bin_of(h, rel)) : 0u;
     const uint32_t dirs = dirs_of_packed(h, cls, inw, oorp);
     if (dirs) part_update(p, m, hot, bin, dirs, by);
 }
@@ -582,7 +582,7 @@ __global__ void __launch_bounds__(kPartThreads, 1) k_part_main(RecArgs r, TableA
                 cc8 += 1u << cls8;
                 const uint64_t rel = ts[j] - h.t0;
                 out[j] = rel >= h.span;
-                bin[j] = W1 ? (uint32_t)rel : (uint32_t)divide(rel, h.div);
+                bin[j] = W1 ? (uint32_t)rel : bin_of(h, rel);
                 dirs[j] = (h.policy >> cls8) & 3u;
             }
             if (__any_sync(kFull, out[0] || out[1])) {  // records outside the window are the exception

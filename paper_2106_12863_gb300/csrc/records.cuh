@@ -30,6 +30,8 @@ struct HistArgs {
     uint64_t span;    // n_bins * w
     Divider div;
     uint32_t w_is_one;
+    uint32_t small;     // span and w are below 2^32: an in-window offset divides by div32
+    Divider32 div32;
     uint32_t policy;  // byte c = direction bits of class c
     uint32_t two_dir; // some class routes to both directions
     uint32_t n_bins;
@@ -51,6 +53,11 @@ struct HistArgs {
     uint64_t *pack_sums;
 };
 constexpr uint32_t kPackBits = 40;
+
+// Bin of an offset within the window.
+__device__ __forceinline__ uint32_t bin_of(const HistArgs &h, uint64_t rel) {
+    return h.small ? divide((uint32_t)rel, h.div32) : (uint32_t)divide(rel, h.div);
+}
 
 // ---------------------------------------------------------------------------
 // Classifier: stages the table image into shared memory (interval or
@@ -234,6 +241,11 @@ struct Classifier<LK_INTERVAL_GLOBAL> {
 
 template <>
 struct Classifier<LK_CLASS_IN> {
+    template <int N>
+    __device__ __forceinline__ void sign_n(const uint32_t (&)[N], uint32_t (&r)[N]) const {
+#pragma unroll
+        for (int i = 0; i < N; ++i) r[i] = 0;
+    }
     __device__ __forceinline__ bool init(const TableArgs &, uint8_t *, uint64_t *, uint32_t *) { return true; }
     static __host__ __device__ uint32_t smem_bytes(const TableArgs &) { return 0; }
     template <int N>
@@ -330,7 +342,7 @@ __device__ __forceinline__ uint32_t route_w(const HistArgs &h, uint32_t cls, uin
         bin = 0;
         return 0u;
     }
-    bin = W1 ? (uint32_t)rel : (uint32_t)divide(rel, h.div);
+    bin = W1 ? (uint32_t)rel : bin_of(h, rel);
     return dirs;
 }
 
@@ -349,11 +361,55 @@ __device__ __forceinline__ uint32_t bin_quad(const HistArgs &h, const Quad &Q, u
     for (int j = 0; j < 4; ++j) {
         const uint64_t rel = Q.ts[j] - h.t0;
         const bool in = rel < h.span;
-        bin[j] = in ? (W1 ? (uint32_t)rel : (uint32_t)divide(rel, h.div)) : 0u;
+        bin[j] = in ? (W1 ? (uint32_t)rel : bin_of(h, rel)) : 0u;
         inr |= (uint32_t)in << j;
     }
     return inr;
 }
+
+// 0xFF in byte k for each of four words whose bit 31 is set.
+__device__ __forceinline__ uint32_t signs4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    uint32_t lo, hi, w;  // byte permutes that replicate a byte's sign
+    asm("prmt.b32 %0, %1, %2, 0xFB;" : "=r"(lo) : "r"(a), "r"(b));
+    asm("prmt.b32 %0, %1, %2, 0xFB;" : "=r"(hi) : "r"(c), "r"(d));
+    asm("prmt.b32 %0, %1, %2, 0x5410;" : "=r"(w) : "r"(lo), "r"(hi));
+    return w;
+}
+
+// Bit k of the result: bit 0 of byte k of w.
+__device__ __forceinline__ uint32_t gather4(uint32_t w) { return ((w & 0x01010101u) * 0x01020408u) >> 24; }
+
+// A quad's records as masks (bit j: record j): source inside, destination
+// inside. Everything that follows from the classes is then a few logic
+// operations for four records at a time.
+template <int LK>
+__device__ __forceinline__ void class_masks(const Classifier<LK> &C, const Quad &Q, uint32_t &src, uint32_t &dst) {
+    if (LK == LK_CLASS_IN) {
+        const uint32_t w = Q.cls[0] | Q.cls[1] << 8 | Q.cls[2] << 16 | Q.cls[3] << 24;
+        src = gather4(w);
+        dst = gather4(w >> 1);
+        return;
+    }
+    uint32_t s[4], d[4];
+    C.template sign_n<4>(Q.src, s);
+    C.template sign_n<4>(Q.dst, d);
+    src = gather4(signs4(s[0], s[1], s[2], s[3]));
+    dst = gather4(signs4(d[0], d[1], d[2], d[3]));
+}
+
+// Which records a direction takes: its bit of the policy of every class as a
+// mask of all records or none, selected by the class masks.
+struct DirMasks {
+    uint32_t c[4];
+    __device__ __forceinline__ DirMasks(uint32_t policy, uint32_t d) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) c[k] = 0u - ((policy >> (8 * k + d)) & 1u);
+    }
+    __device__ __forceinline__ uint32_t of(uint32_t src, uint32_t dst) const {
+        const uint32_t no = (src & c[1]) | (~src & c[0]), yes = (src & c[3]) | (~src & c[2]);
+        return (dst & yes) | (~dst & no);
+    }
+};
 
 // Direction bits of a record from its class; a routed record outside the
 // window routes nowhere and is counted per direction in a packed word (16
