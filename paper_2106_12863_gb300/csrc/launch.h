@@ -129,7 +129,8 @@ struct SortPlan {
     uint64_t sort_tiles;   // tiles of a radix pass (upper bound)
     size_t scratch_bytes;  // total scratch needed
     // offsets into scratch
-    size_t off_keys0, off_vals0, off_keys1, off_vals1, off_hist, off_emit_status, off_sort_status,
+    size_t zero_bytes;     // of the scratch's start, zeroed by every run
+    size_t off_keys0, off_vals0, off_keys1, off_vals1, off_hist, off_emit_status, off_tile_digits,
         off_counters;
 };
 SortPlan plan_sort_reduce(uint64_t n, uint32_t n_bins, bool two_dir);

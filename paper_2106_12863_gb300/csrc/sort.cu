@@ -4,8 +4,8 @@
 //   1. emit:   Algorithm 1 + routing + binning; every routed in-window record
 //              becomes a (key = d * n_bins + bin, bytes) pair, compacted with a
 //              decoupled look-back scan; per-pass digit counts are taken here.
-//   2. sort:   LSD radix sort of the pairs, 8-bit digits, one kernel per pass
-//              (tile ranking with warp match, per-digit decoupled look-back).
+//   2. sort:   LSD radix sort of the pairs, 8-bit digits: per pass the tiles'
+//              digit counts, their scan, and the move (ranking by warp ballots).
 //   3. reduce: reduce-by-key over the sorted pairs (segmented scan per tile);
 //              each run's count and byte sum is scattered into the dense
 //              histogram (runs that cross a tile edge are added atomically).
@@ -27,14 +27,9 @@ constexpr uint64_t kFlagAgg = 1ull << 54;
 constexpr uint64_t kFlagIncl = 2ull << 54;
 constexpr uint64_t kValMask = (1ull << 54) - 1;
 
-__device__ __forceinline__ uint64_t ld_acquire(const uint64_t *p) {
-    uint64_t v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_release(uint64_t *p, uint64_t v) {
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
+// Status words carry all that their readers need, so relaxed accesses do.
+__device__ __forceinline__ uint64_t ld_word(const uint64_t *p) { return *reinterpret_cast<const volatile uint64_t *>(p); }
+__device__ __forceinline__ void st_word(uint64_t *p, uint64_t v) { *reinterpret_cast<volatile uint64_t *>(p) = v; }
 
 // Status word: epoch (8 bits) | flags (2 bits) | value (54 bits). A word whose
 // epoch differs from the reader's is "not ready yet".
@@ -42,32 +37,41 @@ __device__ __forceinline__ uint64_t status_word(uint32_t epoch, uint64_t flag, u
     return (uint64_t)epoch << 56 | flag | (v & kValMask);
 }
 
-// Exclusive prefix of `own` over all predecessor tiles (decoupled look-back).
-// Publishes the aggregate, walks back until an inclusive prefix, publishes the
-// inclusive value. Bounded: a wait that runs out latches SINET_ERR_TIMEOUT.
-__device__ uint64_t look_back(uint64_t *st, uint64_t stride, uint64_t tile, uint64_t own,
-                              uint32_t epoch, uint32_t *status) {
-    if (tile == 0) {
-        st_release(st, status_word(epoch, kFlagIncl, own));
-        return 0;
-    }
-    st_release(st + tile * stride, status_word(epoch, kFlagAgg, own));
-    uint64_t excl = 0;
-    for (int64_t p = (int64_t)tile - 1; p >= 0; --p) {
-        uint64_t w = 0;
-        uint32_t it = 0;
-        for (; it < kSpinLimit; ++it) {
-            w = ld_acquire(st + (uint64_t)p * stride);
-            if ((uint32_t)(w >> 56) == epoch && (w & (kFlagAgg | kFlagIncl))) break;
-        }
+// Waits, bounded, for a predecessor's word (one that ran out latches
+// SINET_ERR_TIMEOUT and reads as an inclusive zero).
+__device__ __forceinline__ uint64_t ready_word(const uint64_t *p, uint64_t w, uint32_t epoch, uint32_t *status) {
+    for (uint32_t it = 0; (uint32_t)(w >> 56) != epoch || !(w & (kFlagAgg | kFlagIncl)); ++it) {
         if (it == kSpinLimit) {
             latch_status(status, SINET_ERR_TIMEOUT);
-            break;
+            return status_word(epoch, kFlagIncl, 0);
         }
-        excl += w & kValMask;
-        if (w & kFlagIncl) break;
+        w = ld_word(p);
     }
-    st_release(st + tile * stride, status_word(epoch, kFlagIncl, excl + own));
+    return w;
+}
+
+// Exclusive prefix of `own` over all predecessor tiles (decoupled look-back) by a
+// whole warp, 32 predecessors a step: publishes the aggregate, walks back to the
+// nearest inclusive prefix, publishes its own. A few hundred tiles are in flight
+// and each step is an L2 round trip (one predecessor a step: emitting 16 M
+// records took 200 us, now 155). Every lane gets the prefix.
+__device__ uint64_t look_back_warp(uint64_t *st, uint64_t tile, uint64_t own, uint32_t epoch, uint32_t *status) {
+    const uint32_t lane = threadIdx.x & 31;
+    if (lane == 0) st_word(st + tile, status_word(epoch, tile ? kFlagAgg : kFlagIncl, own));
+    uint64_t excl = 0;
+    for (int64_t hi = (int64_t)tile; hi > 0; hi -= 32) {
+        const int64_t p = hi - 1 - (int64_t)lane;  // lane 0 is the nearest
+        uint64_t w = status_word(epoch, kFlagIncl, 0);
+        if (p >= 0) w = ready_word(st + p, ld_word(st + p), epoch, status);
+        const uint32_t known = __ballot_sync(kFull, (w & kFlagIncl) != 0);
+        const uint32_t upto = known ? (uint32_t)__ffs(known) - 1 : 31u;
+        uint64_t v = lane <= upto ? w & kValMask : 0;
+#pragma unroll
+        for (int d = 16; d; d >>= 1) v += __shfl_down_sync(kFull, v, d);
+        excl += __shfl_sync(kFull, v, 0);
+        if (known) break;
+    }
+    if (lane == 0 && tile) st_word(st + tile, status_word(epoch, kFlagIncl, excl + own));
     return excl;
 }
 
@@ -75,8 +79,9 @@ struct SortArgs {
     uint32_t *keys0, *vals0, *keys1, *vals1;
     uint32_t *digit_hist;    // [passes][256]
     uint64_t *emit_status;   // [emit tiles]
-    uint64_t *sort_status;   // [sort tiles][256]
-    uint64_t *counters;      // [0] n_emit, [1] emit ticket, [2 + p] pass tickets, [8] reduce ticket
+    uint32_t *tile_digits;   // [256][sort tiles] keys per digit and tile of a pass, then their first places
+    uint64_t sort_tiles;
+    uint64_t *counters;      // [0] n_emit, [1] emit ticket
     uint32_t n_bins;
     uint32_t passes;
 };
@@ -168,9 +173,12 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit(RecArgs r, TableArgs t, H
         const uint32_t k = skey[i];
         for (uint32_t p = 0; p < sa.passes; ++p) atomicAdd(&s_hist[p][(k >> (8 * p)) & 255u], 1u);
     }
-    if (threadIdx.x == 0) {
-        s_goff = look_back(sa.emit_status, 1, tile, total, 1, status);
-        if (tile == n_tiles - 1) sa.counters[0] = s_goff + total;
+    if (warp == 0) {
+        const uint64_t before = look_back_warp(sa.emit_status, tile, total, 1, status);
+        if (lane == 0) {
+            s_goff = before;
+            if (tile == n_tiles - 1) sa.counters[0] = before + total;
+        }
     }
     __syncthreads();
     const uint64_t goff = s_goff;
@@ -207,26 +215,103 @@ __device__ __forceinline__ uint32_t block_excl_scan_256(uint32_t v, uint32_t *s_
     return woff + incl - v;
 }
 
+// Lanes with this lane's digit (0..256; 256 past the end, where the lanes' ranks
+// are not used but their mask must not hold others): a ballot a bit, which costs
+// less than a match instruction's pass over up to 32 different values.
+__device__ __forceinline__ uint32_t same_digit(uint32_t dg) {
+    uint32_t m = kFull;
+#pragma unroll
+    for (int b = 0; b < 9; ++b) {
+        const uint32_t ones = __ballot_sync(kFull, dg >> b & 1u);
+        m &= (dg >> b & 1u) ? ones : ~ones;
+    }
+    return m;
+}
+
 // ---------------------------------------------------------------------------
-// 2. one LSD radix pass on bits [8p, 8p + 8)
-__global__ void __launch_bounds__(kSortThreads) k_radix_pass(SortArgs sa, uint32_t p,
-                                                             const uint32_t *kin, const uint32_t *vin,
-                                                             uint32_t *kout, uint32_t *vout,
-                                                             uint32_t *status) {
+// 2. one LSD radix pass on bits [8p, 8p + 8): count, place, move. The counts
+// of every tile and their scan come first (reading the keys once more, an
+// eighth of a pass's traffic) instead of a look-back per digit inside the pass:
+// with hundreds of tiles in flight its 256 walks of L2 round trips were two
+// thirds of the pass (12.8 M pairs: 199 us walking one tile at a time, 138
+// sixteen at a time; 109 for the three kernels).
+__global__ void __launch_bounds__(kSortThreads) k_radix_count(SortArgs sa, uint32_t p, const uint32_t *kin) {
+    __shared__ uint32_t s_hist[kWarps][256];
+    const uint64_t n = sa.counters[0], tile = blockIdx.x, tbase = tile * kSortTile;
+    if (tbase >= n) return;  // block-uniform
+    for (uint32_t i = threadIdx.x; i < kWarps * 256; i += blockDim.x) (&s_hist[0][0])[i] = 0;
+    __syncthreads();
+    uint32_t k[kSortItems];
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+        const uint64_t i = tbase + (uint64_t)j * kSortThreads + threadIdx.x;
+        k[j] = i < n ? __ldg(kin + i) : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j)
+        if (tbase + (uint64_t)j * kSortThreads + threadIdx.x < n)
+            atomicAdd(&s_hist[threadIdx.x >> 5][(k[j] >> (8 * p)) & 255u], 1u);
+    __syncthreads();
+    uint32_t c = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) c += s_hist[w][threadIdx.x];
+    sa.tile_digits[(uint64_t)threadIdx.x * sa.sort_tiles + tile] = c;
+}
+
+// One CTA per digit: the first place of every tile's keys of that digit.
+__global__ void __launch_bounds__(1024) k_radix_place(SortArgs sa, uint32_t p) {
+    __shared__ uint32_t s_warp[32];
+    __shared__ uint32_t s_at;
+    const uint64_t n = sa.counters[0], tiles = (n + kSortTile - 1) / kSortTile;
+    const uint32_t d = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp == 0) {  // keys of smaller digits
+        uint32_t v = 0;
+        for (uint32_t k = lane; k < d; k += 32) v += sa.digit_hist[p * 256 + k];
+        v = __reduce_add_sync(kFull, v);
+        if (lane == 0) s_at = v;
+    }
+    __syncthreads();
+    uint32_t at = s_at;
+    uint32_t *row = sa.tile_digits + (uint64_t)d * sa.sort_tiles;
+    for (uint64_t t0 = 0; t0 < tiles; t0 += blockDim.x) {
+        const uint64_t t = t0 + threadIdx.x;
+        const uint32_t v = t < tiles ? row[t] : 0u;
+        uint32_t incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(kFull, incl, o);
+            if (lane >= (uint32_t)o) incl += y;
+        }
+        if (lane == 31) s_warp[warp] = incl;
+        __syncthreads();
+        uint32_t before = 0, all = 0;
+#pragma unroll
+        for (uint32_t w = 0; w < 32; ++w) {
+            const uint32_t x = s_warp[w];
+            if (w < warp) before += x;
+            all += x;
+        }
+        if (t < tiles) row[t] = at + before + incl - v;
+        at += all;
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(kSortThreads, 3) k_radix_pass(SortArgs sa, uint32_t p, const uint32_t *kin,
+                                                                const uint32_t *vin, uint32_t *kout,
+                                                                uint32_t *vout) {
     __shared__ uint32_t s_key[kSortTile];
     __shared__ uint32_t s_val[kSortTile];
     __shared__ uint32_t s_whist[kWarps][257];
     __shared__ uint32_t s_lstart[256];
-    __shared__ uint64_t s_gpos[256];
+    __shared__ uint32_t s_gpos[256];
     __shared__ uint32_t s_warp[kWarps];
-    __shared__ uint64_t s_tile;
     const uint64_t n = sa.counters[0];
-    if (threadIdx.x == 0) s_tile = atomicAdd(reinterpret_cast<unsigned long long *>(sa.counters + 2 + p), 1ull);
     for (uint32_t i = threadIdx.x; i < kWarps * 257; i += blockDim.x) (&s_whist[0][0])[i] = 0;
-    __syncthreads();
-    const uint64_t tile = s_tile;
-    const uint64_t tbase = tile * kSortTile;
+    const uint64_t tile = blockIdx.x, tbase = tile * kSortTile;
     if (tbase >= n) return;  // block-uniform
+    __syncthreads();
+    s_gpos[threadIdx.x] = sa.tile_digits[(uint64_t)threadIdx.x * sa.sort_tiles + tile];
     const uint32_t shift = 8 * p;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t lt_mask = (1u << lane) - 1u;
@@ -244,7 +329,7 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_pass(SortArgs sa, uint32
     for (int j = 0; j < kSortItems; ++j) {
         const uint64_t i = tbase + (uint64_t)warp * (32 * kSortItems) + j * 32 + lane;
         const uint32_t dg = i < n ? (key[j] >> shift) & 255u : 256u;
-        const uint32_t peers = __match_any_sync(kFull, dg);
+        const uint32_t peers = same_digit(dg);
         const uint32_t leader = __ffs(peers) - 1;
         uint32_t old = 0;
         if (lane == leader) {
@@ -268,14 +353,6 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_pass(SortArgs sa, uint32
     uint32_t tot;
     const uint32_t lstart = block_excl_scan_256(cnt, s_warp, tot);
     s_lstart[d] = lstart;
-    // global position of this tile's run of digit d
-    {
-        // digit start = exclusive scan of the global digit counts of this pass
-        uint32_t gt;
-        const uint32_t gstart = block_excl_scan_256(sa.digit_hist[p * 256 + d], s_warp, gt);
-        const uint64_t excl = look_back(sa.sort_status + d, 256, tile, cnt, p + 1, status);
-        s_gpos[d] = (uint64_t)gstart + excl;
-    }
     __syncthreads();
     // scatter into the tile in sorted order
 #pragma unroll
@@ -290,7 +367,7 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_pass(SortArgs sa, uint32
     for (uint32_t k = threadIdx.x; k < tot; k += blockDim.x) {
         const uint32_t kk = s_key[k];
         const uint32_t dg = (kk >> shift) & 255u;
-        const uint64_t at = s_gpos[dg] + (k - s_lstart[dg]);
+        const uint32_t at = s_gpos[dg] + (k - s_lstart[dg]);
         kout[at] = kk;
         vout[at] = s_val[k];
     }
@@ -433,9 +510,9 @@ SortPlan plan_sort_reduce(uint64_t n, uint32_t n_bins, bool two_dir) {
     off += al(4 * 256 * 4);
     p.off_emit_status = off;
     off += al(8 * (p.emit_tiles + 1));
-    const size_t small_end = off;
-    p.off_sort_status = off;
-    off += al(8ull * 256 * p.sort_tiles);
+    p.zero_bytes = off;
+    p.off_tile_digits = off;
+    off += al(4ull * 256 * p.sort_tiles);
     p.off_keys0 = off;
     off += al(4 * p.n_emit_max + 4);
     p.off_vals0 = off;
@@ -445,7 +522,6 @@ SortPlan plan_sort_reduce(uint64_t n, uint32_t n_bins, bool two_dir) {
     p.off_vals1 = off;
     off += al(4 * p.n_emit_max + 4);
     p.scratch_bytes = off;
-    (void)small_end;
     return p;
 }
 
@@ -457,15 +533,16 @@ cudaError_t run_sort_reduce(int lk, const RecArgs &r, const TableArgs &t, const 
     sa.counters = reinterpret_cast<uint64_t *>(base + plan.off_counters);
     sa.digit_hist = reinterpret_cast<uint32_t *>(base + plan.off_hist);
     sa.emit_status = reinterpret_cast<uint64_t *>(base + plan.off_emit_status);
-    sa.sort_status = reinterpret_cast<uint64_t *>(base + plan.off_sort_status);
+    sa.tile_digits = reinterpret_cast<uint32_t *>(base + plan.off_tile_digits);
+    sa.sort_tiles = plan.sort_tiles;
     sa.keys0 = reinterpret_cast<uint32_t *>(base + plan.off_keys0);
     sa.vals0 = reinterpret_cast<uint32_t *>(base + plan.off_vals0);
     sa.keys1 = reinterpret_cast<uint32_t *>(base + plan.off_keys1);
     sa.vals1 = reinterpret_cast<uint32_t *>(base + plan.off_vals1);
     sa.n_bins = h.n_bins;
     sa.passes = plan.passes;
-    // counters, digit counts, emit and sort look-back words start at zero
-    cudaError_t e = cudaMemsetAsync(base, 0, plan.off_keys0, c.stream);
+    // counters, digit counts and look-back words start at zero
+    cudaError_t e = cudaMemsetAsync(base, 0, plan.zero_bytes, c.stream);
     if (e != cudaSuccess) return e;
     if (r.g.quads == 0) return cudaSuccess;
 
@@ -496,8 +573,9 @@ cudaError_t run_sort_reduce(int lk, const RecArgs &r, const TableArgs &t, const 
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     uint32_t *kin = sa.keys0, *vin = sa.vals0, *kout = sa.keys1, *vout = sa.vals1;
     for (uint32_t p = 0; p < plan.passes; ++p) {
-        k_radix_pass<<<(unsigned)plan.sort_tiles, kSortThreads, 0, c.stream>>>(sa, p, kin, vin, kout, vout,
-                                                                               c.status);
+        k_radix_count<<<(unsigned)plan.sort_tiles, kSortThreads, 0, c.stream>>>(sa, p, kin);
+        k_radix_place<<<256, 1024, 0, c.stream>>>(sa, p);
+        k_radix_pass<<<(unsigned)plan.sort_tiles, kSortThreads, 0, c.stream>>>(sa, p, kin, vin, kout, vout);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         uint32_t *tk = kin, *tv = vin;
         kin = kout;
