@@ -424,16 +424,19 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
     if (strat == SINET_STRAT_AUTO && watch) strat = SINET_STRAT_GLOBAL_ATOMIC;
     if (strat == SINET_STRAT_AUTO) {
         strat = auto_rule(p, r, cap, lk, tsm, h, ds, capturing);
-        int dev = 0;
-        cudaGetDevice(&dev);
-        const std::string key = auto_key(dev, lk, p, r, h);
         bool cached = false;
+        std::string key;  // needed only once something is or is to be measured
         {
             std::lock_guard<std::mutex> lk_(g_auto_mu);
-            auto it = g_auto.find(key);
-            if (it != g_auto.end()) {
-                strat = it->second;
-                cached = true;
+            if ((p->hints & SINET_HINT_TUNE) || !g_auto.empty()) {
+                int dev = 0;
+                cudaGetDevice(&dev);
+                key = auto_key(dev, lk, p, r, h);
+                auto it = g_auto.find(key);
+                if (it != g_auto.end()) {
+                    strat = it->second;
+                    cached = true;
+                }
             }
         }
         if (!cached && (p->hints & SINET_HINT_TUNE) && !p->accumulate && r.g.n > 0) {

@@ -5,6 +5,9 @@
 // class policy, millisecond binning, and the histogram update of Section 5
 // (a merge-scatter with the associative, commutative integer +).
 #include <algorithm>
+#include <map>
+#include <mutex>
+#include <utility>
 
 #include "combine.cuh"
 #include "launch.h"
@@ -570,18 +573,42 @@ size_t smem_optin_limit() {
     return (size_t)v;
 }
 
+// What the runtime was told and answered about a kernel on a device: the
+// shared-memory limit set so far (only ever raised, so no launch finds it lowered
+// by another thread's) and resident CTAs per SM by block and shared memory. The
+// two calls took a third of a small launch's host time.
+struct KernelFacts {
+    size_t smem_limit = 0;
+    std::map<std::pair<int, size_t>, int> per_sm;
+};
+static std::mutex g_facts_mu;
+static std::map<std::pair<const void *, int>, KernelFacts> g_facts;
+
 template <typename K>
 static cudaError_t launch(K kernel, size_t smem, const LaunchCfg &c, int &grid) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    grid = c.grid;
-    if (grid <= 0) {
-        int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, c.block, smem);
+    std::lock_guard<std::mutex> lk(g_facts_mu);
+    KernelFacts &f = g_facts[{(const void *)kernel, dev}];
+    if (smem > f.smem_limit) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        if (per_sm < 1) return cudaErrorInvalidConfiguration;
-        grid = per_sm * c.sm_count;
+        f.smem_limit = smem;
     }
+    grid = c.grid;
+    if (grid > 0) return cudaSuccess;
+    if (f.per_sm.size() > 256) f.per_sm.clear();  // tables of many sizes
+    int &per_sm = f.per_sm[{c.block, smem}];
+    if (per_sm == 0) {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, c.block, smem);
+        if (e != cudaSuccess) {
+            per_sm = 0;
+            return e;
+        }
+    }
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    grid = per_sm * c.sm_count;
     return cudaSuccess;
 }
 

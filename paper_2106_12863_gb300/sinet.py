@@ -56,6 +56,9 @@ class HistParamsC(ctypes.Structure):
                 ("watch", ctypes.c_void_p)]
 
 
+_Policy = ctypes.c_uint8 * 4
+
+
 class HistOutC(ctypes.Structure):
     _fields_ = [("count", ctypes.c_void_p * 2), ("bytes", ctypes.c_void_p * 2),
                 ("stats", ctypes.c_void_p)]
@@ -67,6 +70,8 @@ class BatchSliceC(ctypes.Structure):
                 ("params", HistParamsC), ("out", HistOutC), ("ready", ctypes.c_void_p),
                 ("ready_value", ctypes.c_uint32)]
 
+
+_Two = ctypes.c_void_p * 2
 
 BATCH_AUTOTUNE = 1
 
@@ -173,8 +178,8 @@ def _dptr(t) -> int | None:
 def _stream(stream) -> int | None:
     import torch
 
-    if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+    if stream is None:  # the current stream, without a Stream object around it
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -377,16 +382,14 @@ class HistParams:
     watch: object = None  # PrefixTable: only records with src or dst in it are binned
 
     def c(self) -> HistParamsC:
-        p = HistParamsC()
-        p.t0_ms, p.bin_width_ms, p.n_bins = self.t0_ms, self.bin_width_ms, self.n_bins
-        for i in range(4):
-            p.policy[i] = self.policy[i]
-        p.accumulate = int(bool(self.accumulate))
-        p.strategy = STRATEGIES[self.strategy] if isinstance(self.strategy, str) else self.strategy
-        p.lookup = LOOKUPS[self.lookup] if isinstance(self.lookup, str) else self.lookup
-        p.hints, p.tile_bins, p.block_threads = self.hints, self.tile_bins, self.block_threads
-        p.watch = self.watch.handle if self.watch is not None else None
-        return p
+        pol = self.policy
+        return HistParamsC(
+            self.t0_ms, self.bin_width_ms, self.n_bins, _Policy(pol[0], pol[1], pol[2], pol[3]),
+            int(bool(self.accumulate)),
+            STRATEGIES[self.strategy] if isinstance(self.strategy, str) else self.strategy,
+            LOOKUPS[self.lookup] if isinstance(self.lookup, str) else self.lookup,
+            self.hints, self.tile_bins, self.block_threads,
+            self.watch.handle if self.watch is not None else None)
 
 
 class Histogram:
@@ -404,13 +407,14 @@ class Histogram:
         self.stats = mk(8, dtype=torch.int64, device=device)
 
     def c(self) -> HistOutC:
-        o = HistOutC()
-        o.count[0] = self.count[0].data_ptr()
-        o.count[1] = self.count[1].data_ptr()
-        o.bytes[0] = self.bytes[0].data_ptr()
-        o.bytes[1] = self.bytes[1].data_ptr()
-        o.stats = self.stats.data_ptr()
-        return o
+        # (the rows' addresses without a tensor view of each: that took longer
+        # than the library's whole call)
+        c, b = self.count, self.bytes
+        if len(c) < 2 or len(b) < 2:
+            raise IndexError("count and bytes hold a row per direction")
+        c0, b0 = c.data_ptr(), b.data_ptr()
+        return HistOutC(_Two(c0, c0 + c.stride(0) * c.element_size()), _Two(b0, b0 + b.stride(0) * b.element_size()),
+                        self.stats.data_ptr())
 
     def to_numpy(self) -> dict:
         return {"count": self.count.cpu().numpy().view(np.uint32),
