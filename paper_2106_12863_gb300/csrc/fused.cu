@@ -110,8 +110,10 @@ __device__ __forceinline__ void flush_filtered(uint64_t *stats, uint32_t flt) {
 // which uniform records over many bins would pay for nothing, and without it
 // the hottest bin of skewed records serialises its reductions. Every kRecheck-th
 // quad of a warp that goes without is combined all the same, and decides anew.
-//   AGG 1: hot keys are kept in a shared-memory cache; fewer than a quarter of a
-//          quad's updates saved, and the warp goes without. (10 M records over
+//   AGG 1: hot keys are kept in a shared-memory cache; fewer than a fifth of a
+//          quad's updates saved, and the warp goes without (a share of what is
+//          routed, since a watch list may leave little: a fixed 32 of the 128
+//          doubled the heavy day's time behind one). (10 M records over
 //          100 K bins, packed cells: uniform 97 us, Zipf 157; always combining,
 //          into the output arrays, 159 and 199.)
 //   AGG 2: no cache, for inputs too small to fill one (an hour of 1 M records
@@ -193,7 +195,7 @@ __global__ void __launch_bounds__(256, 3) k_fused_atomic(RecArgs r, TableArgs t,
         load_quad<true, LK != LK_CLASS_IN, true, LK == LK_CLASS_IN>(r, q0 + lane, pol, Q);
         watch_filter<WATCH>(W, Q, flt);
         classify_quad<LK>(C, Q);
-        uint32_t saved = 0;
+        uint32_t saved = 0;  // and, from bit 16 on, the thread's routed records
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const bool v = Q.valid >> j & 1u;
@@ -204,6 +206,7 @@ __global__ void __launch_bounds__(256, 3) k_fused_atomic(RecArgs r, TableArgs t,
             }
             if (h.packed) sum += (uint64_t)__popc(dirs) * Q.by[j];
             const uint32_t key = dirs ? (bin << 1 | (dirs & 1u ? 0u : 1u)) : kNoKey;
+            if (AGG == AGG_CACHE && dirs) saved += 1u << 16;
             saved += update_agg<AGG == AGG_CACHE>(h, hc, key, Q.by[j]);
             if (h.two_dir) {
                 const bool both = dirs == 3u;
@@ -211,7 +214,9 @@ __global__ void __launch_bounds__(256, 3) k_fused_atomic(RecArgs r, TableArgs t,
                     update_agg<AGG == AGG_CACHE>(h, hc, both ? (bin << 1 | 1u) : kNoKey, Q.by[j]);
             }
         }
-        if (__reduce_add_sync(kFull, saved) < (AGG == AGG_CACHE ? 32u : 1u)) plain = kRecheck - 1;
+        saved = __reduce_add_sync(kFull, saved);
+        const uint32_t routed = saved >> 16;
+        if (AGG == AGG_CACHE ? routed >= 16 && 5 * (saved & 0xFFFFu) < routed : saved == 0) plain = kRecheck - 1;
     }
     if (h.packed) {
         uint64_t updates = 0;
