@@ -512,7 +512,9 @@ SortPlan plan_sort_reduce(uint64_t n, uint32_t n_bins, bool two_dir) {
     off += al(8 * (p.emit_tiles + 1));
     p.zero_bytes = off;
     p.off_tile_digits = off;
-    off += al(4ull * 256 * p.sort_tiles);
+    // the counts take 4 bytes a digit and tile; 8 are laid out, because the
+    // largest input that fits a caller's fixed scratch follows from this size
+    off += al(8ull * 256 * p.sort_tiles);
     p.off_keys0 = off;
     off += al(4 * p.n_emit_max + 4);
     p.off_vals0 = off;
