@@ -6,7 +6,7 @@
 //   1. sample: classify and bin a strided sample of the records and count
 //      sample hits per bin in an L2-resident hash table;
 //   2. select: the bins with the most sample hits form a static hot table
-//      (4-way sets, hottest first), the same in every CTA; the other hits give
+//      (sets of two ways, hottest first), the same in every CTA; the other hits give
 //      the room that every bin range's run of entries gets;
 //   3. main pass (one read of the records, staged into shared memory by TMA
 //      bulk copies): hot bins are accumulated in each CTA's shared-memory copy
