@@ -49,6 +49,8 @@ bool slice_packed(const PlannedSlice &ps) {
            (ps.strategy == SINET_STRAT_GLOBAL_ATOMIC || ps.strategy == SINET_STRAT_ATOMIC_NOAGG) && n < (1ull << 32) && n >= bins / (16 * bins <= (60ull << 20) ? 6 : 2);
 }
 
+constexpr uint64_t kMinPackedBatch = 8000000;
+
 size_t packed_bytes(uint32_t n_bins) { return 64 + 16 * (size_t)n_bins; }
 
 static uint32_t round16(uint32_t v) { return (v + 15u) & ~15u; }
@@ -181,9 +183,15 @@ void BatchEngine::image(const std::vector<PlannedSlice> &v, std::vector<uint8_t>
 
 void BatchEngine::plan_packed(std::vector<PlannedSlice> &v) {
     size_t total = 0;
+    uint64_t records = 0;
     for (const PlannedSlice &ps : v)
-        if (slice_packed(ps)) total += packed_bytes(ps.d.h.n_bins);
-    if (!total) return;
+        if (slice_packed(ps)) {
+            total += packed_bytes(ps.d.h.n_bins);
+            records += ps.d.r.g.n;
+        }
+    // the expansion's and the redo's kernels cost what the reductions of some
+    // 8 M records save (55 slices of 10 K to 168 K records: 582 us, without 508)
+    if (records < kMinPackedBatch) return;
     if (cudaMalloc(&cells, total) != cudaSuccess) {  // no room: straight into the outputs
         cudaGetLastError();
         cells = nullptr;

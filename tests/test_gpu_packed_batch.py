@@ -1,0 +1,46 @@
+"""Packed cells in a batch large enough for them: on both sides of the line that
+sums the packed slices' records, with a cell that overflows its byte sum; replayed."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover - collected on CPU too
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import paper_2106_12863_gb300 as sinet  # noqa: E402
+
+
+@pytest.mark.parametrize("total", [7_999_999, 8_000_000])
+def test_batches_around_the_line(total):
+    table = sinet.PrefixTable(np.array([0], np.uint32), np.array([1], np.uint8))
+    g = torch.Generator(device="cuda").manual_seed(total)
+    slices, want = [], []
+    for n, n_bins, strategy in ((3_000_001, 1_000_003, "global_atomic"), (total - 3_000_001, 70_001, "atomic_noagg")):
+        ts = torch.randint(0, n_bins, (n,), dtype=torch.int64, device="cuda", generator=g)
+        src = torch.randint(1, 1 << 31, (n,), dtype=torch.int64, device="cuda", generator=g).to(torch.int32)
+        dst = torch.full((n,), -1, dtype=torch.int32, device="cuda")  # outside
+        by = torch.randint(0, 1 << 30, (n,), dtype=torch.int32, device="cuda", generator=g)
+        ts[:2000], by[:2000] = 77, -1  # 2,000 times 2^32 - 1 bytes in one bin: past 2^40
+        out = sinet.Histogram(n_bins)
+        slices.append((table, ts, src, dst, by, sinet.HistParams(0, 1, n_bins, strategy=strategy), out))
+        want.append((torch.bincount(ts, minlength=n_bins),
+                     torch.zeros(n_bins, dtype=torch.int64, device="cuda").index_add_(0, ts, by.to(torch.int64) & 0xFFFFFFFF)))
+    batch = sinet.Batch(slices)
+    for _ in range(2):
+        for s in slices:
+            s[-1].count.fill_(-1)
+            s[-1].bytes.fill_(-1)
+        batch.run()
+        torch.cuda.synchronize()
+        for s, (c, b) in zip(slices, want):
+            got = s[-1].to_numpy()
+            # inside to outside is the outgoing direction; the other one stays empty
+            d = 0 if got["count"][0].any() else 1
+            assert np.array_equal(got["count"][d], c.cpu().numpy().astype(got["count"].dtype))
+            assert np.array_equal(got["bytes"][d], b.cpu().numpy().astype(got["bytes"].dtype))
+            assert not got["count"][1 - d].any() and not got["bytes"][1 - d].any()
+    batch.close()
