@@ -481,7 +481,20 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
             ta.tile_bins = T;
             ta.full = 0;
             ta.margin = T / 6;
-            ta.iters = (uint32_t)std::max<uint64_t>(1, (3ull * T) / (4ull * ct.block));
+            // and, where the records of a bin are many, as many records as an eighth
+            // of the tile's bins hold, while every CTA has eight chunks: the flush
+            // takes longer than such a chunk's own span costs. Inclusive, 180 M
+            // records over 1.55 M bins 896 -> 728 us; classified, 115 M over 2 M
+            // 516 -> 439, over 600 K 539 -> 529. Past 512 records a bin it gives
+            // nothing (96 K bins: 547, and 551-575 with longer chunks), and with
+            // four chunks a CTA 20 M records over 96 K bins took 134, not 130
+            const uint64_t per_bin = r.g.n / p->n_bins;
+            uint64_t records = 3ull * T;
+            if (per_bin < 512) {
+                const uint64_t eighth = r.g.n / (16ull * ds->sm_count);
+                records = std::max(records, std::min<uint64_t>({65535, T / 8 * per_bin, eighth}));
+            }
+            ta.iters = (uint32_t)std::max<uint64_t>(1, records / (4ull * ct.block));
         }
         // a chunk stays within 65,535 records: a tile entry counts in 16 bits
         while ((uint64_t)ct.block * 4 * ta.iters > 65535 && ta.iters > 1) ta.iters--;
