@@ -529,7 +529,7 @@ __global__ void __launch_bounds__(kBatchBlock, 2) k_batch(BatchArgs b, uint32_t 
     // first work item of every slice, when the batch is small enough to keep it here
     __shared__ uint32_t s_starts[kBatchSmemStarts + 1];
     // per-CTA state lives in shared memory so the per-record loops keep the registers
-    __shared__ const uint8_t *s_staged;  // image whose leaf or toggle form sits at smem[0]
+    __shared__ const uint8_t *s_staged;  // the table form at smem[0] (see staged_form)
     __shared__ uint32_t s_phase;
     if (threadIdx.x == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar)) : "memory");
@@ -577,18 +577,16 @@ __global__ void __launch_bounds__(kBatchBlock, 2) k_batch(BatchArgs b, uint32_t 
             }
         }
         const uint32_t lk = S.lk;
-        uint32_t tbytes = 0;
-        if (lk != LK_INTERVAL_GLOBAL) {
-            const bool leaf = lk == LK_LEAF2 || lk == LK_LEAF4;
-            tbytes = leaf ? S.t.leaf_bytes : S.t.iv_bytes;
-            if (S.t.image != s_staged) {
+        const uint32_t tbytes = staged_form_bytes(S.t, lk);
+        if (const uint8_t *form = staged_form(S.t, lk)) {
+            if (form != s_staged) {
                 uint32_t phase = s_phase;
-                const bool ok = restage(smem, S.t.image + (leaf ? S.t.off_leaves : 0u), tbytes, smem_u32(&bar), phase, status);
+                const bool ok = restage(smem, form, tbytes, smem_u32(&bar), phase, status);
                 // everyone has read the old s_staged / s_phase; a copy that did
                 // not land ends the whole CTA (the status word says why)
                 if (!__syncthreads_and(ok)) return;
                 if (threadIdx.x == 0) {
-                    s_staged = S.t.image;
+                    s_staged = form;
                     s_phase = phase;
                 }
             }

@@ -25,6 +25,8 @@ struct PlannedSlice {
     uint32_t items = 0;       // work items (0 for a slice run by the plain path)
     uint32_t zero_items = 0;  // zeroing items (0 when accumulating)
     int32_t strategy = 0;     // sinet_strategy; AUTO until resolved
+    uint32_t lk = 0;          // lookup form off the tile ...
+    uint32_t lk_tile = 0;     // ... and on it: the table's smaller form where the tile fits beside that only
     bool tile_fits = false;   // the whole histogram fits a tile next to the table
     uint32_t user_index = 0;  // position in the caller's slice array
 };
@@ -38,7 +40,7 @@ uint32_t batch_grid(const DeviceState *ds);
 sinet_status check_slice(const sinet_batch_slice &u);
 // Quads per work item of a slice run with scheme `scheme` by `grid` CTAs.
 uint32_t item_quads_for(uint64_t quads, uint32_t scheme, uint32_t grid);
-// Set the strategy of a planned slice (scheme, item size, item count).
+// Set the strategy of a planned slice (scheme, lookup form, item size, item count).
 void set_strategy(PlannedSlice &ps, int32_t strategy, uint32_t grid);
 // Plan a checked slice for a batch kernel with `smem` bytes of shared memory.
 sinet_status plan_slice(const sinet_batch_slice &u, const DeviceState *ds, uint32_t smem, PlannedSlice &ps);

@@ -64,6 +64,7 @@ uint32_t item_quads_for(uint64_t quads, uint32_t scheme, uint32_t grid) {
 void set_strategy(PlannedSlice &ps, int32_t strategy, uint32_t grid) {
     ps.strategy = strategy;
     ps.d.strat = batch_scheme(strategy);
+    ps.d.lk = ps.d.strat == BS_TILE ? ps.lk_tile : ps.lk;
     ps.d.item_quads = item_quads_for(ps.d.r.g.quads, ps.d.strat, grid);
     ps.items = strategy == SINET_STRAT_SORT_REDUCE
                    ? 0u
@@ -99,25 +100,26 @@ sinet_status plan_slice(const sinet_batch_slice &u, const DeviceState *ds, uint3
     d.t = t->args;
     d.h = make_hist(&u.params, &u.out);
     d.h.status = ds->status;
-    // the toggle form is staged when it leaves room for the hot-key cache
+    // a form is staged when it leaves room for the hot-key cache
     uint32_t staged = 0;
     const uint32_t form_bytes = t->host.leaf_words ? t->img.leaf_bytes : t->img.iv_bytes;
     if (t->img.iv_fits_smem && round16(form_bytes) + kBatchCacheBytes <= smem) {
         staged = round16(form_bytes);
-        d.lk = (uint32_t)staged_lookup(t);
+        ps.lk = (uint32_t)staged_lookup(t);
     } else if (t->img.iv_fits_smem && toggle_is_smaller(t, staged_lookup(t)) &&
                round16(t->img.iv_bytes) + kBatchCacheBytes <= smem) {
         staged = round16(t->img.iv_bytes);
-        d.lk = (uint32_t)toggle_lookup(t);
+        ps.lk = (uint32_t)toggle_lookup(t);
     } else {
-        d.lk = LK_INTERVAL_GLOBAL;
+        ps.lk = LK_INTERVAL_GLOBAL;
     }
+    ps.lk_tile = ps.lk;
     const uint64_t T = (u.params.n_bins + 3) & ~3ull;
-    if (staged && staged + 16 * T > smem && toggle_is_smaller(t, (int)d.lk) &&
+    if (staged && staged + 16 * T > smem && toggle_is_smaller(t, (int)ps.lk) &&
         round16(t->img.iv_bytes) + 16 * T <= smem) {
         // the whole-histogram tile fits beside the table's smaller form only
         staged = round16(t->img.iv_bytes);
-        d.lk = (uint32_t)toggle_lookup(t);
+        ps.lk_tile = (uint32_t)toggle_lookup(t);
     }
     d.tile_bins = (uint32_t)std::min<uint64_t>(T, 0xFFFFFFFFull);
     ps.tile_fits = staged + 16 * T <= smem;
@@ -435,6 +437,7 @@ sinet_status tune_one(const PlannedSlice &rep, const DeviceState *ds, uint32_t s
     // records into scratch outputs, timed the same way (best of three after a
     // warm-up run)
     if (st == SINET_OK && sort_feasible(ps)) {
+        set_strategy(ps, SINET_STRAT_SORT_REDUCE, (uint32_t)eng.grid);
         const SortPlan plan = plan_sort_reduce(n, nb, ps.d.h.two_dir != 0);
         void *scratch = nullptr, *outs = nullptr;
         cudaError_t e = cudaMalloc(&scratch, std::max<size_t>(plan.scratch_bytes, 256));

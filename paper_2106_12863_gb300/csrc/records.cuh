@@ -176,6 +176,18 @@ struct Classifier<LK_LEAF2> : LeafClassifier<2> {};
 template <>
 struct Classifier<LK_LEAF4> : LeafClassifier<4> {};
 
+// Where the form of a table that lookup `lk` stages as one bulk copy starts, and
+// its size (nullptr and 0: none). One image holds both forms of its table, so
+// what a CTA has staged is named by this address, not by the image.
+__host__ __device__ inline const uint8_t *staged_form(const TableArgs &t, uint32_t lk) {
+    if (lk == LK_LEAF2 || lk == LK_LEAF4) return t.image + t.off_leaves;
+    return lk == LK_TOGGLE2 || lk == LK_INTERVAL ? t.image : nullptr;
+}
+__host__ __device__ inline uint32_t staged_form_bytes(const TableArgs &t, uint32_t lk) {
+    if (lk == LK_LEAF2 || lk == LK_LEAF4) return t.leaf_bytes;
+    return lk == LK_TOGGLE2 || lk == LK_INTERVAL ? t.iv_bytes : 0u;
+}
+
 template <>
 struct Classifier<LK_PML> {
     PmlView v;

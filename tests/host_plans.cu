@@ -1,0 +1,68 @@
+// Host-side planning of the CUDA library, callable without a GPU: compiled by
+// test_host_plans.py and linked against the library's own planning functions.
+#include <cstdint>
+#include <vector>
+
+#include "batch_internal.h"
+#include "partition.h"
+
+using namespace sinet;
+
+namespace {
+
+// A GB300's facts, as device_state() reads them there.
+DeviceState gb300() {
+    DeviceState ds;
+    ds.sm_count = 152;
+    ds.smem_optin = 232448;
+    ds.smem_per_sm = 233472;
+    return ds;
+}
+
+bool host_table(const uint32_t *net, const uint8_t *len, uint32_t n, sinet_prefix_table &t) {
+    if (compile_table(net, len, n, 0, t.host) != SINET_OK) return false;
+    serialise(t.host, t.img);
+    t.args = TableArgs{};
+    t.args.image = reinterpret_cast<const uint8_t *>(uintptr_t(1) << 20);  // not read
+    t.args.iv_bytes = t.img.iv_bytes;
+    t.args.leaf_bytes = t.img.leaf_bytes;
+    t.args.off_leaves = t.img.off_leaves;
+    return true;
+}
+
+}  // namespace
+
+extern "C" {
+
+// One batch slice of n records and n_bins bins: {planned, lookup form, start of
+// the staged form in the image (-1: none), its bytes, dynamic shared memory, tile bins}.
+int plan_batch_slice(const uint32_t *net, const uint8_t *len, uint32_t n_net, uint64_t n, uint64_t n_bins,
+                     int32_t strategy, int64_t *out) {
+    sinet_prefix_table t{};
+    if (!host_table(net, len, n_net, t)) return -1;
+    const DeviceState ds = gb300();
+    sinet_batch_slice u{};
+    u.ts = reinterpret_cast<const uint64_t *>(uintptr_t(1) << 30);
+    u.src = u.dst = u.bytes = reinterpret_cast<const uint32_t *>(uintptr_t(1) << 30);
+    u.n = n;
+    u.table = &t;
+    u.params.bin_width_ms = 1;
+    u.params.n_bins = n_bins;
+    u.params.policy[1] = 1;
+    u.params.policy[2] = 2;
+    u.params.strategy = strategy;
+    PlannedSlice ps;
+    const uint32_t smem = batch_smem(&ds);
+    const sinet_status st = plan_slice(u, &ds, smem, ps);
+    if (st != SINET_OK) return (int)st;
+    const uint8_t *form = staged_form(ps.d.t, ps.d.lk);
+    out[0] = ps.tile_fits;
+    out[1] = ps.d.lk;
+    out[2] = form ? (int64_t)(form - t.args.image) : -1;
+    out[3] = staged_form_bytes(ps.d.t, ps.d.lk);
+    out[4] = smem;
+    out[5] = ps.d.tile_bins;
+    return 0;
+}
+
+}  // extern "C"

@@ -1,0 +1,55 @@
+"""What the library plans on the host before a launch, from its own planning
+functions with a GB300's facts; no GPU is used."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2106_12863_gb300 import _build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+GLOBAL_ATOMIC, SMEM_FULL = 1, 4
+
+
+@pytest.fixture(scope="module")
+def plans(tmp_path_factory):
+    lib = _build.build()
+    out = str(tmp_path_factory.mktemp("plans") / "host_plans.so")
+    subprocess.run([_build._nvcc(), *_build.ARCH, "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
+                    "-I", os.path.join(_build.ROOT, "include"), "-I", _build.CSRC, "-shared", "-o", out,
+                    os.path.join(HERE, "host_plans.cu"), lib, "-Xlinker", "-rpath=" + os.path.dirname(lib)],
+                   check=True)
+    return ctypes.CDLL(out)
+
+
+def prefixes(n, lo, hi, seed):
+    rng = np.random.default_rng(seed)
+    ln = rng.integers(lo, hi + 1, n)
+    net = rng.integers(0, 1 << 31, n) & (0xFFFFFFFF << (32 - ln))
+    return net.astype(np.uint32), ln.astype(np.uint8)
+
+
+def _slice(plans, table, n, n_bins, strategy):
+    out = np.zeros(6, np.int64)
+    rc = plans.plan_batch_slice(*(ctypes.c_void_p(a.ctypes.data) for a in table), ctypes.c_uint32(len(table[0])),
+                                ctypes.c_uint64(n), ctypes.c_uint64(n_bins), ctypes.c_int32(strategy),
+                                ctypes.c_void_p(out.ctypes.data))
+    assert rc == 0
+    return dict(zip(("tile_fits", "lookup", "start", "bytes", "smem", "tile_bins"), out.tolist()))
+
+
+def test_slices_of_one_list_in_both_forms(plans):
+    """A list with a large leaf form: slices whose tile fits beside its smaller form only
+    take that form on the tile alone, and what names a staged form tells the two apart."""
+    table = prefixes(2500, 16, 24, 1)
+    hour = _slice(plans, table, 100_000, 3600, SMEM_FULL)
+    longer = _slice(plans, table, 100_000, 5400, SMEM_FULL)
+    reduced = _slice(plans, table, 100_000, 5400, GLOBAL_ATOMIC)
+    assert hour["tile_fits"] and longer["tile_fits"] and reduced["tile_fits"]
+    assert longer["lookup"] != hour["lookup"] and longer["bytes"] < hour["bytes"]
+    assert longer["start"] != hour["start"]
+    assert (reduced["lookup"], reduced["start"]) == (hour["lookup"], hour["start"])
+    for s in (hour, longer):
+        assert s["bytes"] + 16 * s["tile_bins"] <= s["smem"]
