@@ -301,24 +301,23 @@ __global__ void __launch_bounds__(1024) k_fused_tile(RecArgs r, TableArgs t, His
     __syncthreads();
 
     for (uint64_t ch = blockIdx.x; ch < n_chunks; ch += gridDim.x) {
-        uint32_t base = 0;
-        if (!ta.full) {
-            if (threadIdx.x == 0) {
-                uint32_t b = 0;
-                const uint64_t rel = ts_first - h.t0;
-                if (rel < h.span) {
-                    b = h.w_is_one ? (uint32_t)rel : bin_of(h, rel);
-                    b = b > ta.margin ? b - ta.margin : 0u;
-                }
-                s_base = b;
-                if (ch + gridDim.x < n_chunks) {
-                    const int64_t i1 = quad_base(r.g, (ch + gridDim.x) * qpc);
-                    ts_first = r.ts[i1 < 0 ? 0 : i1];
-                }
+        if (!ta.full && threadIdx.x == 0) {
+            uint32_t b = 0;
+            const uint64_t rel = ts_first - h.t0;
+            if (rel < h.span) {
+                b = h.w_is_one ? (uint32_t)rel : bin_of(h, rel);
+                b = b > ta.margin ? b - ta.margin : 0u;
             }
-            __syncthreads();
-            base = s_base;
+            s_base = b;
+            if (ch + gridDim.x < n_chunks) {
+                const int64_t i1 = quad_base(r.g, (ch + gridDim.x) * qpc);
+                ts_first = r.ts[i1 < 0 ? 0 : i1];
+            }
         }
+        // the tile is placed; and with `full` too, thread 0 has reset s_lo and
+        // s_hi before any warp adds this chunk's range to them
+        __syncthreads();
+        const uint32_t base = ta.full ? 0u : s_base;
         uint32_t omin = 0xFFFFFFFFu, omax = 0;
         for (uint32_t it = 0; it < ta.iters; ++it) {
             uint32_t off[4], by[4], src, dst;

@@ -34,3 +34,26 @@ def test_long_chunks(n, n_bins):
     assert np.array_equal(got["bytes"][d], b.cpu().numpy().astype(np.uint64))
     assert not got["count"][1 - d].any() and not got["bytes"][1 - d].any()
     table.close()
+
+
+def test_whole_histogram_short_chunks(orc):
+    """A whole-histogram tile that leaves one CTA an SM, each with several chunks of one
+    quad a thread: every chunk's bins flushed, though consecutive chunks lie far apart."""
+    from helpers import assert_hist_equal, to_dev
+    from test_host_plans import prefixes
+
+    net, ln = prefixes(8000, 16, 24, 4)
+    n, n_bins = 600_001, 5000
+    rng = np.random.default_rng(1)
+    at = np.arange(n) // 2048 // 152 % 2  # a CTA's chunks in turn: the first bins, the last ones
+    rec = {"ts": (at * 4990 + rng.integers(0, 10, n)).astype(np.uint64), "src": rng.choice(net, n),
+           "dst": rng.integers(1 << 31, 1 << 32, n).astype(np.uint32),
+           "bytes": rng.integers(0, 1 << 32, n).astype(np.uint32)}
+    want = orc.discriminate_histogram(net, ln, rec, 0, 1, n_bins)
+    table, d = sinet.PrefixTable(net, ln), to_dev(rec)
+    for i in range(20):
+        out = sinet.Histogram(n_bins)
+        sinet.discriminate_histogram(table, d["ts"], d["src"], d["dst"], d["bytes"],
+                                     sinet.HistParams(0, 1, n_bins, strategy="smem_full"), out)
+        assert_hist_equal(out.to_numpy(), want, f"call {i}")
+    table.close()
