@@ -738,7 +738,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_part_split(PartDev p) {
                 if (lane >= (uint32_t)d) incl += y;
             }
             const uint32_t o0 = incl - c0 - c1, o1 = incl - c1;
-            cnt[2 * lane] = o0;  // (its own two words: nobody else reads them before the barrier)
+            cnt[2 * lane] = o0;  // (its own two words: nobody else reads them before the __syncwarp)
             cnt[2 * lane + 1] = o1;
             bool fits = true;
             if (c0) {
@@ -754,6 +754,7 @@ __global__ void __launch_bounds__(kSplitThreads, 1) k_part_split(PartDev p) {
                 fits = fits && q <= end && end - q >= c1;
             }
             fits = __all_sync(kFull, fits);
+            __syncwarp();  // every lane's cnt before the scatter reads them (a vote orders no memory)
 #pragma unroll
             for (int j = 0; j < U; ++j) {
                 if (j * 32 >= m) break;
