@@ -1085,13 +1085,15 @@ cudaError_t plan_partition(int lk, uint32_t table_smem, const RecArgs &r, const 
     o = align256(o + 4ull * tiles);
     P.off_hash_cnt = o;
     o = align256(o + (4ull << hb));
+    // zero, since a CTA whose table did not land leaves the main pass without
+    // storing its counts: its runs are then empty, and nothing reads beyond them
+    P.off_counts = o;
+    o = align256(o + 4ull * nb * G);
     P.bytes_zero = o - P.off_zero;
     P.off_cand = o;
     o = align256(o + 8ull * kPartMaxCand);
     P.off_base = o;
     o = align256(o + 4ull * (nb + 1));
-    P.off_counts = o;
-    o = align256(o + 4ull * nb * G);
     P.off_tile_base = o;
     o = align256(o + 4ull * (tiles + 1));
     P.off_tile_cur = o;

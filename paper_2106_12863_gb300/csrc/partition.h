@@ -74,7 +74,7 @@ struct PartDev {
     uint32_t *base;         // [n_buckets + 1]
     uint64_t *entries;      // [g_main][region]
     uint64_t region;
-    uint32_t *counts;       // [n_buckets][g_main] entries of every run
+    uint32_t *counts;       // [n_buckets][g_main] entries of every run (zero until its CTA stores them)
     uint64_t *ovf;          // [ovf_cap] entries that found their run full
     uint32_t *ovf_n;
     uint32_t ovf_cap;

@@ -65,4 +65,22 @@ int plan_batch_slice(const uint32_t *net, const uint8_t *len, uint32_t n_net, ui
     return 0;
 }
 
+// The partition of n aligned records into n_bins bins: {zeroed bytes' start and
+// end, run counts' start and end, scratch bytes}.
+int plan_partition_scratch(uint64_t n, uint32_t n_bins, int lean, uint64_t *out) {
+    RecArgs r{};
+    r.g = make_geom(n, {});
+    HistArgs h{};
+    h.n_bins = n_bins;
+    const DeviceState ds = gb300();
+    PartPlan p;
+    if (plan_partition(LK_LEAF2, 16384, r, h, 0, ds.sm_count, ds.smem_optin, lean != 0, &p) != cudaSuccess) return -1;
+    out[0] = p.off_zero;
+    out[1] = p.off_zero + p.bytes_zero;
+    out[2] = p.off_counts;
+    out[3] = p.off_counts + 4ull * p.d.n_buckets * p.d.g_main;
+    out[4] = p.scratch_bytes;
+    return 0;
+}
+
 }  // extern "C"

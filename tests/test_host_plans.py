@@ -53,3 +53,13 @@ def test_slices_of_one_list_in_both_forms(plans):
     assert (reduced["lookup"], reduced["start"]) == (hour["lookup"], hour["start"])
     for s in (hour, longer):
         assert s["bytes"] + 16 * s["tile_bins"] <= s["smem"]
+
+
+@pytest.mark.parametrize("lean", [0, 1])
+@pytest.mark.parametrize("n,n_bins", [(1, 1), (1_000_000, 10_000), (20_000_000, 21_600_000), (1_600_000_000, 86_400_000)])
+def test_partition_run_counts_start_at_zero(plans, n, n_bins, lean):
+    """A CTA of the main pass that leaves without storing its run counts leaves zeros, not stale memory."""
+    out = np.zeros(5, np.uint64)
+    assert plans.plan_partition_scratch(ctypes.c_uint64(n), ctypes.c_uint32(n_bins), lean, ctypes.c_void_p(out.ctypes.data)) == 0
+    zero0, zero1, counts0, counts1, total = out.tolist()
+    assert zero0 <= counts0 < counts1 <= zero1 <= total
