@@ -641,7 +641,7 @@ cudaError_t run_batch_expand(const BatchArgs &b, int grid, int sm_count, cudaStr
 }
 
 cudaError_t batch_occupancy(uint32_t smem, int *per_sm) {
-    cudaError_t e = cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = raise_smem_limit((const void *)k_batch, smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_batch, kBatchBlock, smem);
 }

@@ -588,6 +588,22 @@ struct KernelFacts {
 static std::mutex g_facts_mu;
 static std::map<std::pair<const void *, int>, KernelFacts> g_facts;
 
+// (g_facts_mu is held)
+static cudaError_t raise_limit(KernelFacts &f, const void *kernel, size_t smem) {
+    if (smem <= f.smem_limit) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) f.smem_limit = smem;
+    return e;
+}
+
+cudaError_t raise_smem_limit(const void *kernel, size_t smem) {
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(g_facts_mu);
+    return raise_limit(g_facts[{kernel, dev}], kernel, smem);
+}
+
 template <typename K>
 static cudaError_t launch(K kernel, size_t smem, const LaunchCfg &c, int &grid) {
     int dev = 0;
@@ -595,11 +611,7 @@ static cudaError_t launch(K kernel, size_t smem, const LaunchCfg &c, int &grid) 
     if (e != cudaSuccess) return e;
     std::lock_guard<std::mutex> lk(g_facts_mu);
     KernelFacts &f = g_facts[{(const void *)kernel, dev}];
-    if (smem > f.smem_limit) {
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        f.smem_limit = smem;
-    }
+    if ((e = raise_limit(f, (const void *)kernel, smem)) != cudaSuccess) return e;
     grid = c.grid;
     if (grid > 0) return cudaSuccess;
     if (f.per_sm.size() > 256) f.per_sm.clear();  // tables of many sizes
@@ -641,8 +653,7 @@ cudaError_t run_pack_finish(int lk, const RecArgs &r, const TableArgs &t, const 
     if (lk == L && (watch != nullptr) == WA) {                                                                \
         const size_t smem = Classifier<L>::smem_bytes(t);                                                     \
         const void *f = (const void *)k_pack_redo<L, WA>;                                                     \
-        e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);                  \
-        if (e != cudaSuccess) return e;                                                                       \
+        if ((e = raise_smem_limit(f, smem)) != cudaSuccess) return e;                                         \
         return cudaLaunchCooperativeKernel(f, dim3(c.sm_count), dim3(256), args, smem, c.stream);             \
     }
     SINET_REDO(LK_INTERVAL, false)

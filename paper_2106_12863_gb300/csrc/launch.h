@@ -50,6 +50,12 @@ cudaError_t run_cells_expand(const HistArgs &h, bool accumulate, const LaunchCfg
 cudaError_t run_pack_finish(int lk, const RecArgs &r, const TableArgs &t, const HistArgs &h, const LaunchCfg &c,
                             const TableArgs *watch);
 
+// Let launches of `kernel` on the current device have `smem` bytes of dynamic
+// shared memory. The limit is one per kernel and device: every launch whose size
+// varies (tables do) sets it here, where it is only ever raised, so no thread
+// finds it lowered by another one's between this call and its launch.
+cudaError_t raise_smem_limit(const void *kernel, size_t smem);
+
 // Largest dynamic shared memory a CTA may use on this device.
 size_t smem_optin_limit();
 

@@ -452,7 +452,7 @@ OwnerPlan plan_owner(uint64_t n, uint32_t n_bins, uint32_t slots, uint32_t grid)
 
 template <typename K>
 static cudaError_t kernel_grid(K kernel, size_t smem, const LaunchCfg &c, int &grid) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = raise_smem_limit((const void *)kernel, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, c.block, smem);

@@ -1111,7 +1111,7 @@ cudaError_t plan_partition(int lk, uint32_t table_smem, const RecArgs &r, const 
 
 template <typename K>
 static cudaError_t set_smem(K kernel, size_t smem) {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return raise_smem_limit((const void *)kernel, smem);
 }
 
 template <int LK>

@@ -556,8 +556,7 @@ cudaError_t run_sort_reduce(int lk, const RecArgs &r, const TableArgs &t, const 
     switch (lk) {
 #define SINET_EMIT(L)                                                                          \
     case L:                                                                                    \
-        e = cudaFuncSetAttribute(k_emit<L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-        if (e != cudaSuccess) return e;                                                        \
+        if ((e = raise_smem_limit((const void *)k_emit<L>, smem)) != cudaSuccess) return e;    \
         k_emit<L><<<(unsigned)plan.emit_tiles, kEmitThreads, smem, c.stream>>>(r, t, h, sa,    \
                                                                               plan.emit_tiles, c.status); \
         break;

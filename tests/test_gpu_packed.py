@@ -104,3 +104,41 @@ def test_batch_slices(orc):
             assert_hist_equal(s[-1].to_numpy(), ref, f"slice {i}")
     assert sinet.sinet_device_status() == 0
     batch.close()
+
+
+@pytest.mark.parametrize("strategy", ["global_atomic", "partition", "sort_reduce", "owner"])
+def test_two_threads_with_tables_of_two_sizes(strategy):
+    """Calls from two host threads whose tables need different amounts of shared memory."""
+    import threading
+
+    import torch
+    from test_host_plans import prefixes
+
+    n, n_bins, errors = 1_000_003, 10_000, []
+    g = torch.Generator(device="cuda").manual_seed(1)
+    ts = torch.randint(0, n_bins, (n,), dtype=torch.int64, device="cuda", generator=g)
+    ip = [torch.randint(-(1 << 31), 1 << 31, (n,), dtype=torch.int64, device="cuda", generator=g).to(torch.int32)
+          for _ in range(2)]
+    by = torch.randint(0, 1500, (n,), dtype=torch.int32, device="cuda", generator=g)
+    p = sinet.HistParams(0, 1, n_bins, strategy=strategy)
+    tables = [sinet.PrefixTable(*prefixes(k, 16, 24, 4)) for k in (16, 9000)]
+    torch.cuda.synchronize()
+
+    def work(table):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                out = sinet.Histogram(n_bins)
+                for _ in range(400):
+                    sinet.discriminate_histogram(table, ts, *ip, by, p, out)
+                torch.cuda.current_stream().synchronize()
+                assert int(out.stats[:4].sum()) == n
+        except Exception as e:  # noqa: BLE001 - reported by the test's thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(t,)) for t in tables]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    assert sinet.sinet_device_status() == 0
