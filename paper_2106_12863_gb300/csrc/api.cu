@@ -257,11 +257,10 @@ static cudaError_t run_cells(int lk, const RecArgs &r, const TableArgs &ta_tab, 
 static bool packed_pays(uint64_t n_bins, uint64_t n) {
     return 16 * n_bins <= (60ull << 20) && n >= 1000000 && n >= n_bins / 6;
 }
-// Not beyond 2^32 records, up to which the totals that check the cells cannot
-// wrap, and not while the stream is captured: a graph with an allocation of its
-// own can be instantiated only once at a time.
-static bool use_packed(const sinet_hist_params *p, uint64_t n, bool capturing) {
-    return !p->accumulate && !capturing && packed_pays(p->n_bins, n) && n < (1ull << 32);
+// Not while the stream is captured: a graph with an allocation of its own can be
+// instantiated only once at a time.
+static bool use_packed(const sinet_hist_params *p, const HistArgs &h, uint64_t n, bool capturing) {
+    return !p->accumulate && !capturing && packed_pays(p->n_bins, n) && packed_countable(n, h.two_dir != 0);
 }
 
 static bool is_capturing(cudaStream_t s) {
@@ -540,7 +539,7 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
         oplan = plan_owner(r.g.n, h.n_bins, S, (uint32_t)g);
     }
 
-    const bool packed = strat == SINET_STRAT_GLOBAL_ATOMIC && use_packed(p, r.g.n, capturing);
+    const bool packed = strat == SINET_STRAT_GLOBAL_ATOMIC && use_packed(p, h, r.g.n, capturing);
     if ((strat == SINET_STRAT_ATOMIC_CELL || strat == SINET_STRAT_OWNER || strat == SINET_STRAT_PARTITION || packed) &&
         !p->accumulate && r.g.n > 0) {
         // the expansion (cells), the owners or the cold pass write every bin;

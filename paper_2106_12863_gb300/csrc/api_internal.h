@@ -58,6 +58,10 @@ bool aligned(const void *p, size_t a);
 sinet_status check_params(const sinet_hist_params *p);
 sinet_status check_out(const sinet_hist_out *o);
 HistArgs make_hist(const sinet_hist_params *p, const sinet_hist_out *o);
+// Whether the totals that check packed cells (HistArgs::packed) hold every total
+// of n records: below 2^32 updates, whose bytes stay below 2^64. Past that the
+// byte totals wrap, and cells that lost 2^64 bytes and a count could agree.
+inline bool packed_countable(uint64_t n, bool two_dir) { return n < (two_dir ? 1ull << 31 : 1ull << 32); }
 sinet_status zero_outputs(const sinet_hist_params *p, const sinet_hist_out *o, cudaStream_t s);
 // The shared-memory form of a table that has one: its leaf form, else its toggle form.
 int staged_lookup(const sinet_prefix_table *t);

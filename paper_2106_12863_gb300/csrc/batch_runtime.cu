@@ -46,7 +46,8 @@ bool sort_feasible(const PlannedSlice &ps) {
 bool slice_packed(const PlannedSlice &ps) {
     const uint64_t n = ps.d.r.g.n, bins = ps.d.h.n_bins;
     return ps.d.zero && !ps.d.ready &&
-           (ps.strategy == SINET_STRAT_GLOBAL_ATOMIC || ps.strategy == SINET_STRAT_ATOMIC_NOAGG) && n < (1ull << 32) && n >= bins / (16 * bins <= (60ull << 20) ? 6 : 2);
+           (ps.strategy == SINET_STRAT_GLOBAL_ATOMIC || ps.strategy == SINET_STRAT_ATOMIC_NOAGG) &&
+           packed_countable(n, ps.d.h.two_dir != 0) && n >= bins / (16 * bins <= (60ull << 20) ? 6 : 2);
 }
 
 constexpr uint64_t kMinPackedBatch = 8000000;

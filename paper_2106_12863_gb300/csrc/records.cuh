@@ -47,8 +47,9 @@ struct HistArgs {
     // then the same as the expanded cells give them. A
     // cell whose byte sum reaches 2^kPackBits decodes to less than it holds, and
     // then one whose count alone overflows does, and nothing ever decodes to
-    // more: the totals agree exactly when every cell is right (and where they
-    // do not, the call is redone without cells).
+    // more: the totals, which stay below 2^64 (packed_countable), agree exactly
+    // when every cell is right (and where they do not, the call is redone
+    // without cells).
     uint64_t *packed;
     uint64_t *pack_sums;
 };

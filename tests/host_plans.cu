@@ -65,6 +65,18 @@ int plan_batch_slice(const uint32_t *net, const uint8_t *len, uint32_t n_net, ui
     return 0;
 }
 
+// Whether a batch slice of n records and n_bins bins on plain reductions takes packed cells.
+int plan_packed_slice(uint64_t n, uint32_t n_bins, int two_dir) {
+    PlannedSlice ps;
+    ps.d = BatchSlice{};
+    ps.d.r.g = make_geom(n, {});
+    ps.d.h.n_bins = n_bins;
+    ps.d.h.two_dir = two_dir != 0;
+    ps.d.zero = 1;
+    ps.strategy = SINET_STRAT_ATOMIC_NOAGG;
+    return slice_packed(ps);
+}
+
 // The partition of n aligned records into n_bins bins: {zeroed bytes' start and
 // end, run counts' start and end, scratch bytes}.
 int plan_partition_scratch(uint64_t n, uint32_t n_bins, int lean, uint64_t *out) {

@@ -63,3 +63,11 @@ def test_partition_run_counts_start_at_zero(plans, n, n_bins, lean):
     assert plans.plan_partition_scratch(ctypes.c_uint64(n), ctypes.c_uint32(n_bins), lean, ctypes.c_void_p(out.ctypes.data)) == 0
     zero0, zero1, counts0, counts1, total = out.tolist()
     assert zero0 <= counts0 < counts1 <= zero1 <= total
+
+
+def test_packed_cells_only_below_2_32_updates(plans):
+    """The totals that check packed cells count bytes modulo 2^64: 2^32 updates at most, both directions' together."""
+    packed = lambda n, two: plans.plan_packed_slice(ctypes.c_uint64(n), ctypes.c_uint32(1000), two)
+    for two, limit in ((0, 1 << 32), (1, 1 << 31)):
+        assert packed(limit - 1, two) and not packed(limit, two)
+        assert (limit - 1) * (1 + two) * ((1 << 32) - 1) < 1 << 64
