@@ -631,10 +631,10 @@ cudaError_t run_batch_zero(const BatchArgs &b, int grid, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t run_batch_expand(const BatchArgs &b, int grid, int sm_count, cudaStream_t s, uint32_t *status) {
+cudaError_t run_batch_expand(const BatchArgs &b, int grid, int sm_count, bool redo, cudaStream_t s, uint32_t *status) {
     k_batch_expand<<<grid, 256, 0, s>>>(b);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || !redo) return e;
     BatchArgs ba = b;
     void *args[] = {&ba, &status};
     return cudaLaunchCooperativeKernel((const void *)k_batch_redo, dim3(sm_count), dim3(256), args, 0, s);

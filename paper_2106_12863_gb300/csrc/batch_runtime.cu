@@ -233,7 +233,7 @@ sinet_status BatchEngine::capture(uint32_t *status) {
     if (e == cudaSuccess) {
         cudaError_t e1 = run_batch_zero(args, zgrid, cs);
         cudaError_t e2 = e1 == cudaSuccess ? run_batch(args, smem, grid, cs, status) : e1;
-        if (e2 == cudaSuccess && packed) e2 = run_batch_expand(args, zgrid, sm_count, cs, status);
+        if (e2 == cudaSuccess && packed) e2 = run_batch_expand(args, zgrid, sm_count, true, cs, status);
         // slices on the plain path: their outputs were zeroed (or are
         // accumulated into) like every other slice's, so the chain adds
         LaunchCfg lc;
@@ -413,7 +413,10 @@ sinet_status tune_one(const PlannedSlice &rep, const DeviceState *ds, uint32_t s
             e = cudaEventRecord(e0, s);
             if (e == cudaSuccess) e = run_batch_zero(eng.args, eng.zgrid, s);
             if (e == cudaSuccess) e = run_batch(eng.args, smem, eng.grid, s, ds->status);
-            if (e == cudaSuccess && packed) e = run_batch_expand(eng.args, eng.zgrid, ds->sm_count, s, ds->status);
+            // copies that share an area share its cells and totals: no redo, which
+            // counts a slice's arrivals there (the copies' sums are nobody's result)
+            if (e == cudaSuccess && packed)
+                e = run_batch_expand(eng.args, eng.zgrid, ds->sm_count, separate, s, ds->status);
             if (e == cudaSuccess) e = cudaEventRecord(e1, s);
             if (e == cudaSuccess) e = cudaEventSynchronize(e1);
             float t = 0.f;

@@ -120,9 +120,9 @@ cudaError_t run_batch_zero(const BatchArgs &b, int grid, cudaStream_t s);
 // CTA (table region + work region of any slice must fit).
 cudaError_t run_batch(const BatchArgs &b, uint32_t smem, int grid, cudaStream_t s, uint32_t *status);
 // After it, where slices use packed cells (HistArgs::packed): their expansion
-// into the outputs (with the zeroing kernel's grid), and the slices redone whose
-// totals show that a cell overflowed.
-cudaError_t run_batch_expand(const BatchArgs &b, int grid, int sm_count, cudaStream_t s, uint32_t *status);
+// into the outputs (with the zeroing kernel's grid), and, with `redo`, the slices
+// redone whose totals show that a cell overflowed (every slice has cells of its own).
+cudaError_t run_batch_expand(const BatchArgs &b, int grid, int sm_count, bool redo, cudaStream_t s, uint32_t *status);
 // Set the batch kernel's dynamic shared memory limit; returns CTAs per SM.
 cudaError_t batch_occupancy(uint32_t smem, int *per_sm);
 

@@ -44,3 +44,25 @@ def test_batches_around_the_line(total):
             assert np.array_equal(got["bytes"][d], b.cpu().numpy().astype(got["bytes"].dtype))
             assert not got["count"][1 - d].any() and not got["bytes"][1 - d].any()
     batch.close()
+
+
+@pytest.mark.parametrize("n_bins", [2_000_003, 300_001], ids=["shared area", "areas of their own"])
+def test_tuning_a_slice_that_overflows_a_cell(n_bins):
+    """The tuner times copies of a slice whose cells overflow; no wait of theirs runs out."""
+    table = sinet.PrefixTable(np.array([0], np.uint32), np.array([1], np.uint8))
+    n = 1_000_003
+    g = torch.Generator(device="cuda").manual_seed(n_bins)
+    # ten copies of 40 bytes a bin: beyond the tuner's 512 MB with the larger histogram
+    ts = torch.randint(0, n_bins, (n,), dtype=torch.int64, device="cuda", generator=g)
+    src = torch.randint(1, 1 << 31, (n,), dtype=torch.int64, device="cuda", generator=g).to(torch.int32)
+    dst = torch.full((n,), -1, dtype=torch.int32, device="cuda")  # outside
+    by = torch.randint(0, 1 << 30, (n,), dtype=torch.int32, device="cuda", generator=g)
+    ts[:2000], by[:2000] = 77, -1
+    out = sinet.Histogram(n_bins)
+    # a width of 7 ms, which no other test of this size has: a class not tuned before
+    batch = sinet.Batch([(table, ts * 7, src, dst, by, sinet.HistParams(0, 7, n_bins), out)], autotune=True)
+    batch.run()
+    torch.cuda.synchronize()
+    assert sinet.sinet_device_status() == 0
+    assert torch.equal(out.count[0].long() + out.count[1], torch.bincount(ts, minlength=n_bins))
+    batch.close()
