@@ -332,6 +332,14 @@ sinet_status sinet_discriminate_histogram_noalloc(const sinet_prefix_table *t, c
  * histogram with the strategy chosen for it. The launch (a zeroing kernel
  * for non-accumulating slices, then the batch kernel) is captured once as a
  * CUDA graph at creation; sinet_batch_run replays it.
+ *
+ * Non-accumulating slices without a ready word that run on global reductions
+ * and have enough records (one per six bins, per two where 16 bytes a bin
+ * exceed 60 MB; 8 M in all such slices) add into packed cells instead of their
+ * outputs: 16 bytes a bin, allocated at creation after everything else and held
+ * for the batch's life. Two further kernels of the graph expand the cells into
+ * the outputs and redo a slice one of whose cells overflowed, straight into its
+ * outputs. Where the cells cannot be had, the slices add into their outputs.
  */
 typedef struct {
     const uint64_t *ts;               /* device records, as in sinet_discriminate_histogram */

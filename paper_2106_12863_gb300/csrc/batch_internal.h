@@ -92,6 +92,8 @@ struct BatchEngine {
     void image(const std::vector<PlannedSlice> &v, std::vector<uint8_t> &buf) const;
     // packed cells for the slices of v that gain by them (before image and capture)
     void plan_packed(std::vector<PlannedSlice> &v);
+    // without them after all
+    void drop_packed(std::vector<PlannedSlice> &v);
     // scratch for the slices of v run by the plain path (before capture)
     sinet_status plan_sorts(const std::vector<PlannedSlice> &v, const DeviceState *ds);
     sinet_status capture(uint32_t *status);  // capture zero + batch kernels (+ plain chains) as a graph

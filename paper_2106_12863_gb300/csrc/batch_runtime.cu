@@ -210,6 +210,18 @@ void BatchEngine::plan_packed(std::vector<PlannedSlice> &v) {
     }
 }
 
+void BatchEngine::drop_packed(std::vector<PlannedSlice> &v) {
+    if (exec) cudaGraphExecDestroy(exec);
+    if (graph) cudaGraphDestroy(graph);
+    exec = nullptr;
+    graph = nullptr;
+    cudaFree(cells);
+    cudaGetLastError();
+    cells = nullptr;
+    packed = false;
+    for (PlannedSlice &ps : v) ps.d.h.packed = ps.d.h.pack_sums = nullptr;
+}
+
 sinet_status BatchEngine::plan_sorts(const std::vector<PlannedSlice> &v, const DeviceState *ds) {
     (void)ds;
     for (const PlannedSlice &ps : v) {
@@ -587,16 +599,19 @@ sinet_status sinet_batch_create(const sinet_batch_slice *slices, uint32_t n_slic
     b->items = items;
     b->records = records;
     st = b->eng.init(n_slices, ds, smem);
-    if (st == SINET_OK) b->eng.plan_packed(v);
+    // the plain path's scratch first: it must be had, the cells need not
     if (st == SINET_OK) st = b->eng.plan_sorts(v, ds);
+    if (st == SINET_OK) b->eng.plan_packed(v);
     std::vector<uint8_t> buf;
-    if (st == SINET_OK) {
+    while (st == SINET_OK) {
         b->eng.image(v, buf);
         cudaError_t e = cudaMemcpyAsync(b->eng.d_mem, buf.data(), buf.size(), cudaMemcpyHostToDevice, stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(stream);  // host image goes out of scope
-        if (e != cudaSuccess) st = cuda_fail(e);
+        st = e == cudaSuccess ? b->eng.capture(ds->status) : cuda_fail(e);
+        if (st != SINET_ERR_OOM || !b->eng.packed) break;
+        b->eng.drop_packed(v);  // the graph found no room beside the cells
+        st = SINET_OK;
     }
-    if (st == SINET_OK) st = b->eng.capture(ds->status);
     if (st != SINET_OK) {
         b->eng.release();
         delete b;

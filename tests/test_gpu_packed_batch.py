@@ -14,6 +14,23 @@ if not torch.cuda.is_available():  # pragma: no cover - collected on CPU too
 import paper_2106_12863_gb300 as sinet  # noqa: E402
 
 
+@pytest.fixture
+def free_memory():
+    """A function that takes device memory until about so many bytes are free; given back after the test."""
+    held = []
+
+    def leave(nbytes):
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        spare = torch.cuda.mem_get_info()[0] - nbytes
+        assert spare > 0
+        held.append(torch.empty(spare, dtype=torch.uint8, device="cuda"))
+
+    yield leave
+    held.clear()
+    torch.cuda.empty_cache()
+
+
 @pytest.mark.parametrize("total", [7_999_999, 8_000_000])
 def test_batches_around_the_line(total):
     table = sinet.PrefixTable(np.array([0], np.uint32), np.array([1], np.uint8))
@@ -65,4 +82,27 @@ def test_tuning_a_slice_that_overflows_a_cell(n_bins):
     torch.cuda.synchronize()
     assert sinet.sinet_device_status() == 0
     assert torch.equal(out.count[0].long() + out.count[1], torch.bincount(ts, minlength=n_bins))
+    batch.close()
+
+
+def test_cells_give_way_to_the_plain_path(free_memory):
+    """Memory for the plain path's scratch or for packed cells, not for both: the cells are left out."""
+    table = sinet.PrefixTable(np.array([0], np.uint32), np.array([1], np.uint8))
+    n, n_bins = 20_000_003, 20_000_000
+    g = torch.Generator(device="cuda").manual_seed(9)
+    ts = torch.randint(0, n_bins, (n,), dtype=torch.int64, device="cuda", generator=g)
+    src = torch.randint(1, 1 << 31, (n,), dtype=torch.int64, device="cuda", generator=g).to(torch.int32)
+    dst = torch.full((n,), -1, dtype=torch.int32, device="cuda")  # outside
+    by = torch.randint(0, 1 << 30, (n,), dtype=torch.int32, device="cuda", generator=g)
+    outs = [sinet.Histogram(n_bins) for _ in range(2)]
+    # 320 MB of cells, 330 MB of scratch
+    free_memory(480 << 20)
+    batch = sinet.Batch([(table, ts, src, dst, by, sinet.HistParams(0, 1, n_bins, strategy=s), o)
+                         for s, o in zip(("global_atomic", "sort_reduce"), outs)])
+    batch.run()
+    torch.cuda.synchronize()
+    assert sinet.sinet_device_status() == 0
+    for k in ("count", "bytes", "stats"):
+        assert torch.equal(getattr(outs[0], k), getattr(outs[1], k)), k
+    assert int(outs[0].stats[:4].sum()) == n
     batch.close()
