@@ -392,6 +392,16 @@ class HistParams:
             self.watch.handle if self.watch is not None else None)
 
 
+def _rows(a):
+    """Addresses of the two directions' rows of a tensor, or of a pair of tensors."""
+    if len(a) < 2:
+        raise IndexError("count and bytes hold a row per direction")
+    if not hasattr(a, "data_ptr"):
+        return _Two(a[0].data_ptr(), a[1].data_ptr())
+    p = a.data_ptr()  # (without a view of each row: that took longer than the library's whole call)
+    return _Two(p, p + a.stride(0) * a.element_size())
+
+
 class Histogram:
     """Device outputs: count[2, n_bins] (uint32 bits in int32), bytes[2, n_bins]
     (uint64 bits in int64) and stats[8] (uint64 bits in int64)."""
@@ -407,14 +417,7 @@ class Histogram:
         self.stats = mk(8, dtype=torch.int64, device=device)
 
     def c(self) -> HistOutC:
-        # (the rows' addresses without a tensor view of each: that took longer
-        # than the library's whole call)
-        c, b = self.count, self.bytes
-        if len(c) < 2 or len(b) < 2:
-            raise IndexError("count and bytes hold a row per direction")
-        c0, b0 = c.data_ptr(), b.data_ptr()
-        return HistOutC(_Two(c0, c0 + c.stride(0) * c.element_size()), _Two(b0, b0 + b.stride(0) * b.element_size()),
-                        self.stats.data_ptr())
+        return HistOutC(_rows(self.count), _rows(self.bytes), self.stats.data_ptr())
 
     def to_numpy(self) -> dict:
         return {"count": self.count.cpu().numpy().view(np.uint32),

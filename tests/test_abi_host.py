@@ -446,3 +446,20 @@ def test_ctypes_layouts_and_constants_match_the_header(tmp_path):
             assert int(got[f"{cname}.{fname}"]) == getattr(cls, fname).offset, f"{cname}.{fname}"
     for name, v in consts.items():
         assert int(got[name]) == v, name
+
+
+def test_histogram_rows_as_a_tensor_and_as_a_pair():
+    """count and bytes are a tensor of two rows (of any row stride) or a pair of tensors."""
+    import torch
+
+    h = sinet.Histogram(8, device="cpu")
+    wide = torch.zeros((2, 20), dtype=torch.int32)
+    for count in (h.count, wide[:, 3:11], [h.count[1], wide[0]], (wide[1], h.count[0])):
+        h.count = count
+        h.bytes = [torch.zeros(8, dtype=torch.int64) for _ in range(2)]
+        o = h.c()
+        assert list(o.count) == [count[0].data_ptr(), count[1].data_ptr()]
+        assert list(o.bytes) == [h.bytes[0].data_ptr(), h.bytes[1].data_ptr()]
+    h.count = wide[:1]
+    with pytest.raises(IndexError):
+        h.c()
