@@ -545,7 +545,9 @@ sinet_status sinet_histogram_sparse(const sinet_hist_out *in, uint64_t n_bins, u
  * least one record per four bins (the 32-byte cells where the partition's
  * limits are exceeded, or where its scratch does not fit the free device
  * memory at the call) or of 90 MB or more with at least 6 M records, warp
- * combining otherwise). No kernel runs.
+ * combining otherwise). The answer is for outputs whose rows share no memory
+ * and a stream that is not captured: rows that overlap, and below 256 MB a
+ * capture, take warp combining where this names the partition. No kernel runs.
  */
 sinet_status sinet_auto_strategy(const sinet_prefix_table *t, uint64_t n, const sinet_hist_params *p,
                                  int32_t *strategy);

@@ -152,6 +152,32 @@ HistArgs make_hist(const sinet_hist_params *p, const sinet_hist_out *o) {
     return h;
 }
 
+void output_ranges(const HistArgs &h, uint32_t owner, std::vector<OutputRange> &v) {
+    for (int d = 0; d < 2; ++d) {
+        const uintptr_t c = (uintptr_t)h.cnt[d], b = (uintptr_t)h.byt[d];
+        v.push_back({c, c + 4 * (uintptr_t)h.n_bins, owner});
+        v.push_back({b, b + 8 * (uintptr_t)h.n_bins, owner});
+    }
+}
+
+void mark_overlaps(std::vector<OutputRange> &v, std::vector<bool> &mark) {
+    std::sort(v.begin(), v.end(), [](const OutputRange &a, const OutputRange &b) { return a.lo < b.lo; });
+    size_t far = 0;  // the range before i that ends last
+    for (size_t i = 1; i < v.size(); ++i) {
+        if (v[i].lo < v[far].hi) mark[v[i].owner] = mark[v[far].owner] = true;
+        if (v[i].hi > v[far].hi) far = i;
+    }
+}
+
+bool rows_apart(const HistArgs &h) {
+    if (!h.cnt[0]) return true;  // no outputs given (sinet_auto_strategy)
+    const uintptr_t lo[4] = {(uintptr_t)h.cnt[0], (uintptr_t)h.cnt[1], (uintptr_t)h.byt[0], (uintptr_t)h.byt[1]};
+    for (int i = 0; i < 4; ++i)
+        for (int k = 0; k < 4; ++k)
+            if (k != i && lo[k] >= lo[i] && lo[k] < lo[i] + (i < 2 ? 4 : 8) * (uintptr_t)h.n_bins) return false;
+    return true;
+}
+
 sinet_status zero_outputs(const sinet_hist_params *p, const sinet_hist_out *o, cudaStream_t s) {
     if (p->accumulate) return SINET_OK;
     SINET_CUDA(cudaMemsetAsync(o->count[0], 0, 4 * p->n_bins, s));
@@ -228,9 +254,6 @@ static uint32_t tile_capacity_pair(const DeviceState *ds, uint32_t tsm) {
     return (uint32_t)((per_cta - used) / 16) & ~3u;
 }
 
-// What AUTO runs without a measurement: the whole-histogram tile for small
-// histograms, the chunk tile for time-sorted input, the cells for unsorted
-// input over a histogram far beyond L2, warp combining otherwise.
 // The cell strategy: zeroed cells, the combining kernel into them, then the
 // expansion into the outputs.
 static cudaError_t run_cells(int lk, const RecArgs &r, const TableArgs &ta_tab, HistArgs h,
@@ -260,7 +283,8 @@ static bool packed_pays(uint64_t n_bins, uint64_t n) {
 // Not while the stream is captured: a graph with an allocation of its own can be
 // instantiated only once at a time.
 static bool use_packed(const sinet_hist_params *p, const HistArgs &h, uint64_t n, bool capturing) {
-    return !p->accumulate && !capturing && packed_pays(p->n_bins, n) && packed_countable(n, h.two_dir != 0);
+    return !p->accumulate && !capturing && packed_pays(p->n_bins, n) && packed_countable(n, h.two_dir != 0) &&
+           rows_apart(h);
 }
 
 static bool is_capturing(cudaStream_t s) {
@@ -287,6 +311,9 @@ static cudaError_t run_packed(int lk, const RecArgs &r, const TableArgs &tab, Hi
     return e == cudaSuccess ? e2 : e;
 }
 
+// What AUTO runs without a measurement: the whole-histogram tile for small
+// histograms, the chunk tile for time-sorted input, the partition (else the
+// cells) for unsorted input over large histograms, warp combining otherwise.
 static int auto_rule(const sinet_hist_params *p, const RecArgs &r, uint32_t cap, int lk, uint32_t tsm,
                      const HistArgs &h, const DeviceState *ds, bool capturing) {
     if (2ull * p->n_bins <= 8192 && p->n_bins <= cap) return SINET_STRAT_SMEM_FULL;
@@ -301,8 +328,9 @@ static int auto_rule(const sinet_hist_params *p, const RecArgs &r, uint32_t cap,
     // fixed costs (about 80 us) lose below some 5 M records, and to warp
     // combining where bins outnumber records
     const bool large = 24 * p->n_bins >= kCellMinHistBytes;
-    if (large ? r.g.n >= p->n_bins / 4
-              : !capturing && 24 * p->n_bins >= kPartMinHistBytes && r.g.n >= kPartMinRecords) {
+    if ((large ? r.g.n >= p->n_bins / 4
+               : !capturing && 24 * p->n_bins >= kPartMinHistBytes && r.g.n >= kPartMinRecords) &&
+        rows_apart(h)) {
         PartPlan probe{};
         if (plan_partition(lk, tsm, r, h, 0, ds->sm_count, ds->smem_optin, false, &probe) == cudaSuccess)
             return SINET_STRAT_PARTITION;

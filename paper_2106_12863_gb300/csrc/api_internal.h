@@ -1,6 +1,7 @@
 // Host helpers shared by the C-ABI translation units.
 #pragma once
 #include <initializer_list>
+#include <vector>
 
 #include <nvtx3/nvToolsExt.h>
 
@@ -58,6 +59,17 @@ bool aligned(const void *p, size_t a);
 sinet_status check_params(const sinet_hist_params *p);
 sinet_status check_out(const sinet_hist_out *o);
 HistArgs make_hist(const sinet_hist_params *p, const sinet_hist_out *o);
+// An update adds to its output words, so outputs may share memory: two slices
+// of a batch that fill one histogram, both directions in one array. What stores
+// every bin of its outputs instead asks here whether they stand apart.
+struct OutputRange {
+    uintptr_t lo, hi;
+    uint32_t owner;
+};
+void output_ranges(const HistArgs &h, uint32_t owner, std::vector<OutputRange> &v);
+// Sets mark[owner] for every owner of a range that overlaps another range.
+void mark_overlaps(std::vector<OutputRange> &v, std::vector<bool> &mark);
+bool rows_apart(const HistArgs &h);
 // Whether the totals that check packed cells (HistArgs::packed) hold every total
 // of n records: below 2^32 updates, whose bytes stay below 2^64. Past that the
 // byte totals wrap, and cells that lost 2^64 bytes and a count could agree.

@@ -185,12 +185,17 @@ void BatchEngine::image(const std::vector<PlannedSlice> &v, std::vector<uint8_t>
 }
 
 void BatchEngine::plan_packed(std::vector<PlannedSlice> &v) {
+    // the expansion stores every bin, so not where outputs share memory
+    std::vector<OutputRange> ranges;
+    std::vector<bool> shared(v.size());
+    for (size_t i = 0; i < v.size(); ++i) output_ranges(v[i].d.h, (uint32_t)i, ranges);
+    mark_overlaps(ranges, shared);
     size_t total = 0;
     uint64_t records = 0;
-    for (const PlannedSlice &ps : v)
-        if (slice_packed(ps)) {
-            total += packed_bytes(ps.d.h.n_bins);
-            records += ps.d.r.g.n;
+    for (size_t i = 0; i < v.size(); ++i)
+        if (slice_packed(v[i]) && !shared[i]) {
+            total += packed_bytes(v[i].d.h.n_bins);
+            records += v[i].d.r.g.n;
         }
     // the expansion's and the redo's kernels cost what the reductions of some
     // 8 M records save (55 slices of 10 K to 168 K records: 582 us, without 508)
@@ -202,11 +207,12 @@ void BatchEngine::plan_packed(std::vector<PlannedSlice> &v) {
     }
     packed = true;
     uint8_t *m = static_cast<uint8_t *>(cells);
-    for (PlannedSlice &ps : v) {
-        if (!slice_packed(ps)) continue;
-        ps.d.h.pack_sums = reinterpret_cast<uint64_t *>(m);
-        ps.d.h.packed = ps.d.h.pack_sums + 8;
-        m += packed_bytes(ps.d.h.n_bins);
+    for (size_t i = 0; i < v.size(); ++i) {
+        HistArgs &h = v[i].d.h;
+        if (!slice_packed(v[i]) || shared[i]) continue;
+        h.pack_sums = reinterpret_cast<uint64_t *>(m);
+        h.packed = h.pack_sums + 8;
+        m += packed_bytes(h.n_bins);
     }
 }
 

@@ -77,6 +77,25 @@ int plan_packed_slice(uint64_t n, uint32_t n_bins, int two_dir) {
     return slice_packed(ps);
 }
 
+// Which of n histograms' outputs (count[0], count[1], bytes[0], bytes[1] and
+// bins each) overlap any other rows: by the batch's sweep, and each by itself.
+void output_overlaps(const uint64_t *at, const uint32_t *bins, uint32_t n, uint8_t *shared, uint8_t *rows_overlap) {
+    std::vector<OutputRange> v;
+    std::vector<bool> mark(n);
+    for (uint32_t i = 0; i < n; ++i) {
+        HistArgs h{};
+        for (int d = 0; d < 2; ++d) {
+            h.cnt[d] = reinterpret_cast<uint32_t *>(at[4 * i + d]);
+            h.byt[d] = reinterpret_cast<uint64_t *>(at[4 * i + 2 + d]);
+        }
+        h.n_bins = bins[i];
+        output_ranges(h, i, v);
+        rows_overlap[i] = !rows_apart(h);
+    }
+    mark_overlaps(v, mark);
+    for (uint32_t i = 0; i < n; ++i) shared[i] = mark[i];
+}
+
 // The partition of n aligned records into n_bins bins: {zeroed bytes' start and
 // end, run counts' start and end, scratch bytes}.
 int plan_partition_scratch(uint64_t n, uint32_t n_bins, int lean, uint64_t *out) {

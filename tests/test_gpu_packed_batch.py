@@ -106,3 +106,63 @@ def test_cells_give_way_to_the_plain_path(free_memory):
         assert torch.equal(getattr(outs[0], k), getattr(outs[1], k)), k
     assert int(outs[0].stats[:4].sum()) == n
     batch.close()
+
+
+def _uniform(n, n_bins, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    ts = torch.randint(0, n_bins, (n,), dtype=torch.int64, device="cuda", generator=g)
+    ip = [torch.randint(-(1 << 31), 1 << 31, (n,), dtype=torch.int64, device="cuda", generator=g).to(torch.int32)
+          for _ in range(2)]
+    return ts, *ip, torch.randint(0, 1 << 30, (n,), dtype=torch.int32, device="cuda", generator=g)
+
+
+def test_slices_that_fill_one_histogram():
+    """Slices whose outputs are the same rows, overlap in part, or are added to by another slice."""
+    table = sinet.PrefixTable(np.array([0], np.uint32), np.array([1], np.uint8))
+    n, n_bins = 3_000_001, 100_000
+    recs = [_uniform(n, n_bins, i) for i in range(5)]
+    apart = [sinet.Histogram(n_bins) for _ in recs]
+    for r, o in zip(recs, apart):
+        sinet.discriminate_histogram(table, *r, sinet.HistParams(0, 1, n_bins, strategy="atomic_noagg"), o)
+    one, alone = sinet.Histogram(n_bins), sinet.Histogram(n_bins)
+    day = sinet.Histogram(150_000)
+
+    class Part:  # bins [first, first + n_bins) of the day
+        def __init__(self, first):
+            self.h = sinet.Histogram(1)
+            self.h.count, self.h.bytes = day.count[:, first:first + n_bins], day.bytes[:, first:first + n_bins]
+
+        def c(self):
+            return self.h.c()
+
+    parts = [Part(0), Part(50_000)]
+    p = sinet.HistParams(0, 1, n_bins, strategy="atomic_noagg")
+    add = sinet.HistParams(0, 1, n_bins, strategy="global_atomic", accumulate=True)
+    batch = sinet.Batch([(table, *recs[0], p, one), (table, *recs[1], add, one), (table, *recs[2], p, parts[0]),
+                         (table, *recs[3], p, parts[1]), (table, *recs[4], p, alone)])
+    for _ in range(2):
+        batch.run()
+    torch.cuda.synchronize()
+    for k in ("count", "bytes"):
+        a = [getattr(h, k) for h in apart]
+        assert torch.equal(getattr(one, k), a[0] + a[1]), k
+        want = torch.zeros_like(getattr(day, k))
+        want[:, :n_bins] += a[2]
+        want[:, 50_000:] += a[3]
+        assert torch.equal(getattr(day, k), want), k
+        assert torch.equal(getattr(alone, k), a[4]), k
+    batch.close()
+
+
+@pytest.mark.parametrize("strategy,n,n_bins", [("global_atomic", 1_000_003, 100_000), ("auto", 1_000_003, 100_000),
+                                               ("auto", 6_000_001, 4_000_000)])
+def test_both_directions_in_one_row(strategy, n, n_bins):
+    table = sinet.PrefixTable(np.array([0], np.uint32), np.array([1], np.uint8))
+    rec = _uniform(n, n_bins, 7)
+    two, one = sinet.Histogram(n_bins), sinet.Histogram(n_bins)
+    sinet.discriminate_histogram(table, *rec, sinet.HistParams(0, 1, n_bins, strategy="atomic_noagg"), two)
+    count, nbytes = one.count[0], one.bytes[0]
+    one.count, one.bytes = [count, count], [nbytes, nbytes]
+    sinet.discriminate_histogram(table, *rec, sinet.HistParams(0, 1, n_bins, strategy=strategy), one)
+    assert torch.equal(count, two.count.sum(0, dtype=torch.int32))
+    assert torch.equal(nbytes, two.bytes.sum(0))

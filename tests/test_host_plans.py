@@ -71,3 +71,21 @@ def test_packed_cells_only_below_2_32_updates(plans):
     for two, limit in ((0, 1 << 32), (1, 1 << 31)):
         assert packed(limit - 1, two) and not packed(limit, two)
         assert (limit - 1) * (1 + two) * ((1 << 32) - 1) < 1 << 64
+
+
+@pytest.mark.parametrize("seed", range(40))
+def test_outputs_that_share_memory(plans, seed):
+    """What keeps a slice or a call out of the schemes that store every bin, against every pair of rows."""
+    rng = np.random.default_rng(seed)
+    n = int(rng.integers(1, 9))
+    bins = rng.integers(1, 50, n).astype(np.uint32)
+    at = (4096 + 8 * rng.integers(0, (200, 2000)[seed % 2], (n, 4))).astype(np.uint64)
+    shared, own = np.zeros(n, np.uint8), np.zeros(n, np.uint8)
+    plans.output_overlaps(*(ctypes.c_void_p(a.ctypes.data) for a in (at, bins)), ctypes.c_uint32(n),
+                          *(ctypes.c_void_p(a.ctypes.data) for a in (shared, own)))
+    rows = [(i, int(at[i, k]), int(at[i, k]) + (4, 4, 8, 8)[k] * int(bins[i])) for i in range(n) for k in range(4)]
+    meets = lambda a, b: a is not b and a[1] < b[2] and b[1] < a[2]
+    for i in range(n):
+        mine = [r for r in rows if r[0] == i]
+        assert shared[i] == any(meets(a, b) for a in mine for b in rows)
+        assert own[i] == any(meets(a, b) for a in mine for b in mine)
