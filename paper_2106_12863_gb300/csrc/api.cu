@@ -581,16 +581,17 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
     if (r.g.n == 0) return SINET_OK;
 
     cudaError_t e = cudaSuccess;
+    // where scratch cannot be had: combining straight into the outputs, which takes none
+    auto straight = [&]() {
+        cudaGetLastError();
+        st = zero_outputs(p, o, s);
+        return st == SINET_OK ? run_fused_atomic(lk, true, r, ta_tab, h, kCacheSetBits, c, watch) : cudaSuccess;
+    };
     switch (strat) {
         case SINET_STRAT_GLOBAL_ATOMIC:
             if (packed) {
                 e = run_packed(lk, r, ta_tab, h, c, s, watch);
-                if (e == cudaErrorMemoryAllocation) {  // no room for the cells: straight into the outputs
-                    cudaGetLastError();
-                    st = zero_outputs(p, o, s);
-                    if (st != SINET_OK) return st;
-                    e = run_fused_atomic(lk, true, r, ta_tab, h, kCacheSetBits, c, watch);
-                }
+                if (e == cudaErrorMemoryAllocation) e = straight();
                 break;
             }
             e = run_fused_atomic(lk, true, r, ta_tab, h, kCacheSetBits, c, watch);
@@ -600,6 +601,7 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
             break;
         case SINET_STRAT_ATOMIC_CELL:
             e = run_cells(lk, r, ta_tab, h, p, c, s, watch);
+            if (e == cudaErrorMemoryAllocation && p->strategy == SINET_STRAT_AUTO) e = straight();
             break;
         case SINET_STRAT_PRIV_TILE:
         case SINET_STRAT_SMEM_FULL:
@@ -634,6 +636,7 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
                 // far less scratch and zero the same outputs (none)
                 cudaGetLastError();
                 e = run_cells(lk, r, ta_tab, h, p, c, s);
+                if (e == cudaErrorMemoryAllocation) e = straight();
                 break;
             }
             if (e != cudaSuccess) return cuda_fail(e);
@@ -656,7 +659,7 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
             e = cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return cuda_fail(e);
-    return SINET_OK;
+    return st;
 }
 
 }  // namespace sinet

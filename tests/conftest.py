@@ -33,3 +33,22 @@ def orc():
     import oracle
 
     return oracle.get()
+
+
+@pytest.fixture
+def free_memory():
+    """A function that takes device memory until about so many bytes are free; given back after the test."""
+    import torch
+
+    held = []
+
+    def leave(nbytes):
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        spare = torch.cuda.mem_get_info()[0] - nbytes
+        assert spare > 0
+        held.append(torch.empty(spare, dtype=torch.uint8, device="cuda"))
+
+    yield leave
+    held.clear()
+    torch.cuda.empty_cache()

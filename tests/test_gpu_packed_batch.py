@@ -14,23 +14,6 @@ if not torch.cuda.is_available():  # pragma: no cover - collected on CPU too
 import paper_2106_12863_gb300 as sinet  # noqa: E402
 
 
-@pytest.fixture
-def free_memory():
-    """A function that takes device memory until about so many bytes are free; given back after the test."""
-    held = []
-
-    def leave(nbytes):
-        torch.cuda.synchronize()
-        torch.cuda.empty_cache()
-        spare = torch.cuda.mem_get_info()[0] - nbytes
-        assert spare > 0
-        held.append(torch.empty(spare, dtype=torch.uint8, device="cuda"))
-
-    yield leave
-    held.clear()
-    torch.cuda.empty_cache()
-
-
 @pytest.mark.parametrize("total", [7_999_999, 8_000_000])
 def test_batches_around_the_line(total):
     table = sinet.PrefixTable(np.array([0], np.uint32), np.array([1], np.uint8))

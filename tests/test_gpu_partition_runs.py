@@ -76,3 +76,26 @@ def test_misleading_sample(orc, n_bins, elsewhere):
     far = (np.arange(n) // 512 % stride != 0) & (rng.random(n) < elsewhere)
     ts[far] = 7 + n_bins // 2 + rng.integers(0, 2000, int(far.sum()))
     _check(orc, _records(ts, 4), n_bins)
+
+
+@pytest.mark.parametrize("accumulate", [False, True])
+@pytest.mark.parametrize("n_bins", [4_000_000, 12_000_000], ids=["96 MB", "288 MB"])
+def test_auto_without_room_for_scratch(orc, free_memory, n_bins, accumulate):
+    """AUTO's partition, and the cells that replace it, do not fit: the call runs without scratch."""
+    import torch
+
+    table = sinet.PrefixTable(*NET)
+    rng = np.random.default_rng(n_bins)
+    rec = _records(rng.integers(0, n_bins, 6_000_001), 3)
+    d = to_dev(rec)
+    p = sinet.HistParams(0, 1, n_bins, accumulate=accumulate)
+    assert sinet.auto_strategy(table, len(rec["ts"]), p) == "partition"
+    out = sinet.Histogram(n_bins)
+    if not accumulate:
+        out.count.fill_(-1)
+        out.bytes.fill_(-1)
+    free_memory(48 << 20)  # the partition takes over 100 MB, the cells 32 bytes a bin
+    sinet.discriminate_histogram(table, d["ts"], d["src"], d["dst"], d["bytes"], p, out)
+    torch.cuda.synchronize()
+    assert_hist_equal(out.to_numpy(), orc.discriminate_histogram(*NET, rec, 0, 1, n_bins))
+    assert sinet.sinet_device_status() == 0
