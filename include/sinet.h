@@ -96,8 +96,8 @@ typedef enum {
                                       8-byte (bin, direction, bytes) entry to the CTA's run of its
                                       bin range, large histograms' runs are split by tile of bins,
                                       and each tile is summed in shared memory and every bin of it
-                                      stored once. The outputs need no zeroing and see no
-                                      read-modify-write. tile_bins, a power of two of at most 2^20,
+                                      stored once (accumulating: added to, where it has updates).
+                                      The outputs need no zeroing. tile_bins, a power of two of at most 2^20,
                                       asks for that many bins per range (taken to the nearest size
                                       the cold pass sums without a split: one to eight tiles of at
                                       most 2^13 bins; default: as measured best).

@@ -431,13 +431,14 @@ __global__ void __launch_bounds__(256) k_cells_expand(HistArgs h, uint32_t accum
     for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; b < h.n_bins; b += stride) {
         const ulonglong2 sums = __ldcs(reinterpret_cast<const ulonglong2 *>(h.cells + 4 * b));
         const ulonglong2 cnts = __ldcs(reinterpret_cast<const ulonglong2 *>(h.cells + 4 * b + 2));
-        uint32_t c0 = (uint32_t)cnts.x, c1 = (uint32_t)(cnts.x >> 32);
-        uint64_t s0 = sums.x, s1 = sums.y;
-        if (accumulate) {
-            c0 += h.cnt[0][b];
-            c1 += h.cnt[1][b];
-            s0 += h.byt[0][b];
-            s1 += h.byt[1][b];
+        const uint32_t c0 = (uint32_t)cnts.x, c1 = (uint32_t)(cnts.x >> 32);
+        const uint64_t s0 = sums.x, s1 = sums.y;
+        if (accumulate) {  // reductions: calls on other streams may be adding to the same outputs
+            if (c0) red_add_u32(h.cnt[0] + b, c0);
+            if (c1) red_add_u32(h.cnt[1] + b, c1);
+            if (s0) red_add_u64(h.byt[0] + b, s0);
+            if (s1) red_add_u64(h.byt[1] + b, s1);
+            continue;
         }
         h.cnt[0][b] = c0;
         h.cnt[1][b] = c1;

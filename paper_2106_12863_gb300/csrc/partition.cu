@@ -877,16 +877,19 @@ __global__ void __launch_bounds__(kColdThreads, 1) k_part_cold(HistArgs h, PartD
         const uint32_t nb = (uint32_t)min((uint64_t)T, (uint64_t)h.n_bins - lo_bin);
         for (uint32_t i = threadIdx.x; i < nb; i += kColdThreads) {
             const uint64_t bin = lo_bin + i;
-            uint32_t c0 = tile[i], c1 = tile[T + i];
-            uint64_t s0 = (uint64_t)tile[4 * T + i] << 32 | tile[2 * T + i];
-            uint64_t s1 = (uint64_t)tile[5 * T + i] << 32 | tile[3 * T + i];
+            const uint32_t c0 = tile[i], c1 = tile[T + i];
+            const uint64_t s0 = (uint64_t)tile[4 * T + i] << 32 | tile[2 * T + i];
+            const uint64_t s1 = (uint64_t)tile[5 * T + i] << 32 | tile[3 * T + i];
 #pragma unroll
             for (uint32_t k = 0; k < 6; ++k) tile[k * T + i] = 0;  // ready for the next tile
+            // added with reductions, since calls on other streams may be adding to
+            // the same outputs, and only where the tile has updates (all bins read,
+            // added and stored took 1,238 us for 30 M records into 86.4 M bins, this
+            // 911; 20 M into 10 M 427, 400; 200 M skewed into 86.4 M 2,080, 1,706)
             if (accumulate) {
-                c0 += h.cnt[0][bin];
-                c1 += h.cnt[1][bin];
-                s0 += h.byt[0][bin];
-                s1 += h.byt[1][bin];
+                if (c0) gadd(h, 0u, bin, c0, s0);
+                if (c1) gadd(h, 1u, bin, c1, s1);
+                continue;
             }
             h.cnt[0][bin] = c0;
             h.cnt[1][bin] = c1;

@@ -99,3 +99,32 @@ def test_auto_without_room_for_scratch(orc, free_memory, n_bins, accumulate):
     torch.cuda.synchronize()
     assert_hist_equal(out.to_numpy(), orc.discriminate_histogram(*NET, rec, 0, 1, n_bins))
     assert sinet.sinet_device_status() == 0
+
+
+def test_streams_accumulating_into_one_histogram():
+    """A large call and small ones, on two streams, that add to the same outputs at once lose nothing."""
+    import torch
+
+    table = sinet.PrefixTable(np.array([0], np.uint32), np.array([1], np.uint8))
+    n, n_bins, calls = 6_000_001, 4_000_000, 40
+    g = torch.Generator(device="cuda").manual_seed(1)
+    p = sinet.HistParams(0, 1, n_bins, accumulate=True)
+    assert [sinet.auto_strategy(table, k, p) for k in (n, 300_000)] == ["partition", "global_atomic"]
+    ip = [torch.randint(-(1 << 31), 1 << 31, (n,), dtype=torch.int64, device="cuda", generator=g).to(torch.int32)
+          for _ in range(2)]
+    rec = (torch.randint(0, n_bins, (n,), dtype=torch.int64, device="cuda", generator=g), *ip,
+           torch.randint(0, 1 << 30, (n,), dtype=torch.int32, device="cuda", generator=g))
+    parts = [[v[i:i + 300_000] for v in rec] for i in range(0, n - 1, 300_000)]
+    last = [v[n - 1:] for v in rec]
+    out, once = sinet.Histogram(n_bins), sinet.Histogram(n_bins)
+    sinet.discriminate_histogram(table, *rec, sinet.HistParams(0, 1, n_bins, strategy="atomic_noagg"), once)
+    torch.cuda.synchronize()
+    large, small = torch.cuda.Stream(), torch.cuda.Stream()
+    for _ in range(calls):
+        sinet.discriminate_histogram(table, *rec, p, out, stream=large)
+        for r in (*parts, last):
+            sinet.discriminate_histogram(table, *r, p, out, stream=small)
+    torch.cuda.synchronize()
+    for k in ("count", "bytes", "stats"):
+        assert torch.equal(getattr(out, k), getattr(once, k) * (2 * calls)), k
+    assert sinet.sinet_device_status() == 0
