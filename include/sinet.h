@@ -335,7 +335,8 @@ sinet_status sinet_discriminate_histogram_noalloc(const sinet_prefix_table *t, c
  *
  * Non-accumulating slices without a ready word that run on global reductions
  * and have enough records (one per six bins, per two where 16 bytes a bin
- * exceed 60 MB; 8 M in all such slices) add into packed cells instead of their
+ * exceed 60 MB; 8 M in all such slices, where an AUTO slice that the fixed
+ * rule puts on the tile does not count) add into packed cells instead of their
  * outputs: 16 bytes a bin, allocated at creation after everything else and held
  * for the batch's life. Two further kernels of the graph expand the cells into
  * the outputs and redo a slice one of whose cells overflowed, straight into its
@@ -374,16 +375,17 @@ typedef struct sinet_batch sinet_batch;
  * descriptors and capture the launch. Slices with strategy AUTO get one from
  * the autotuner: slices are grouped into classes (lookup form, whether the
  * histogram fits a shared-memory tile, log2 of n_bins and of n, unit bin
- * width, both-direction policy); with SINET_BATCH_AUTOTUNE, each class not
+ * width, both-direction policy, packed cells); with SINET_BATCH_AUTOTUNE, each class not
  * yet in the process-wide cache is tuned by timing every candidate strategy
  * on its largest slice (its first 8 M records at most, into scratch outputs:
  * the slice's own outputs are not touched). The candidates are the batch
  * kernel's schemes (warp combining, plain atomics, the whole-histogram tile
- * when it fits), each run as enough copies to keep every CTA busy, and the
+ * when it fits), each run as enough copies to keep every CTA busy (with packed
+ * cells where the batch would run them), and the
  * plain path (sort + reduce by key), run as its own chain; the fastest per record is cached and, if the environment
  * variable SINET_AUTOTUNE_CACHE names a file, appended to it as a line
  * "class strategy ns_per_record" (the file is read on first use). Without the flag a class absent from the
- * cache takes a fixed rule. Tuning runs on `stream` and synchronises it.
+ * cache takes its choice without packed cells if that is there, else a fixed rule. Tuning runs on `stream` and synchronises it.
  * The records, tables and outputs are referenced, not copied: they must
  * stay valid, and the records unchanged between runs only if the caller
  * wants the same result. Returns SINET_ERR_INVALID_ARG for a NULL slice

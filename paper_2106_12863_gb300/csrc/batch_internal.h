@@ -28,6 +28,7 @@ struct PlannedSlice {
     uint32_t lk = 0;          // lookup form off the tile ...
     uint32_t lk_tile = 0;     // ... and on it: the table's smaller form where the tile fits beside that only
     bool tile_fits = false;   // the whole histogram fits a tile next to the table
+    bool pack = false;        // its global reductions go to packed cells (plan_cells)
     uint32_t user_index = 0;  // position in the caller's slice array
 };
 
@@ -48,8 +49,10 @@ sinet_status plan_slice(const sinet_batch_slice &u, const DeviceState *ds, uint3
 // candidates (tune), or by the fixed rule.
 sinet_status resolve_strategies(std::vector<PlannedSlice> &v, bool tune, const DeviceState *ds,
                                 uint32_t smem, cudaStream_t s);
-// Whether a slice's reductions go to packed cells (HistArgs::packed), and the
-// bytes of its cells and their totals.
+// Decide for the slices of a batch, before their strategies are resolved, whose
+// global reductions go to packed cells (HistArgs::packed).
+void plan_cells(std::vector<PlannedSlice> &v);
+// Whether a slice with a strategy runs on them, and the bytes of its cells and their totals.
 bool slice_packed(const PlannedSlice &ps);
 size_t packed_bytes(uint32_t n_bins);
 // Map a public strategy to the batch kernel's update scheme.
@@ -90,7 +93,7 @@ struct BatchEngine {
     sinet_status init(uint32_t capacity, const DeviceState *ds, uint32_t smem_bytes);
     // host image (header, starts, descriptors) of `v` in descriptor order
     void image(const std::vector<PlannedSlice> &v, std::vector<uint8_t> &buf) const;
-    // packed cells for the slices of v that gain by them (before image and capture)
+    // packed cells for the slices of v that run on them (before image and capture)
     void plan_packed(std::vector<PlannedSlice> &v);
     // without them after all
     void drop_packed(std::vector<PlannedSlice> &v);

@@ -43,14 +43,19 @@ bool sort_feasible(const PlannedSlice &ps) {
 // and reads 16 bytes a bin more, from one per two bins on. Not with a ready word:
 // what it leaves out after a wait that ran out, a redo would add. 256 slices of 1.06 B
 // records: 11.96 -> 9.37 ms.
-bool slice_packed(const PlannedSlice &ps) {
+static bool cells_pay(const PlannedSlice &ps) {
     const uint64_t n = ps.d.r.g.n, bins = ps.d.h.n_bins;
-    return ps.d.zero && !ps.d.ready &&
-           (ps.strategy == SINET_STRAT_GLOBAL_ATOMIC || ps.strategy == SINET_STRAT_ATOMIC_NOAGG) &&
-           packed_countable(n, ps.d.h.two_dir != 0) && n >= bins / (16 * bins <= (60ull << 20) ? 6 : 2);
+    return ps.d.zero && !ps.d.ready && packed_countable(n, ps.d.h.two_dir != 0) &&
+           n >= bins / (16 * bins <= (60ull << 20) ? 6 : 2);
 }
 
 constexpr uint64_t kMinPackedBatch = 8000000;
+
+static bool on_reductions(int32_t strategy) {
+    return strategy == SINET_STRAT_GLOBAL_ATOMIC || strategy == SINET_STRAT_ATOMIC_NOAGG;
+}
+
+bool slice_packed(const PlannedSlice &ps) { return ps.pack && on_reductions(ps.strategy); }
 
 size_t packed_bytes(uint32_t n_bins) { return 64 + 16 * (size_t)n_bins; }
 
@@ -185,21 +190,10 @@ void BatchEngine::image(const std::vector<PlannedSlice> &v, std::vector<uint8_t>
 }
 
 void BatchEngine::plan_packed(std::vector<PlannedSlice> &v) {
-    // the expansion stores every bin, so not where outputs share memory
-    std::vector<OutputRange> ranges;
-    std::vector<bool> shared(v.size());
-    for (size_t i = 0; i < v.size(); ++i) output_ranges(v[i].d.h, (uint32_t)i, ranges);
-    mark_overlaps(ranges, shared);
     size_t total = 0;
-    uint64_t records = 0;
-    for (size_t i = 0; i < v.size(); ++i)
-        if (slice_packed(v[i]) && !shared[i]) {
-            total += packed_bytes(v[i].d.h.n_bins);
-            records += v[i].d.r.g.n;
-        }
-    // the expansion's and the redo's kernels cost what the reductions of some
-    // 8 M records save (55 slices of 10 K to 168 K records: 582 us, without 508)
-    if (records < kMinPackedBatch) return;
+    for (const PlannedSlice &ps : v)
+        if (slice_packed(ps)) total += packed_bytes(ps.d.h.n_bins);
+    if (!total) return;
     if (cudaMalloc(&cells, total) != cudaSuccess) {  // no room: straight into the outputs
         cudaGetLastError();
         cells = nullptr;
@@ -207,12 +201,11 @@ void BatchEngine::plan_packed(std::vector<PlannedSlice> &v) {
     }
     packed = true;
     uint8_t *m = static_cast<uint8_t *>(cells);
-    for (size_t i = 0; i < v.size(); ++i) {
-        HistArgs &h = v[i].d.h;
-        if (!slice_packed(v[i]) || shared[i]) continue;
-        h.pack_sums = reinterpret_cast<uint64_t *>(m);
-        h.packed = h.pack_sums + 8;
-        m += packed_bytes(h.n_bins);
+    for (PlannedSlice &ps : v) {
+        if (!slice_packed(ps)) continue;
+        ps.d.h.pack_sums = reinterpret_cast<uint64_t *>(m);
+        ps.d.h.packed = ps.d.h.pack_sums + 8;
+        m += packed_bytes(ps.d.h.n_bins);
     }
 }
 
@@ -337,7 +330,7 @@ std::string class_key(const PlannedSlice &ps, const DeviceState *ds) {
     std::snprintf(b, sizeof b, "sm%d/lk%u/tile%d/bins2^%u/n2^%u/w1%u/two%u", ds->sm_count, ps.d.lk,
                   ps.tile_fits ? 1 : 0, ceil_log2(ps.d.h.n_bins), floor_log2(ps.d.r.g.n + 1),
                   ps.d.h.w_is_one, ps.d.h.two_dir);
-    return b;
+    return ps.pack ? std::string(b) + "/packed" : b;
 }
 
 void load_cache_file() {
@@ -374,7 +367,8 @@ int32_t fixed_rule(const PlannedSlice &ps) {
     return SINET_STRAT_ATOMIC_NOAGG;
 }
 
-// Time the candidates on one representative slice; returns the fastest per
+// Time the candidates on one representative slice, with packed cells where the
+// batch runs them (plan_cells decided from the whole slice); returns the fastest per
 // record. A batch keeps every CTA busy, so each candidate runs on enough
 // copies of the slice (its first kTuneRecords records) to give the grid two
 // work items per CTA: timed alone, a slice cut into few large items would
@@ -387,8 +381,6 @@ sinet_status tune_one(const PlannedSlice &rep, const DeviceState *ds, uint32_t s
     ps.d.r.g = make_geom(n, {{ps.d.r.ts, 8}, {ps.d.r.src, 4}, {ps.d.r.dst, 4}, {ps.d.r.bytes, 4}});
     const uint32_t nb = ps.d.h.n_bins;
     const size_t hist_bytes = (((size_t)8 * nb + 15) & ~(size_t)15) + (size_t)16 * nb + 64;
-    // with room for the cells of a candidate that packs them
-    const size_t out_bytes = hist_bytes + packed_bytes(nb);
     ps.d.zero = 1;
     ps.zero_items = (nb + kZeroBins - 1) / kZeroBins;
     int32_t cands[3] = {SINET_STRAT_GLOBAL_ATOMIC, SINET_STRAT_ATOMIC_NOAGG, SINET_STRAT_SMEM_FULL};
@@ -402,13 +394,21 @@ sinet_status tune_one(const PlannedSlice &rep, const DeviceState *ds, uint32_t s
     sinet_status st = SINET_OK;
     for (int c = 0; c < nc && st == SINET_OK; ++c) {
         set_strategy(ps, cands[c], (uint32_t)eng.grid);
-        const bool packed = rep.d.zero && slice_packed(ps);
+        bool packed = slice_packed(ps);
+        size_t out_bytes = hist_bytes + (packed ? packed_bytes(nb) : 0);
         uint32_t copies = ps.items ? (uint32_t)((2ull * eng.grid + ps.items - 1) / ps.items) : 1u;
         copies = std::max<uint32_t>(1, std::min<uint32_t>({copies, eng.cap,
                                                            (uint32_t)std::max<uint64_t>(1, (4 * kTuneRecords) / std::max<uint64_t>(n, 1))}));
-        const bool separate = (size_t)copies * out_bytes <= (512ull << 20);
+        bool separate = (size_t)copies * out_bytes <= (512ull << 20);
         void *scratch = nullptr;
         cudaError_t e = cudaMalloc(&scratch, separate ? copies * out_bytes : out_bytes);
+        if (e == cudaErrorMemoryAllocation && packed) {  // as a batch runs that cannot have its cells
+            cudaGetLastError();
+            packed = false;
+            out_bytes = hist_bytes;
+            separate = (size_t)copies * out_bytes <= (512ull << 20);
+            e = cudaMalloc(&scratch, separate ? copies * out_bytes : out_bytes);
+        }
         std::vector<PlannedSlice> v(copies, ps);
         for (uint32_t k = 0; k < copies && e == cudaSuccess; ++k) {
             uint8_t *m = static_cast<uint8_t *>(scratch) + (separate ? k * out_bytes : 0);
@@ -463,7 +463,7 @@ sinet_status tune_one(const PlannedSlice &rep, const DeviceState *ds, uint32_t s
         const SortPlan plan = plan_sort_reduce(n, nb, ps.d.h.two_dir != 0);
         void *scratch = nullptr, *outs = nullptr;
         cudaError_t e = cudaMalloc(&scratch, std::max<size_t>(plan.scratch_bytes, 256));
-        if (e == cudaSuccess) e = cudaMalloc(&outs, out_bytes);
+        if (e == cudaSuccess) e = cudaMalloc(&outs, hist_bytes);
         HistArgs h = ps.d.h;
         if (e == cudaSuccess) {
             uint8_t *m = static_cast<uint8_t *>(outs);
@@ -480,7 +480,7 @@ sinet_status tune_one(const PlannedSlice &rep, const DeviceState *ds, uint32_t s
         float ms = 1e30f;
         for (int rep_i = 0; rep_i < 4 && e == cudaSuccess; ++rep_i) {
             e = cudaEventRecord(e0, s);
-            if (e == cudaSuccess) e = cudaMemsetAsync(outs, 0, out_bytes, s);
+            if (e == cudaSuccess) e = cudaMemsetAsync(outs, 0, hist_bytes, s);
             if (e == cudaSuccess) e = run_sort_reduce((int)ps.d.lk, ps.d.r, ps.d.t, h, plan, scratch, true, lc);
             if (e == cudaSuccess) e = cudaEventRecord(e1, s);
             if (e == cudaSuccess) e = cudaEventSynchronize(e1);
@@ -506,6 +506,27 @@ sinet_status tune_one(const PlannedSlice &rep, const DeviceState *ds, uint32_t s
 }
 
 }  // namespace
+
+void plan_cells(std::vector<PlannedSlice> &v) {
+    // the expansion stores every bin, so not where outputs share memory
+    std::vector<OutputRange> ranges;
+    std::vector<bool> shared(v.size());
+    for (size_t i = 0; i < v.size(); ++i) output_ranges(v[i].d.h, (uint32_t)i, ranges);
+    mark_overlaps(ranges, shared);
+    // Decided before the strategies, so that the tuner times what runs: slices
+    // that are to be resolved count here unless the rule for them is the tile.
+    uint64_t records = 0;
+    for (size_t i = 0; i < v.size(); ++i) {
+        PlannedSlice &ps = v[i];
+        const bool open = ps.strategy == SINET_STRAT_AUTO;
+        ps.pack = cells_pay(ps) && !shared[i] && (open || on_reductions(ps.strategy));
+        if (ps.pack && (!open || fixed_rule(ps) != SINET_STRAT_SMEM_FULL)) records += ps.d.r.g.n;
+    }
+    // the expansion's and the redo's kernels cost what the reductions of some
+    // 8 M records save (55 slices of 10 K to 168 K records: 582 us, without 508)
+    if (records < kMinPackedBatch)
+        for (PlannedSlice &ps : v) ps.pack = false;
+}
 
 sinet_status resolve_strategies(std::vector<PlannedSlice> &v, bool tune, const DeviceState *ds,
                                 uint32_t smem, cudaStream_t s) {
@@ -544,6 +565,8 @@ sinet_status resolve_strategies(std::vector<PlannedSlice> &v, bool tune, const D
     for (size_t i = 0; i < v.size(); ++i) {
         if (v[i].strategy != SINET_STRAT_AUTO) continue;
         auto it = g_tune.find(keys[i]);
+        if (it == g_tune.end() && v[i].pack)  // a class's choice without cells is better than none
+            it = g_tune.find(keys[i].substr(0, keys[i].rfind('/')));
         int32_t s_ = it != g_tune.end() ? it->second : fixed_rule(v[i]);
         if (s_ == SINET_STRAT_SMEM_FULL && !v[i].tile_fits) s_ = fixed_rule(v[i]);
         if (s_ == SINET_STRAT_SORT_REDUCE && !sort_feasible(v[i])) s_ = fixed_rule(v[i]);
@@ -586,6 +609,7 @@ sinet_status sinet_batch_create(const sinet_batch_slice *slices, uint32_t n_slic
         v[i].user_index = i;
         records += slices[i].n;
     }
+    plan_cells(v);
     if ((st = resolve_strategies(v, (flags & SINET_BATCH_AUTOTUNE) != 0, ds, smem, stream)) != SINET_OK)
         return st;
     uint64_t items = 0, zitems = 0;

@@ -72,9 +72,39 @@ int plan_packed_slice(uint64_t n, uint32_t n_bins, int two_dir) {
     ps.d.r.g = make_geom(n, {});
     ps.d.h.n_bins = n_bins;
     ps.d.h.two_dir = two_dir != 0;
+    for (int d = 0; d < 2; ++d) {
+        ps.d.h.cnt[d] = reinterpret_cast<uint32_t *>((uint64_t)(1 + d) << 40);
+        ps.d.h.byt[d] = reinterpret_cast<uint64_t *>((uint64_t)(3 + d) << 40);
+    }
     ps.d.zero = 1;
     ps.strategy = SINET_STRAT_ATOMIC_NOAGG;
-    return slice_packed(ps);
+    std::vector<PlannedSlice> v(1, ps);
+    plan_cells(v);
+    return slice_packed(v[0]);
+}
+
+// plan_cells for a batch of n_slices slices: records, bins, strategy, accumulate,
+// ready word and "same outputs as slice 0" of each; pack[i] is its decision.
+void plan_batch_cells(const uint64_t *n, const uint32_t *bins, const int32_t *strategy, const uint8_t *accumulate,
+                      const uint8_t *ready, const uint8_t *as_first, uint32_t n_slices, uint8_t *pack) {
+    std::vector<PlannedSlice> v(n_slices);
+    for (uint32_t i = 0; i < n_slices; ++i) {
+        PlannedSlice &ps = v[i];
+        ps.d = BatchSlice{};
+        ps.d.r.g = make_geom(n[i], {});
+        const uintptr_t at = as_first[i] ? 1 : 1 + (uintptr_t)i;
+        for (int d = 0; d < 2; ++d) {
+            ps.d.h.cnt[d] = reinterpret_cast<uint32_t *>((2 * at + d) << 40);
+            ps.d.h.byt[d] = reinterpret_cast<uint64_t *>(((2 * at + d) << 40) + (1ull << 39));
+        }
+        ps.d.h.n_bins = bins[i];
+        ps.d.zero = !accumulate[i];
+        ps.d.ready = ready[i] ? reinterpret_cast<const uint32_t *>(uintptr_t(64)) : nullptr;
+        ps.tile_fits = bins[i] <= 4000;
+        ps.strategy = strategy[i];
+    }
+    plan_cells(v);
+    for (uint32_t i = 0; i < n_slices; ++i) pack[i] = v[i].pack;
 }
 
 // Which of n histograms' outputs (count[0], count[1], bytes[0], bytes[1] and

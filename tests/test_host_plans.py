@@ -89,3 +89,30 @@ def test_outputs_that_share_memory(plans, seed):
         mine = [r for r in rows if r[0] == i]
         assert shared[i] == any(meets(a, b) for a in mine for b in rows)
         assert own[i] == any(meets(a, b) for a in mine for b in mine)
+
+
+AUTO, NOAGG, SORT_REDUCE = 0, 5, 3
+M = 1_000_000
+
+
+@pytest.mark.parametrize("slices,want", [
+    # (records, bins, strategy, accumulate, ready, as_first) of every slice; 8 M records are the line
+    ([(20 * M, 21_600_000, AUTO, 0, 0, 0)], [1]),
+    ([(7_999_999, M, AUTO, 0, 0, 0)], [0]),
+    ([(7_999_999, M, NOAGG, 0, 0, 0), (1000, 6000, GLOBAL_ATOMIC, 0, 0, 0)], [1, 1]),
+    # a slice that the rule puts on the tile does not count, but has cells if the tuner takes it off the tile
+    ([(20 * M, 4000, AUTO, 0, 0, 0), (7_999_999, M, AUTO, 0, 0, 0)], [0, 0]),
+    ([(20 * M, 4000, AUTO, 0, 0, 0), (8 * M, M, AUTO, 0, 0, 0)], [1, 1]),
+    # too few records a bin; added to; waited for; outputs that another slice has too; other strategies
+    ([(9 * M, M, NOAGG, 0, 0, 0), (16_666, 100_000, NOAGG, 0, 0, 0), (16_665, 100_000, NOAGG, 0, 0, 0)], [1, 1, 0]),
+    ([(9 * M, 3_932_160, NOAGG, 0, 0, 0), (5 * M, 10 * M, NOAGG, 0, 0, 0), (5 * M - 1, 10 * M, NOAGG, 0, 0, 0)], [1, 1, 0]),
+    ([(9 * M, M, NOAGG, 0, 0, 0), (9 * M, M, NOAGG, 1, 0, 0), (9 * M, M, NOAGG, 0, 1, 0)], [1, 0, 0]),
+    ([(9 * M, M, NOAGG, 0, 0, 0), (9 * M, M, NOAGG, 0, 0, 1), (9 * M, M, NOAGG, 0, 0, 0)], [0, 0, 1]),
+    ([(9 * M, M, SORT_REDUCE, 0, 0, 0), (9 * M, 4000, SMEM_FULL, 0, 0, 0), (7 * M, M, NOAGG, 0, 0, 0)], [0, 0, 0]),
+])
+def test_cells_are_decided_before_the_strategies(plans, slices, want):
+    cols = [np.array(c, t) for c, t in zip(zip(*slices), (np.uint64, np.uint32, np.int32, np.uint8, np.uint8, np.uint8))]
+    pack = np.zeros(len(slices), np.uint8)
+    plans.plan_batch_cells(*(ctypes.c_void_p(c.ctypes.data) for c in cols), ctypes.c_uint32(len(slices)),
+                           ctypes.c_void_p(pack.ctypes.data))
+    assert pack.tolist() == want
