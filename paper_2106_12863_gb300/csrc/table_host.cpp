@@ -26,18 +26,24 @@ static uint32_t iv_image_bytes(uint32_t n_iv, uint32_t k) {
     return pad16(4 * n_iv) * 2 + pad16(2 * ((1u << k) + 1));
 }
 
+// Where membership flips: the addresses in (0, 2^32) at which an interval
+// starts or has just ended, ascending.
+static std::vector<uint32_t> toggles(const TableHost &t) {
+    std::vector<uint32_t> tog;
+    tog.reserve(2 * t.lo.size());
+    for (size_t i = 0; i < t.lo.size(); i++) {
+        if (t.lo[i]) tog.push_back(t.lo[i]);
+        if (t.hi[i] != 0xFFFFFFFFu) tog.push_back(t.hi[i] + 1);
+    }
+    return tog;
+}
+
 // Fills the leaf form (table_host.h) if it fits `budget` bytes: two words a
 // leaf where that fits, else four; within a width, the bucket bits that take
 // the least room. The budget is never below the toggle form's size plus one
 // block, so a one-block toggle table always has a four-word leaf form (its
 // buckets need no cut, and the second pure leaf is the extra block).
-static void build_leaves(TableHost &t, size_t budget) {
-    // toggles in (0, 2^32): where membership flips
-    std::vector<uint32_t> tog;
-    for (size_t i = 0; i < t.lo.size(); i++) {
-        if (t.lo[i]) tog.push_back(t.lo[i]);
-        if (t.hi[i] != 0xFFFFFFFFu) tog.push_back(t.hi[i] + 1);
-    }
+static void build_leaves(TableHost &t, const std::vector<uint32_t> &tog, size_t budget) {
     const bool first_in = !t.lo.empty() && t.lo[0] == 0;
     const size_t n = tog.size();
     t.leaf_words = 0;
@@ -54,29 +60,42 @@ static void build_leaves(TableHost &t, size_t budget) {
         }
         uint32_t best_bits = 0;
         size_t best = budget + 1;
-        std::vector<uint8_t> size_log2, best_log2;  // per bucket: leaf size, or 0xFF when pure
-        for (uint32_t kb = 6; kb <= 14; kb++) {
-            const uint32_t sh = 32 - kb, m = (1u << sh) - 1;
-            size_log2.assign(1u << kb, 0xFF);
-            for (uint32_t v : tog)
-                if (v & m) size_log2[v >> sh] = (uint8_t)sh;
-            for (size_t i = 0; i < cut.size(); i++)
-                if (cut[i] < sh) {
-                    uint8_t &s = size_log2[tog[i + words] >> sh];
-                    s = std::min(s, cut[i]);
+        // one walk over the toggles per bucket count: done(bucket, log2 of its
+        // leaves' size) for every bucket that is not pure, until it says false. A
+        // bucket that holds a toggle off its first address is one leaf, or as many
+        // as its smallest cut asks for
+        auto walk = [&](uint32_t sh, auto &&done) {
+            const uint32_t m = (1u << sh) - 1;
+            for (size_t i = 0; i < n;) {
+                const uint32_t b = tog[i] >> sh;
+                uint32_t s = 0xFF;
+                for (; i < n && tog[i] >> sh == b; i++) {
+                    if (tog[i] & m) s = std::min(s, sh);
+                    if (i >= words && cut[i - words] < sh) s = std::min<uint32_t>(s, cut[i - words]);
                 }
+                if (s != 0xFF && !done(b, s)) return;
+            }
+        };
+        for (uint32_t kb = 6; kb <= 14; kb++) {
+            const uint32_t sh = 32 - kb;
             size_t leaves = 2;
-            for (uint8_t s : size_log2)
-                if (s != 0xFF) leaves += (size_t)1 << (sh - s);
+            walk(sh, [&](uint32_t, uint32_t s) {
+                leaves += (size_t)1 << (sh - s);
+                return 4 * words * leaves < best;
+            });
             const size_t bytes = ((4 * words * leaves + 15) & ~(size_t)15) + (4ull << kb);
             if (bytes < best) {
                 best = bytes;
                 best_bits = kb;
-                best_log2 = size_log2;
             }
         }
         if (!best_bits) continue;
         const uint32_t sh = 32 - best_bits;
+        std::vector<uint8_t> best_log2(1u << best_bits, 0xFF);  // per bucket: leaf size, or 0xFF when pure
+        walk(sh, [&](uint32_t b, uint32_t s) {
+            best_log2[b] = (uint8_t)s;
+            return true;
+        });
         t.leaf_bits = best_bits;
         t.leaf_words = words;
         t.leaf_desc.assign(1u << best_bits, 0);
@@ -193,61 +212,57 @@ int compile_table(const uint32_t *net, const uint8_t *len, uint32_t n, uint32_t 
     t.index_bits = k;
     t.max_range = build_index(k);
 
-    // toggle form `form` (1, 2 or 0, see table_host.h) at kb bucket bits;
-    // returns (most blocks one bucket needs, image bytes), or ~0 when the form
-    // cannot hold this table
-    auto build_toggles = [&](uint32_t kb, uint32_t form, bool keep) {
-        const uint32_t nb = 1u << kb;
-        const auto fail = std::pair<uint32_t, size_t>(~0u, ~size_t(0));
-        std::vector<uint32_t> desc(nb, 0), blocks(4, 0x7FFFFFFFu);
-        uint32_t maxb = 1, j = 0;
-        std::vector<uint32_t> tog;
+    // toggle form `form` (1, 2 or 0, see table_host.h) at kb bucket bits: its
+    // image bytes, or ~0 when the form cannot hold this table
+    const std::vector<uint32_t> tog = toggles(t);
+    auto toggle_size = [&](uint32_t kb, uint32_t form) {
+        const uint32_t sh = 32 - kb, m = (1u << sh) - 1;
+        const uint32_t most = form ? form : 15, last = form == 1 ? 0x7FFFu : form == 2 ? 0x7FFEu : 0xFFFFFFu;
+        size_t blocks = 1;
+        for (size_t i = 0; i < tog.size();) {
+            const uint32_t b = tog[i] >> sh;
+            uint32_t inside = 0;
+            for (; i < tog.size() && tog[i] >> sh == b; i++) inside += (tog[i] & m) != 0;
+            const uint32_t need = (inside + 3) / 4;
+            if (need > most || (need && blocks > last)) return ~size_t(0);
+            blocks += need;
+        }
+        return 16 * blocks + ((size_t)4 << kb);
+    };
+    auto build_toggles = [&](uint32_t kb, uint32_t form) {
+        const uint32_t nb = 1u << kb, sh = 32 - kb, m = (1u << sh) - 1;
+        t.desc.assign(nb, 0);
+        t.blocks.assign(4, 0x7FFFFFFFu);
+        t.max_blocks = 1;
+        size_t j = 0;
+        bool in = n_iv && t.lo[0] == 0;  // membership just below toggle j
         for (uint32_t b = 0; b < nb; b++) {
-            const uint64_t start = (uint64_t)b << (32 - kb);
-            const uint64_t end = start + (1ull << (32 - kb)) - 1;
-            while (j < n_iv && (uint64_t)t.hi[j] < start) j++;  // first with hi >= start
-            const uint32_t s0 = (j < n_iv && (uint64_t)t.lo[j] <= start) ? 1u : 0u;
-            tog.clear();
-            for (uint32_t e = j; e < n_iv && (uint64_t)t.lo[e] <= end; e++) {
-                if ((uint64_t)t.lo[e] > start) tog.push_back((uint32_t)((uint64_t)t.lo[e] - start));
-                if ((uint64_t)t.hi[e] < end) tog.push_back((uint32_t)((uint64_t)t.hi[e] + 1 - start));
+            if (j < tog.size() && tog[j] == b << sh) {  // flips on the bucket's first address
+                in = !in;
+                j++;
             }
-            const uint32_t need = (uint32_t)(tog.size() + 3) / 4;
-            maxb = std::max(maxb, need ? need : 1u);
-            uint32_t first = 0;
-            if (need) {
-                first = (uint32_t)blocks.size() / 4;
-                for (uint32_t i = 0; i < need * 4; i++) blocks.push_back(i < tog.size() ? tog[i] - 1 : 0x7FFFFFFFu);
+            const uint32_t s0 = in;
+            const uint32_t first = (uint32_t)t.blocks.size() / 4;
+            for (; j < tog.size() && tog[j] >> sh == b; j++) {
+                t.blocks.push_back((tog[j] & m) - 1);
+                in = !in;
             }
-            if (form == 1) {
-                if (need > 1 || first > 0x7FFFu) return fail;
-                desc[b] = first | (s0 << 31);
-            } else if (form == 2) {
-                if (need > 2 || first + 1 > 0x7FFFu) return fail;
-                desc[b] = first | ((need == 2 ? first + 1 : 0u) << 15) | (s0 << 31);
-            } else {
-                const uint32_t nblk = need ? need : 1u;
-                if (nblk > 15 || first > 0xFFFFFFu) return fail;
-                desc[b] = first | (nblk << 24) | (s0 << 31);
-            }
+            while (t.blocks.size() % 4) t.blocks.push_back(0x7FFFFFFFu);
+            const uint32_t need = (uint32_t)t.blocks.size() / 4 - first, at = need ? first : 0;
+            t.max_blocks = std::max(t.max_blocks, need);
+            if (form == 1) t.desc[b] = at | (s0 << 31);
+            else if (form == 2) t.desc[b] = at | ((need == 2 ? at + 1 : 0u) << 15) | (s0 << 31);
+            else t.desc[b] = at | (std::max(need, 1u) << 24) | (s0 << 31);
         }
-        const size_t bytes = 4 * blocks.size() + 4 * (size_t)nb;
-        if (keep) {
-            t.desc.swap(desc);
-            t.blocks.swap(blocks);
-            t.desc_bits = kb;
-            t.max_blocks = maxb;
-            t.toggle_form = form;
-        }
-        return std::pair<uint32_t, size_t>(maxb, bytes);
+        t.desc_bits = kb;
+        t.toggle_form = form;
     };
     // one block per bucket if some bit count allows it, else two, else as
     // many as needed; within a form, the fewest bits that fit the budget
     uint32_t kb = 0, form = 0;
     for (uint32_t f : {1u, 2u}) {
         for (uint32_t c = 8; c <= 14 && !kb; c++) {
-            auto r = build_toggles(c, f, false);
-            if (r.first != ~0u && r.second <= kSmemTableBudget) {
+            if (toggle_size(c, f) <= kSmemTableBudget) {
                 kb = c;
                 form = f;
             }
@@ -257,18 +272,17 @@ int compile_table(const uint32_t *net, const uint8_t *len, uint32_t n, uint32_t 
     if (!kb) {
         size_t best = ~size_t(0);
         for (uint32_t c = 8; c <= 14; c++) {
-            auto r = build_toggles(c, 0, false);
-            if (r.first != ~0u && r.second < best) {
-                best = r.second;
+            const size_t size = toggle_size(c, 0);
+            if (size < best) {
+                best = size;
                 kb = c;
             }
         }
-        if (!kb) kb = 14;
         form = 0;
     }
-    build_toggles(kb, form, true);
+    if (kb) build_toggles(kb, form);  // (else global lookups)
     const size_t toggle_bytes = pad16(4 * (uint32_t)t.blocks.size()) + pad16(4 * (uint32_t)t.desc.size());
-    if (t.max_blocks <= 15 && toggle_bytes <= kSmemTableBudget) build_leaves(t, std::max<size_t>(kLeafBudget, toggle_bytes + 16));
+    if (t.max_blocks <= 15 && toggle_bytes <= kSmemTableBudget) build_leaves(t, tog, std::max<size_t>(kLeafBudget, toggle_bytes + 16));
     return SINET_OK;
 }
 
