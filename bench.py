@@ -211,6 +211,20 @@ def kernel_source_hash(kernel: str | None = None):
     return h.hexdigest()[:16]
 
 
+def kernels_per_step(strategy: str, n: int, n_bins: int) -> int:
+    """The library's kernels in one call (zeroing is cudaMemsetAsync): one fused kernel; with it the
+    expansion of the 32-byte cells, or the expansion and the redo of packed ones where warp combining
+    takes them (16 bytes a bin within 60 MB, 1 M records, a record per six bins); run boundaries, their
+    scan and the remainder for the owner strategy; sample, levels, candidates, hot table, main pass,
+    tiles and finish for the partition, and the split where the histogram has more than 384 ranges of
+    2^15 bins."""
+    if strategy == "global_atomic":
+        return 3 if n >= 1_000_000 and n >= n_bins // 6 and 16 * n_bins <= 60 << 20 else 1
+    if strategy == "partition":
+        return 8 if -(-n_bins >> 15) > 384 else 7
+    return {"atomic_cell": 2, "owner": 4}.get(strategy, 1)
+
+
 def recorded_traffic(kernel: str, workload: str):
     """Per-launch DRAM bytes from the committed ncu summary, if it was taken
     on the current kernel sources (else None)."""
@@ -1027,12 +1041,7 @@ def run_window_bench(args, w, rank, world, dev, extras: bool):
                           "call_frac": alg_bytes / (kern_ms / 1e3) / 1e9 / peak,
                           "timed": "whole step (CUDA events on the launching stream): "
                                    + ("the library call" if own else "output zeroing + the library call")}
-    # kernels per step: one fused kernel (zeroing is cudaMemsetAsync), plus
-    # the cell expansion for the cell strategy; the run boundaries, their scan
-    # and the remainder for the owner strategy; sample, levels, total,
-    # candidates, hot table, main pass, three page-grouping kernels, cold pass
-    # and hot totals for the partition
-    result["gpu_launches"] = args.steps * {"atomic_cell": 2, "owner": 4, "partition": 8}.get(strategy, 1)
+    result["gpu_launches"] = args.steps * kernels_per_step(strategy, n, w.n_bins)
     result["config"] = {"workload": w.name, "records": n, "prefixes": w.table.n,
                         "n_bins": w.n_bins, "bin_width_ms": w.bin_width, "strategy": strategy,
                         "tune_ms": tune, "l2": f"inputs larger than L2 ({RECORD_BYTES * n / 1e9:.1f} GB of records)",
