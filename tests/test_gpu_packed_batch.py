@@ -149,3 +149,53 @@ def test_both_directions_in_one_row(strategy, n, n_bins):
     sinet.discriminate_histogram(table, *rec, sinet.HistParams(0, 1, n_bins, strategy=strategy), one)
     assert torch.equal(count, two.count.sum(0, dtype=torch.int32))
     assert torch.equal(nbytes, two.bytes.sum(0))
+
+
+def test_packed_slices_beside_others(orc):
+    """Both-direction policies, unaligned streams, records outside the window, several cells that
+    overflow, widths, and tile, accumulating and plain-path neighbours in one batch; replayed."""
+    from helpers import assert_hist_equal, to_dev
+
+    net, ln = np.array([10 << 24], np.uint32), np.array([8], np.uint8)
+    table = sinet.PrefixTable(net, ln)
+    kinds = [  # records, bins, width, strategy, policy, overflowing cells, accumulate
+        (2_500_003, 300_001, 1, "atomic_noagg", sinet.INCLUSIVE, 3, False),
+        (2_000_001, 70_000, 10, "global_atomic", sinet.INCLUSIVE, 1, False),
+        (1_500_002, 140_003, 7, "atomic_noagg", sinet.PAPER_ALG1, 2, False),
+        (2_100_000, 1_000_000, 1, "global_atomic", sinet.EXCLUSIVE, 0, False),
+        (60_000, 10_001, 1, "atomic_noagg", sinet.EXCLUSIVE, 1, False),
+        (100_001, 3_000, 1, "smem_full", sinet.INCLUSIVE, 1, False),
+        (100_002, 90_000, 1, "atomic_noagg", sinet.EXCLUSIVE, 1, True),
+        (100_003, 80_000, 1, "sort_reduce", sinet.INCLUSIVE, 1, False),
+    ]
+    slices, want = [], []
+    for i, (n, n_bins, width, strategy, policy, hot, accumulate) in enumerate(kinds):
+        rng = np.random.default_rng(i)
+        cls = rng.choice(4, n, p=[0.1, 0.4, 0.4, 0.1])
+        host = lambda inside: np.where(inside, 0x0A000000 | rng.integers(0, 1 << 24, n), rng.integers(1 << 31, 1 << 32, n))
+        span = n_bins * width
+        rec = {"ts": 1000 + rng.integers(-span // 20, span + span // 20, n).clip(-1000), "src": host(cls & 1),
+               "dst": host(cls & 2), "bytes": rng.integers(0, 1 << 30, n)}
+        for k in range(hot):
+            at = slice(700 * k, 700 * (k + 1))
+            rec["ts"][at], rec["bytes"][at] = 1000 + (span // 3) * k, 0xFFFFFFFF
+        rec = {k: v.astype(np.uint64 if k == "ts" else np.uint32) for k, v in rec.items()}
+        d = to_dev(rec, offsets={k: (i + j) % 4 for j, k in enumerate(rec)})
+        out = sinet.Histogram(n_bins)
+        slices.append((table, d["ts"], d["src"], d["dst"], d["bytes"],
+                       sinet.HistParams(1000, width, n_bins, policy=policy, strategy=strategy, accumulate=accumulate), out))
+        want.append(orc.discriminate_histogram(net, ln, rec, 1000, width, n_bins, policy=policy))
+    batch = sinet.Batch(slices)
+    for run in range(1, 4):
+        for s, kind in zip(slices, kinds):
+            if not kind[-1]:
+                s[-1].count.fill_(-1)
+                s[-1].bytes.fill_(-1)
+        batch.run()
+        torch.cuda.synchronize()
+        for i, (s, ref, kind) in enumerate(zip(slices, want, kinds)):
+            if kind[-1]:
+                ref = {k: v * np.array(run, v.dtype) for k, v in ref.items()}
+            assert_hist_equal(s[-1].to_numpy(), ref, f"slice {i}, run {run}")
+    assert sinet.sinet_device_status() == 0
+    batch.close()
