@@ -214,12 +214,14 @@ def kernel_source_hash(kernel: str | None = None):
 def kernels_per_step(strategy: str, n: int, n_bins: int) -> int:
     """The library's kernels in one call (zeroing is cudaMemsetAsync): one fused kernel; with it the
     expansion of the 32-byte cells, or the expansion and the redo of packed ones where warp combining
-    takes them (16 bytes a bin within 60 MB, 1 M records, a record per six bins); run boundaries, their
-    scan and the remainder for the owner strategy; sample, levels, candidates, hot table, main pass,
-    tiles and finish for the partition, and the split where the histogram has more than 384 ranges of
-    2^15 bins."""
+    takes them (the library's rule on bins and records); run boundaries, their scan and the remainder
+    for the owner strategy; sample, levels, candidates, hot table, main pass, tiles and finish for the
+    partition, and the split where the histogram has more than 384 ranges of 2^15 bins."""
     if strategy == "global_atomic":
-        return 3 if n >= 1_000_000 and n >= n_bins // 6 and 16 * n_bins <= 60 << 20 else 1
+        most = (60 << 20) // 16
+        need = (max(500_000, 3 * n_bins // 2) if n_bins <= 600_000
+                else max(1_000_000, min(9 * n_bins // 2, 6_000_000, 5 * (most - n_bins))))
+        return 3 if n_bins <= most and n >= need else 1
     if strategy == "partition":
         return 8 if -(-n_bins >> 15) > 384 else 7
     return {"atomic_cell": 2, "owner": 4}.get(strategy, 1)

@@ -272,13 +272,24 @@ static cudaError_t run_cells(int lk, const RecArgs &r, const TableArgs &ta_tab, 
 // Warp combining through packed cells (one reduction an update instead of two,
 // see HistArgs::packed) while the cells stay in L2, which keeps about 60 MB for
 // one set of accesses (3.6 M bins: 58 MB of cells stay, 86 MB of output arrays
-// did not): 16 bytes a bin are zeroed and read besides the outputs' 24 written.
-// 20 M uniform records over 3.6 M bins 411 -> 186 us, 10 M over 100 K 159 -> 98,
-// 1 M over 3.6 M 87 -> 78. Below a record per six bins or 1 M records the
-// expansion costs more than the reductions it saves (100 K over 3.6 M: 59 us,
-// straight into the outputs 42).
-static bool packed_pays(uint64_t n_bins, uint64_t n) {
-    return 16 * n_bins <= (60ull << 20) && n >= 1000000 && n >= n_bins / 6;
+// do not). 16 bytes a bin are zeroed and read besides the outputs' 24 written,
+// so it takes records to pay for bins. Packed and straight into the outputs, us
+// (uniform; skewed):
+//   300 K bins: 200 K records 27, 29; 30, 34. 1 M 36, 40; 51, 69. 25 M 186, 278
+//   500 K: 500 K 36, 37; 44, 55. 2 M 57, 60; 63, 64    5 K: 200 K 26, 24. 500 K 30, 33
+//   600 K: 500 K 39, 37; 47, 50. 1 M 41, 40; 60, 69. 3 M 63, 66; 75, 77
+//   1 M: 1 M 48, 41; 74, 81. 4.5 M 77, 78; 102, 98. 7 M 91, 104; 130, 129
+//   1.5 M: 1 M 54, 41; 78, 74. 4.5 M 85, 78; 112, 103. 7 M 98, 103; 139, 136
+//   2.5 M: 2 M 83, 68; 94, 82. 6 M 100, 101; 138, 133. 25 M 204, 281; 369, 381
+// and where the output arrays no longer stay in L2 it pays sooner:
+//   3.1 M: 2.5 M 89, 80; 108, 94. 4 M 93, 102; 123, 112
+//   3.6 M: 1 M 77, 75; 97, 96. 2 M 93, 91; 105, 95. 3 M 93, 108; 116, 112. 10 M 129, 229
+//   3.9 M: 1 M 80, 87; 103, 109. 3 M 98, 126; 118, 121. 25 M 228, 548; 386, 403
+bool packed_pays(uint64_t n_bins, uint64_t n) {
+    const uint64_t most = (60ull << 20) / 16;
+    if (n_bins > most) return false;
+    if (n_bins <= 600000) return n >= std::max<uint64_t>(500000, 3 * n_bins / 2);
+    return n >= std::max<uint64_t>(1000000, std::min({9 * n_bins / 2, uint64_t(6000000), 5 * (most - n_bins)}));
 }
 // Not while the stream is captured: a graph with an allocation of its own can be
 // instantiated only once at a time.

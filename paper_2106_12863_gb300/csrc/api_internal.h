@@ -74,6 +74,8 @@ bool rows_apart(const HistArgs &h);
 // of n records: below 2^32 updates, whose bytes stay below 2^64. Past that the
 // byte totals wrap, and cells that lost 2^64 bytes and a count could agree.
 inline bool packed_countable(uint64_t n, bool two_dir) { return n < (two_dir ? 1ull << 31 : 1ull << 32); }
+// Whether a call of n records over n_bins bins on warp combining gains by packed cells.
+bool packed_pays(uint64_t n_bins, uint64_t n);
 sinet_status zero_outputs(const sinet_hist_params *p, const sinet_hist_out *o, cudaStream_t s);
 // The shared-memory form of a table that has one: its leaf form, else its toggle form.
 int staged_lookup(const sinet_prefix_table *t);

@@ -83,6 +83,8 @@ int plan_packed_slice(uint64_t n, uint32_t n_bins, int two_dir) {
     return slice_packed(v[0]);
 }
 
+int call_packed(uint64_t n_bins, uint64_t n) { return packed_pays(n_bins, n); }
+
 // plan_cells for a batch of n_slices slices: records, bins, strategy, accumulate,
 // ready word and "same outputs as slice 0" of each; pack[i] is its decision.
 void plan_batch_cells(const uint64_t *n, const uint32_t *bins, const int32_t *strategy, const uint8_t *accumulate,

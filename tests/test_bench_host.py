@@ -59,5 +59,5 @@ def test_kernels_per_step():
     # the partition with and without its split: 384 ranges of 2^15 bins are the line
     assert [k("partition", 10**9, b) for b in (86_400_000, (384 << 15) + 1, 384 << 15)] == [8, 8, 7]
     # warp combining with and without packed cells
-    assert [k("global_atomic", n, b) for n, b in ((10**6, 3_600_000), (999_999, 3_600_000), (10**8, 86_400_000))] == [3, 1, 1]
+    assert [k("global_atomic", n, b) for n, b in ((10**7, 3_600_000), (10**6, 3_600_000), (10**8, 86_400_000))] == [3, 1, 1]
     assert [k(s, 10**8, 10**6) for s in ("priv_tile", "atomic_cell", "owner")] == [1, 2, 4]
