@@ -521,17 +521,14 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
             ta.margin = T / 6;
             // and, where the records of a bin are many, as many records as an eighth
             // of the tile's bins hold, while every CTA has eight chunks: the flush
-            // takes longer than such a chunk's own span costs. Inclusive, 180 M
-            // records over 1.55 M bins 896 -> 728 us; classified, 115 M over 2 M
-            // 516 -> 439, over 600 K 539 -> 529. Past 512 records a bin it gives
-            // nothing (96 K bins: 547, and 551-575 with longer chunks), and with
-            // four chunks a CTA 20 M records over 96 K bins took 134, not 130
-            const uint64_t per_bin = r.g.n / p->n_bins;
-            uint64_t records = 3ull * T;
-            if (per_bin < 512) {
-                const uint64_t eighth = r.g.n / (16ull * ds->sm_count);
-                records = std::max(records, std::min<uint64_t>({65535, T / 8 * per_bin, eighth}));
-            }
+            // takes longer than such a chunk's own span costs. Classified, 115 M
+            // records over 2 M bins 359 -> 322 us, over 600 K 349 -> 305, over 96 K
+            // 346 -> 308; fused, 600 K 455 -> 423; inclusive, 180 M over 1.55 M
+            // 772 -> 670. With four chunks a CTA 20 M records over 96 K bins took
+            // 134, not 130
+            const uint64_t eighth = r.g.n / (16ull * ds->sm_count), per_bin = r.g.n / p->n_bins;
+            const uint64_t records =
+                std::max<uint64_t>(3ull * T, std::min<uint64_t>({65535, T / 8 * per_bin, eighth}));
             ta.iters = (uint32_t)std::max<uint64_t>(1, records / (4ull * ct.block));
         }
         // a chunk stays within 65,535 records: a tile entry counts in 16 bits
@@ -544,8 +541,16 @@ static sinet_status run_hist(const sinet_prefix_table *t, int lk, const RecArgs 
         if (ta.full) {
             const uint64_t rounds = (all + ta.iters - 1) / ta.iters;
             ta.iters = (uint32_t)((all + rounds - 1) / rounds);
-        } else {
+        } else if (r.g.n) {
             ta.iters = (uint32_t)std::min<uint64_t>(ta.iters, all);
+            // Half of the room that the chunk's own bins leave goes below its first
+            // record, which may itself be late: with a sixth of the tile there, one
+            // chunk in three of records up to 500 bins early or late had some below
+            // it, and long chunks over few bins made each of those costly. 115 M
+            // classified records over 600 K bins 484 -> 307 us, over 96 K 496 -> 347;
+            // fused 517 -> 425; sparser than 2,000 bins a chunk as before
+            const uint64_t span = 4ull * ct.block * ta.iters * p->n_bins / r.g.n, T = ta.tile_bins;
+            if (span < T) ta.margin = (uint32_t)std::max<uint64_t>(T / 6, (T - span) / 2);
         }
     }
     if (strat == SINET_STRAT_SORT_REDUCE && r.g.n * (h.two_dir ? 2ull : 1ull) >= 0xFFFFFFF0ull)
