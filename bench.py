@@ -220,7 +220,7 @@ def kernels_per_step(strategy: str, n: int, n_bins: int) -> int:
     if strategy == "global_atomic":
         most = (60 << 20) // 16
         need = (max(500_000, 3 * n_bins // 2) if n_bins <= 600_000
-                else max(1_000_000, min(9 * n_bins // 2, 6_000_000, 5 * (most - n_bins))))
+                else min(9 * n_bins // 2, 6_000_000, 5 * (4_200_000 - n_bins)))
         return 3 if n_bins <= most and n >= need else 1
     if strategy == "partition":
         return 8 if -(-n_bins >> 15) > 384 else 7

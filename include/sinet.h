@@ -64,7 +64,7 @@ typedef enum {
     SINET_STRAT_GLOBAL_ATOMIC = 1, /* warp match + reduce (while that saves updates), then global
                                       atomics; not accumulating, outside a capture, with up to
                                       3.9 M bins and enough records (0.5 M to 0.9 M up to 0.6 M
-                                      bins, 1 M to 6 M beyond) they go to stream-ordered scratch of 16
+                                      bins, 1.3 M to 6 M beyond) they go to stream-ordered scratch of 16
                                       bytes a bin, then expanded (straight to the outputs when
                                       it cannot be had) */
     SINET_STRAT_PRIV_TILE = 2,     /* shared-memory bin tile per chunk (time-sorted input) */

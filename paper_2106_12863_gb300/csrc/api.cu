@@ -289,7 +289,7 @@ bool packed_pays(uint64_t n_bins, uint64_t n) {
     const uint64_t most = (60ull << 20) / 16;
     if (n_bins > most) return false;
     if (n_bins <= 600000) return n >= std::max<uint64_t>(500000, 3 * n_bins / 2);
-    return n >= std::max<uint64_t>(1000000, std::min({9 * n_bins / 2, uint64_t(6000000), 5 * (most - n_bins)}));
+    return n >= std::min({9 * n_bins / 2, uint64_t(6000000), 5 * (4200000 - n_bins)});
 }
 // Not while the stream is captured: a graph with an allocation of its own can be
 // instantiated only once at a time.

@@ -142,3 +142,11 @@ def test_two_threads_with_tables_of_two_sizes(strategy):
         t.join()
     assert not errors, errors
     assert sinet.sinet_device_status() == 0
+
+
+@pytest.mark.parametrize("n,n_bins", [(1_339_200, 3_932_160), (1_339_199, 3_932_160), (3_000_001, 3_600_001),
+                                      (2_700_004, 600_001), (900_000, 600_000), (899_999, 600_000), (500_000, 333_333)])
+def test_packed_at_the_edges_of_the_rule(orc, n, n_bins):
+    """Calls on both sides of the lines in records and bins from which packed cells are taken."""
+    rng = np.random.default_rng(n)
+    _check(orc, _records(rng.integers(0, n_bins + 1, n), rng.integers(0, 1 << 32, n), 1), n_bins, policy=sinet.INCLUSIVE)
