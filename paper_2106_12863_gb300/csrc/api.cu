@@ -229,7 +229,8 @@ static uint32_t table_smem(const sinet_prefix_table *t, int lk) {
 // miss, and one sector per update instead of two halves the DRAM traffic.
 static const uint64_t kCellMinHistBytes = 256ull << 20;
 // Smaller ones take the partition from these sizes on (see auto_rule).
-static const uint64_t kPartMinHistBytes = 90ull << 20, kPartMinRecords = 6000000;
+static const uint64_t kPartMinHistBytes = 90ull << 20;
+static uint64_t part_min_records(bool accumulate) { return accumulate ? 8000000 : 6000000; }
 
 // Hot-key cache of the warp-aggregated atomic kernel: 2^9 sets x 4 ways
 // (32 KB of shared memory per CTA).
@@ -336,11 +337,13 @@ static int auto_rule(const sinet_hist_params *p, const RecArgs &r, uint32_t cap,
     // Measured, us, the partition against the faster of combining and plain
     // reductions: 20 M records over 21.6 M bins 455 / 1,074; skewed, over 8.6 M
     // bins 286 / 352; 100 M over 86.4 M 1,588 / 6,054, skewed 1,044 / 2,163. Its
-    // fixed costs (about 80 us) lose below some 5 M records, and to warp
+    // fixed costs (about 80 us) lose below some 5 M records, or 8 M where there is
+    // nothing to zero (accumulating, 6 M over 3.9 M bins 170 / 153, skewed over
+    // 10.6 M 147 / 134; 8 M 189 / 194, 164 / 164), and to warp
     // combining where bins outnumber records
     const bool large = 24 * p->n_bins >= kCellMinHistBytes;
     if ((large ? r.g.n >= p->n_bins / 4
-               : !capturing && 24 * p->n_bins >= kPartMinHistBytes && r.g.n >= kPartMinRecords) &&
+               : !capturing && 24 * p->n_bins >= kPartMinHistBytes && r.g.n >= part_min_records(p->accumulate != 0)) &&
         rows_apart(h)) {
         PartPlan probe{};
         if (plan_partition(lk, tsm, r, h, 0, ds->sm_count, ds->smem_optin, false, &probe) == cudaSuccess)
