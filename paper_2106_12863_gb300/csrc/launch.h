@@ -133,6 +133,7 @@ struct SortPlan {
     uint32_t passes;       // 8-bit digit passes
     uint64_t emit_tiles;   // tiles of the emit kernel
     uint64_t sort_tiles;   // tiles of a radix pass (upper bound)
+    bool few;              // so few that a pass is one kernel
     size_t scratch_bytes;  // total scratch needed
     // offsets into scratch
     size_t zero_bytes;     // of the scratch's start, zeroed by every run

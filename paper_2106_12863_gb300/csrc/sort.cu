@@ -23,6 +23,11 @@ constexpr int kSortItems = 16;
 constexpr int kSortTile = kSortThreads * kSortItems;  // 4096 keys
 constexpr int kWarps = kSortThreads / 32;
 
+// Inputs of up to so many sort tiles take a radix pass as one kernel, with a
+// look-back per digit, instead of three: launches are their time. 30 K records
+// over 400 K bins 103 us with three kernels a pass, 76 with one; 1 M 128, 111;
+// 2 M (489 tiles) 154, 139; 3 M (733) 180, 179; 16 M 640, 940.
+constexpr uint64_t kFewTiles = 512;
 constexpr uint64_t kFlagAgg = 1ull << 54;
 constexpr uint64_t kFlagIncl = 2ull << 54;
 constexpr uint64_t kValMask = (1ull << 54) - 1;
@@ -48,6 +53,22 @@ __device__ __forceinline__ uint64_t ready_word(const uint64_t *p, uint64_t w, ui
         w = ld_word(p);
     }
     return w;
+}
+
+// Exclusive prefix of `own` over all predecessor tiles by one thread, a
+// predecessor a step (words `stride` apart).
+__device__ uint64_t look_back(uint64_t *st, uint64_t stride, uint64_t tile, uint64_t own, uint32_t epoch,
+                              uint32_t *status) {
+    st_word(st + tile * stride, status_word(epoch, tile ? kFlagAgg : kFlagIncl, own));
+    uint64_t excl = 0;
+    for (uint64_t p = tile; p > 0; --p) {
+        const uint64_t *at = st + (p - 1) * stride;
+        const uint64_t w = ready_word(at, ld_word(at), epoch, status);
+        excl += w & kValMask;
+        if (w & kFlagIncl) break;
+    }
+    if (tile) st_word(st + tile * stride, status_word(epoch, kFlagIncl, excl + own));
+    return excl;
 }
 
 // Exclusive prefix of `own` over all predecessor tiles (decoupled look-back) by a
@@ -80,8 +101,9 @@ struct SortArgs {
     uint32_t *digit_hist;    // [passes][256]
     uint64_t *emit_status;   // [emit tiles]
     uint32_t *tile_digits;   // [256][sort tiles] keys per digit and tile of a pass, then their first places
+    uint64_t *digit_status;  // [sort tiles][256] look-back words, in the same place (k_radix_pass<true>)
     uint64_t sort_tiles;
-    uint64_t *counters;      // [0] n_emit, [1] emit ticket
+    uint64_t *counters;      // [0] n_emit, [1] emit ticket, [2 + p] pass tickets
     uint32_t n_bins;
     uint32_t passes;
 };
@@ -297,21 +319,28 @@ __global__ void __launch_bounds__(1024) k_radix_place(SortArgs sa, uint32_t p) {
     }
 }
 
+// FEW: small inputs, whose time is launches, take the pass as one kernel: tiles
+// are numbered as CTAs claim them, and a thread per digit looks back over the
+// tiles before its own (sa.digit_status) for the digit's first place.
+template <bool FEW>
 __global__ void __launch_bounds__(kSortThreads, 3) k_radix_pass(SortArgs sa, uint32_t p, const uint32_t *kin,
                                                                 const uint32_t *vin, uint32_t *kout,
-                                                                uint32_t *vout) {
+                                                                uint32_t *vout, uint32_t *status) {
     __shared__ uint32_t s_key[kSortTile];
     __shared__ uint32_t s_val[kSortTile];
     __shared__ uint32_t s_whist[kWarps][257];
     __shared__ uint32_t s_lstart[256];
     __shared__ uint32_t s_gpos[256];
     __shared__ uint32_t s_warp[kWarps];
+    __shared__ uint32_t s_tile;
     const uint64_t n = sa.counters[0];
     for (uint32_t i = threadIdx.x; i < kWarps * 257; i += blockDim.x) (&s_whist[0][0])[i] = 0;
-    const uint64_t tile = blockIdx.x, tbase = tile * kSortTile;
-    if (tbase >= n) return;  // block-uniform
+    if (FEW && threadIdx.x == 0)
+        s_tile = (uint32_t)atomicAdd(reinterpret_cast<unsigned long long *>(sa.counters + 2 + p), 1ull);
     __syncthreads();
-    s_gpos[threadIdx.x] = sa.tile_digits[(uint64_t)threadIdx.x * sa.sort_tiles + tile];
+    const uint64_t tile = FEW ? s_tile : blockIdx.x, tbase = tile * kSortTile;
+    if (tbase >= n) return;  // block-uniform; no tile behind it either
+    if (!FEW) s_gpos[threadIdx.x] = sa.tile_digits[(uint64_t)threadIdx.x * sa.sort_tiles + tile];
     const uint32_t shift = 8 * p;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t lt_mask = (1u << lane) - 1u;
@@ -353,6 +382,11 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_radix_pass(SortArgs sa, uin
     uint32_t tot;
     const uint32_t lstart = block_excl_scan_256(cnt, s_warp, tot);
     s_lstart[d] = lstart;
+    if (FEW) {
+        uint32_t all;
+        const uint32_t first = block_excl_scan_256(sa.digit_hist[p * 256 + d], s_warp, all);
+        s_gpos[d] = first + (uint32_t)look_back(sa.digit_status + d, 256, tile, cnt, p + 1, status);
+    }
     __syncthreads();
     // scatter into the tile in sorted order
 #pragma unroll
@@ -512,9 +546,12 @@ SortPlan plan_sort_reduce(uint64_t n, uint32_t n_bins, bool two_dir) {
     off += al(8 * (p.emit_tiles + 1));
     p.zero_bytes = off;
     p.off_tile_digits = off;
-    // the counts take 4 bytes a digit and tile; 8 are laid out, because the
-    // largest input that fits a caller's fixed scratch follows from this size
+    // counts take 4 bytes a digit and tile, look-back words 8; 8 are laid out for
+    // both, because the largest input that fits a caller's fixed scratch follows
+    // from this size
     off += al(8ull * 256 * p.sort_tiles);
+    p.few = p.sort_tiles <= kFewTiles;
+    if (p.few) p.zero_bytes = off;
     p.off_keys0 = off;
     off += al(4 * p.n_emit_max + 4);
     p.off_vals0 = off;
@@ -536,6 +573,7 @@ cudaError_t run_sort_reduce(int lk, const RecArgs &r, const TableArgs &t, const 
     sa.digit_hist = reinterpret_cast<uint32_t *>(base + plan.off_hist);
     sa.emit_status = reinterpret_cast<uint64_t *>(base + plan.off_emit_status);
     sa.tile_digits = reinterpret_cast<uint32_t *>(base + plan.off_tile_digits);
+    sa.digit_status = reinterpret_cast<uint64_t *>(base + plan.off_tile_digits);
     sa.sort_tiles = plan.sort_tiles;
     sa.keys0 = reinterpret_cast<uint32_t *>(base + plan.off_keys0);
     sa.vals0 = reinterpret_cast<uint32_t *>(base + plan.off_vals0);
@@ -574,9 +612,14 @@ cudaError_t run_sort_reduce(int lk, const RecArgs &r, const TableArgs &t, const 
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     uint32_t *kin = sa.keys0, *vin = sa.vals0, *kout = sa.keys1, *vout = sa.vals1;
     for (uint32_t p = 0; p < plan.passes; ++p) {
-        k_radix_count<<<(unsigned)plan.sort_tiles, kSortThreads, 0, c.stream>>>(sa, p, kin);
-        k_radix_place<<<256, 1024, 0, c.stream>>>(sa, p);
-        k_radix_pass<<<(unsigned)plan.sort_tiles, kSortThreads, 0, c.stream>>>(sa, p, kin, vin, kout, vout);
+        const unsigned tiles = (unsigned)plan.sort_tiles;
+        if (plan.few) {
+            k_radix_pass<true><<<tiles, kSortThreads, 0, c.stream>>>(sa, p, kin, vin, kout, vout, c.status);
+        } else {
+            k_radix_count<<<tiles, kSortThreads, 0, c.stream>>>(sa, p, kin);
+            k_radix_place<<<256, 1024, 0, c.stream>>>(sa, p);
+            k_radix_pass<false><<<tiles, kSortThreads, 0, c.stream>>>(sa, p, kin, vin, kout, vout, c.status);
+        }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         uint32_t *tk = kin, *tv = vin;
         kin = kout;

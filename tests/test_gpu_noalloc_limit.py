@@ -58,3 +58,27 @@ def test_the_largest_input_stays_the_largest(policy, dirs):
     with pytest.raises(sinet.SinetError, match="BUDGET"):
         run(sinet.sinet_discriminate_histogram_noalloc, n + 1)
     table.close()
+
+
+@pytest.mark.parametrize("policy,dirs", [("EXCLUSIVE", 1), ("INCLUSIVE", 2)])
+@pytest.mark.parametrize("tiles", [1, 2, 511, 512, 513, 1500])
+@pytest.mark.parametrize("over", [-1, 0, 1])
+def test_plain_path_at_the_edges_of_tiles(tiles, over, policy, dirs):
+    """One kernel a radix pass up to 512 sort tiles of 4,096 pairs, three beyond: equal to plain reductions."""
+    n, n_bins = tiles * 4096 // dirs + over, 70_001
+    table = sinet.PrefixTable(np.array([0], np.uint32), np.array([1], np.uint8))
+    g = torch.Generator(device="cuda").manual_seed(tiles)
+    ts = torch.randint(0, n_bins + 5, (n,), dtype=torch.int64, device="cuda", generator=g)
+    # every record routed: inside to outside, or (both directions) inside to inside
+    src = torch.randint(1, 1 << 31, (n,), dtype=torch.int64, device="cuda", generator=g).to(torch.int32)
+    dst = src.clone() if dirs == 2 else torch.full((n,), -1, dtype=torch.int32, device="cuda")
+    by = torch.randint(-(1 << 31), 1 << 31, (n,), dtype=torch.int64, device="cuda", generator=g).to(torch.int32)
+    outs = []
+    for strategy in ("sort_reduce", "atomic_noagg"):
+        outs.append(sinet.Histogram(n_bins))
+        p = sinet.HistParams(0, 1, n_bins, policy=getattr(sinet, policy), strategy=strategy)
+        sinet.discriminate_histogram(table, ts, src, dst, by, p, outs[-1])
+    for k in ("count", "bytes", "stats"):
+        assert torch.equal(getattr(outs[0], k), getattr(outs[1], k)), k
+    assert sinet.sinet_device_status() == 0
+    table.close()
