@@ -26,8 +26,11 @@ __global__ void __launch_bounds__(512, LK == LK_INTERVAL ? 2 : 3) k_discriminate
                                                          uint32_t *status) {
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ uint64_t bar;
+    __shared__ unsigned long long s_cnt[4];
+    if (threadIdx.x < 4) s_cnt[threadIdx.x] = 0;
     Classifier<LK> C;
     if (!C.init(t, smem, &bar, status)) return;  // table not staged: the status word says so
+    __syncthreads();
     const uint64_t pol = policy_evict_first();
     uint32_t n_rec = 0, n_src = 0, n_dst = 0, n_both = 0;  // 8 x the thread's records of each kind
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
@@ -69,13 +72,8 @@ __global__ void __launch_bounds__(512, LK == LK_INTERVAL ? 2 : 3) k_discriminate
         n_both += __popc(S & D);
     }
     // at most 2^40 records over at least one 512-thread CTA per SM: a thread's counts stay below 2^28
-    const uint32_t v[4] = {n_rec - n_src - n_dst + n_both, n_src - n_both, n_dst - n_both, n_both};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const uint32_t sum = __reduce_add_sync(kFull, v[k] / 8);
-        if ((threadIdx.x & 31) == 0 && sum)
-            atomicAdd(reinterpret_cast<unsigned long long *>(counts + k), (unsigned long long)sum);
-    }
+    const uint32_t v[4] = {(n_rec - n_src - n_dst + n_both) / 8, (n_src - n_both) / 8, (n_dst - n_both) / 8, n_both / 8};
+    flush_cta(s_cnt, v, counts);
 }
 
 // Watch list (the blocklist views of Section 6, as a filter): a record whose
@@ -407,16 +405,7 @@ __global__ void __launch_bounds__(1024) k_fused_tile(RecArgs r, TableArgs t, His
     }
     // (a thread's counts stay far below 2^32: at most 2^40 records over the grid)
     const uint32_t cc[6] = {n_rec - n_src - n_dst + n_both, n_src - n_both, n_dst - n_both, n_both, oor[0], oor[1]};
-    // one global add a CTA and counter: from every warp, 29,000 of them queued at
-    // the same addresses when all CTAs end together (20 M records 135 us, 113 so)
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const uint32_t v = __reduce_add_sync(kFull, cc[k]);
-        if (lane == 0 && v) atomicAdd(s_cnt + k, (unsigned long long)v);
-    }
-    __syncthreads();
-    if (threadIdx.x < 6 && s_cnt[threadIdx.x])
-        atomicAdd(reinterpret_cast<unsigned long long *>(h.stats) + threadIdx.x, s_cnt[threadIdx.x]);
+    flush_cta(s_cnt, cc, h.stats);
 }
 
 // ---------------------------------------------------------------------------

@@ -480,6 +480,22 @@ __device__ __forceinline__ void drain_packed(uint64_t &cc, uint32_t &oorp, unsig
     oorp = 0;
 }
 
+// The CTA's totals of N per-thread counters added to `to`: one global add a CTA and
+// counter. From every warp, up to 29,000 additions queue at the same few words
+// when all CTAs end together, 10 us of a small call's time. `s`: N words of shared
+// memory, zero since a barrier. Reached by every thread.
+template <int N>
+__device__ __forceinline__ void flush_cta(unsigned long long *s, const uint32_t (&v)[N], uint64_t *to) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const uint32_t x = __reduce_add_sync(kFull, v[k]);
+        if ((threadIdx.x & 31) == 0 && x) atomicAdd(s + k, (unsigned long long)x);
+    }
+    __syncthreads();
+    if (threadIdx.x < N && s[threadIdx.x])
+        atomicAdd(reinterpret_cast<unsigned long long *>(to) + threadIdx.x, s[threadIdx.x]);
+}
+
 // Warp totals of the per-thread counters into stats (lane 0 of every warp).
 __device__ __forceinline__ void flush_counters(uint64_t *stats, const uint32_t cc[4],
                                                const uint32_t oor[2], bool with_oor) {
