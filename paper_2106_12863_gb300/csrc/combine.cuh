@@ -78,13 +78,18 @@ __device__ __forceinline__ uint32_t update_agg(const HistArgs &h, HotCache &hc, 
     return c - 1;
 }
 
-// The warp's totals of updates and of their bytes added to `to` (lane 0).
-__device__ __forceinline__ void flush_totals(uint64_t *to, uint64_t updates, uint64_t bytes) {
+// The warp's totals of updates and of their bytes, in lane 0.
+__device__ __forceinline__ void warp_totals(uint64_t &updates, uint64_t &bytes) {
 #pragma unroll
     for (int d = 16; d; d >>= 1) {
         updates += __shfl_down_sync(kFull, updates, d);
         bytes += __shfl_down_sync(kFull, bytes, d);
     }
+}
+
+// The same added to `to` (lane 0).
+__device__ __forceinline__ void flush_totals(uint64_t *to, uint64_t updates, uint64_t bytes) {
+    warp_totals(updates, bytes);
     if ((threadIdx.x & 31) == 0 && updates) {
         red_add_u64(to, updates);
         red_add_u64(to + 1, bytes);

@@ -98,11 +98,6 @@ __device__ __forceinline__ void watch_filter(const Classifier<LK_INTERVAL_GLOBAL
     }
 }
 
-__device__ __forceinline__ void flush_filtered(uint64_t *stats, uint32_t flt) {
-    const uint32_t v = __reduce_add_sync(kFull, flt);
-    if ((threadIdx.x & 31) == 0 && v) atomicAdd(reinterpret_cast<unsigned long long *>(stats + 6), (unsigned long long)v);
-}
-
 // With AGG a warp combines its lanes' equal keys only while that saves global
 // updates: combining costs about twice the instructions of a plain reduction,
 // which uniform records over many bins would pay for nothing, and without it
@@ -129,6 +124,9 @@ __global__ void __launch_bounds__(256, 3) k_fused_atomic(RecArgs r, TableArgs t,
     if (!C.init(t, smem, &bar, status)) return;  // table not staged: the status word says so
     Classifier<LK_INTERVAL_GLOBAL> W;
     if (WATCH) W.attach(wt, nullptr);
+    __shared__ unsigned long long s_cnt[9];  // stats[0 .. 6], then updates and their bytes
+    if (threadIdx.x < 9) s_cnt[threadIdx.x] = 0;
+    __syncthreads();
     const uint64_t pol = policy_evict_first();
     uint32_t cc[4] = {0, 0, 0, 0}, oor[2] = {0, 0}, flt = 0;
     const uint32_t lane = threadIdx.x & 31;
@@ -143,8 +141,8 @@ __global__ void __launch_bounds__(256, 3) k_fused_atomic(RecArgs r, TableArgs t,
                 gadd(h, key & 1u, key >> 1, c, s);
             });
         }
-        flush_counters(h.stats, cc, oor, true);
-        if (WATCH) flush_filtered(h.stats, flt);
+        const uint32_t v[7] = {cc[0], cc[1], cc[2], cc[3], oor[0], oor[1], flt};
+        flush_cta(s_cnt, v, h.stats);
         return;
     }
     // hot-key cache after the staged table
@@ -220,7 +218,12 @@ __global__ void __launch_bounds__(256, 3) k_fused_atomic(RecArgs r, TableArgs t,
         uint64_t updates = 0;
 #pragma unroll
         for (int k = 0; k < 4; ++k) updates += (uint64_t)cc[k] * __popc((h.policy >> (8 * k)) & 3u);
-        flush_totals(h.pack_sums, updates - oor[0] - oor[1], sum);
+        updates -= oor[0] + (uint64_t)oor[1];
+        warp_totals(updates, sum);
+        if (lane == 0 && updates) {
+            atomicAdd(s_cnt + 7, (unsigned long long)updates);
+            atomicAdd(s_cnt + 8, (unsigned long long)sum);
+        }
     }
     if (AGG == AGG_CACHE) {
         __syncthreads();
@@ -229,8 +232,9 @@ __global__ void __launch_bounds__(256, 3) k_fused_atomic(RecArgs r, TableArgs t,
             if (c) gadd(h, hc.keys[i] & 1u, hc.keys[i] >> 1, c, (uint64_t)hc.hi[i] << 32 | hc.lo[i]);
         }
     }
-    flush_counters(h.stats, cc, oor, true);
-    if (WATCH) flush_filtered(h.stats, flt);
+    const uint32_t v[7] = {cc[0], cc[1], cc[2], cc[3], oor[0], oor[1], flt};
+    flush_cta(s_cnt, v, h.stats);
+    if (h.packed && threadIdx.x < 2) red_add_u64(h.pack_sums + threadIdx.x, s_cnt[7 + threadIdx.x]);
 }
 
 // One record into entry e of a tile: byte sum's low word, then count << 16 with
@@ -454,6 +458,9 @@ __global__ void __launch_bounds__(256) k_cells_expand(HistArgs h, uint32_t accum
 // aligned and n_bins a multiple of four); else one, four rows in flight.
 template <bool VEC>
 __global__ void __launch_bounds__(256) k_pack_expand(HistArgs h) {
+    __shared__ unsigned long long s_sum[2];
+    if (threadIdx.x < 2) s_sum[threadIdx.x] = 0;
+    __syncthreads();
     uint64_t updates = 0, bytes = 0;
     constexpr uint64_t kMask = (1ull << kPackBits) - 1;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, first = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -507,7 +514,13 @@ __global__ void __launch_bounds__(256) k_pack_expand(HistArgs h) {
             }
         }
     }
-    flush_totals(h.pack_sums + 2, updates, bytes);
+    warp_totals(updates, bytes);
+    if ((threadIdx.x & 31) == 0 && updates) {
+        atomicAdd(s_sum, (unsigned long long)updates);
+        atomicAdd(s_sum + 1, (unsigned long long)bytes);
+    }
+    __syncthreads();  // one global add a CTA (see flush_cta)
+    if (threadIdx.x < 2) red_add_u64(h.pack_sums + 2 + threadIdx.x, s_sum[threadIdx.x]);
 }
 
 __device__ __forceinline__ bool pack_right(const uint64_t *s) {
