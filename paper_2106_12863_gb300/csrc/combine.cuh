@@ -20,7 +20,9 @@ struct HotCache {
     static constexpr uint32_t kWays = 4;
     static constexpr uint32_t kSlotBytes = 16;
 
-    __device__ __forceinline__ bool add(uint32_t key, uint32_t c, uint64_t s) {
+    // False, and nothing added, when no slot takes the key; `claim`: a key that
+    // the cache does not hold may take a free one.
+    __device__ __forceinline__ bool add(uint32_t key, uint32_t c, uint64_t s, bool claim = true) {
         const uint32_t set = (key * 0x9E3779B1u) >> (32 - set_bits);
         uint32_t *kp = keys + kWays * set;
         uint4 k4;
@@ -28,7 +30,7 @@ struct HotCache {
                      : "=r"(k4.x), "=r"(k4.y), "=r"(k4.z), "=r"(k4.w)
                      : "r"(smem_u32(kp)));
         int way = k4.x == key ? 0 : k4.y == key ? 1 : k4.z == key ? 2 : k4.w == key ? 3 : -1;
-        if (way < 0) {
+        if (way < 0 && claim) {
             const uint32_t cur[4] = {k4.x, k4.y, k4.z, k4.w};
             bool tried = false;
 #pragma unroll
@@ -59,9 +61,10 @@ struct HotCache {
 // leader that adds the group's count (popc of the peer mask) and byte sum.
 // Byte sums are reduced as two 16-bit halves so 32 values of up to 2^32 - 1
 // cannot overflow the 32-bit warp reduction; they are recombined in 64 bits.
-// CACHED: the group's sum goes to the hot-key cache if it takes the key.
+// CACHED: the group's sum goes to the hot-key cache if it takes the key (2: if it
+// has it or the group is of several lanes).
 // Returns (in the leader) the global updates this saved against one per lane.
-template <bool CACHED>
+template <int CACHED>
 __device__ __forceinline__ uint32_t update_agg(const HistArgs &h, HotCache &hc, uint32_t key, uint32_t b) {
     const uint32_t peers = __match_any_sync(kFull, key);
     if (key == kNoKey) return 0u;
@@ -73,7 +76,7 @@ __device__ __forceinline__ uint32_t update_agg(const HistArgs &h, HotCache &hc, 
         s = (uint64_t)lo + ((uint64_t)hi << 16);
     }
     if ((threadIdx.x & 31) != (uint32_t)(__ffs(peers) - 1)) return 0u;
-    if (CACHED && hc.add(key, c, s)) return c;
+    if (CACHED && hc.add(key, c, s, CACHED == 1 || c > 1)) return c;
     gadd(h, key & 1u, key >> 1, c, s);
     return c - 1;
 }

@@ -109,11 +109,12 @@ __device__ __forceinline__ void watch_filter(const Classifier<LK_INTERVAL_GLOBAL
 //          doubled the heavy day's time behind one). (10 M records over
 //          100 K bins, packed cells: uniform 97 us, Zipf 157; always combining,
 //          into the output arrays, 159 and 199.)
-//   AGG 2: no cache, for inputs too small to fill one (an hour of 1 M records
-//          over 3.6 M bins: 75 us, with the cache 95); none saved, and it goes
-//          without (a hot bin's warps all save some).
-enum : int { AGG_NONE = 0, AGG_CACHE = 1, AGG_WARP = 2 };
+//   AGG 2: a small cache that only keys which repeat within a warp enter (8 KB a
+//          CTA leave its L1); none saved, and the warp goes without (a hot bin's
+//          warps all save some). run_fused_atomic says where each is taken.
+enum : int { AGG_NONE = 0, AGG_CACHE = 1, AGG_REPEATS = 2 };
 constexpr uint32_t kRecheck = 16;
+constexpr uint32_t kRepeatSetBits = 7;
 
 template <int LK, int AGG, bool WATCH>
 __global__ void __launch_bounds__(256, 3) k_fused_atomic(RecArgs r, TableArgs t, HistArgs h,
@@ -154,15 +155,13 @@ __global__ void __launch_bounds__(256, 3) k_fused_atomic(RecArgs r, TableArgs t,
     hc.lo = hc.cnt + slots;
     hc.hi = hc.lo + slots;
     hc.set_bits = cache_set_bits;
-    if (AGG == AGG_CACHE) {
-        for (uint32_t i = threadIdx.x; i < slots; i += blockDim.x) {
-            hc.keys[i] = kNoKey;
-            hc.cnt[i] = 0;
-            hc.lo[i] = 0;
-            hc.hi[i] = 0;
-        }
-        __syncthreads();
+    for (uint32_t i = threadIdx.x; i < slots; i += blockDim.x) {
+        hc.keys[i] = kNoKey;
+        hc.cnt[i] = 0;
+        hc.lo[i] = 0;
+        hc.hi[i] = 0;
     }
+    __syncthreads();
     uint64_t sum = 0;  // bytes of the thread's updates, for the check of packed cells
     uint32_t plain = 0;  // quads the warp takes next without combining
     // warp-uniform trip count: every lane reaches the warp-synchronous updates
@@ -203,11 +202,11 @@ __global__ void __launch_bounds__(256, 3) k_fused_atomic(RecArgs r, TableArgs t,
             if (h.packed) sum += (uint64_t)__popc(dirs) * Q.by[j];
             const uint32_t key = dirs ? (bin << 1 | (dirs & 1u ? 0u : 1u)) : kNoKey;
             if (AGG == AGG_CACHE && dirs) saved += 1u << 16;
-            saved += update_agg<AGG == AGG_CACHE>(h, hc, key, Q.by[j]);
+            saved += update_agg<AGG>(h, hc, key, Q.by[j]);
             if (h.two_dir) {
                 const bool both = dirs == 3u;
                 if (__any_sync(kFull, both))
-                    update_agg<AGG == AGG_CACHE>(h, hc, both ? (bin << 1 | 1u) : kNoKey, Q.by[j]);
+                    update_agg<AGG>(h, hc, both ? (bin << 1 | 1u) : kNoKey, Q.by[j]);
             }
         }
         saved = __reduce_add_sync(kFull, saved);
@@ -225,12 +224,10 @@ __global__ void __launch_bounds__(256, 3) k_fused_atomic(RecArgs r, TableArgs t,
             atomicAdd(s_cnt + 8, (unsigned long long)sum);
         }
     }
-    if (AGG == AGG_CACHE) {
-        __syncthreads();
-        for (uint32_t i = threadIdx.x; i < slots; i += blockDim.x) {
-            const uint32_t c = hc.cnt[i];
-            if (c) gadd(h, hc.keys[i] & 1u, hc.keys[i] >> 1, c, (uint64_t)hc.hi[i] << 32 | hc.lo[i]);
-        }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < slots; i += blockDim.x) {
+        const uint32_t c = hc.cnt[i];
+        if (c) gadd(h, hc.keys[i] & 1u, hc.keys[i] >> 1, c, (uint64_t)hc.hi[i] << 32 | hc.lo[i]);
     }
     const uint32_t v[7] = {cc[0], cc[1], cc[2], cc[3], oor[0], oor[1], flt};
     flush_cta(s_cnt, v, h.stats);
@@ -720,19 +717,27 @@ cudaError_t run_fused_atomic(int lk, bool agg, const RecArgs &r, const TableArgs
     int grid = 0;
     cudaError_t e;
     const TableArgs none{};
-    // below about 17 records a thread (the kernel's grid is three CTAs an SM) a
-    // cache costs more to fill and flush than it saves
-    const int mode = !agg ? AGG_NONE : r.g.n < 13000ull * (uint64_t)c.sm_count ? AGG_WARP : AGG_CACHE;
+    // The large cache pays where updates miss L2 (outputs beyond about 90 MB) and
+    // hot keys therefore must not reach memory, from half a million records on:
+    // small and large, us (uniform; skewed), 1.2 M records over 5.7 M bins 78, 83;
+    // 73, 64. 5 M 183, 187; 132, 117. 8 M over 40 M 667, 666; 346, 301. In L2 the
+    // small one is better or equal: 1.2 M over 600 K 32, 40; 42, 42. 13 M over
+    // 100 K 104, 112; 168, 184. 130 M over 600 K 811, 769; 1,382, 1,530. And with a
+    // watch list, whose lookups want the L1 that the large one takes: 60 M over
+    // 600 K with 1,500 entries 775, 2,465
+    const bool large = !watch && 24ull * h.n_bins > (90ull << 20) && r.g.n >= 500000;
+    const int mode = !agg ? AGG_NONE : large ? AGG_CACHE : AGG_REPEATS;
+    const uint32_t bits = large ? cache_set_bits : std::min<uint32_t>(cache_set_bits, kRepeatSetBits);
 #define SINET_ATOM(L, A, WA)                                                                    \
     if (lk == L && mode == A && (watch != nullptr) == WA) {                                     \
         size_t smem = ((Classifier<L>::smem_bytes(t) + 15u) & ~15u) +                           \
-                      (A == AGG_CACHE ? (size_t)HotCache::kSlotBytes * (HotCache::kWays << cache_set_bits) : 0ull); \
+                      (A ? (size_t)HotCache::kSlotBytes * (HotCache::kWays << bits) : 0ull);    \
         if ((e = launch(k_fused_atomic<L, A, WA>, smem, c, grid)) != cudaSuccess) return e;     \
-        k_fused_atomic<L, A, WA><<<grid, c.block, smem, c.stream>>>(r, t, h, cache_set_bits,     \
+        k_fused_atomic<L, A, WA><<<grid, c.block, smem, c.stream>>>(r, t, h, bits,               \
                                                                    WA ? *watch : none, c.status); \
         return cudaGetLastError();                                                              \
     }
-#define SINET_ATOM2(L, WA) SINET_ATOM(L, AGG_CACHE, WA) SINET_ATOM(L, AGG_WARP, WA) SINET_ATOM(L, AGG_NONE, WA)
+#define SINET_ATOM2(L, WA) SINET_ATOM(L, AGG_CACHE, WA) SINET_ATOM(L, AGG_REPEATS, WA) SINET_ATOM(L, AGG_NONE, WA)
     SINET_ATOM2(LK_INTERVAL, false)
     SINET_ATOM2(LK_LEAF2, false)
     SINET_ATOM2(LK_LEAF4, false)
