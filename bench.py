@@ -218,10 +218,9 @@ def kernels_per_step(strategy: str, n: int, n_bins: int) -> int:
     for the owner strategy; sample, levels, candidates, hot table, main pass, tiles and finish for the
     partition, and the split where the histogram has more than 384 ranges of 2^15 bins."""
     if strategy == "global_atomic":
-        most = (60 << 20) // 16
-        need = (max(500_000, 3 * n_bins // 2) if n_bins <= 600_000
-                else min(9 * n_bins // 2, 6_000_000, 5 * (4_200_000 - n_bins)))
-        return 3 if n_bins <= most and n >= need else 1
+        need = (300_000 if n_bins <= 600_000
+                else min(11 * (n_bins - 550_000) // 2, 4_500_000, 3 * (4_250_000 - n_bins)))
+        return 3 if 16 * n_bins <= 60 << 20 and n >= need else 1
     if strategy == "partition":
         return 8 if -(-n_bins >> 15) > 384 else 7
     return {"atomic_cell": 2, "owner": 4}.get(strategy, 1)

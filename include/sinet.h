@@ -63,10 +63,10 @@ typedef enum {
     SINET_STRAT_AUTO = 0,          /* autotuner / heuristics choose */
     SINET_STRAT_GLOBAL_ATOMIC = 1, /* warp match + reduce (while that saves updates), then global
                                       atomics; not accumulating, outside a capture, with up to
-                                      3.9 M bins and enough records (0.5 M to 0.9 M up to 0.6 M
-                                      bins, 1.3 M to 6 M beyond) they go to stream-ordered scratch of 16
-                                      bytes a bin, then expanded (straight to the outputs when
-                                      it cannot be had) */
+                                      3.9 M bins and enough records (0.3 M up to 0.6 M bins,
+                                      up to 4.5 M beyond) they go to stream-ordered scratch of
+                                      16 bytes a bin, then expanded (straight to the outputs
+                                      when it cannot be had) */
     SINET_STRAT_PRIV_TILE = 2,     /* shared-memory bin tile per chunk (time-sorted input) */
     SINET_STRAT_SORT_REDUCE = 3,   /* plain path: discriminate, radix sort, reduce by key */
     SINET_STRAT_SMEM_FULL = 4,     /* whole histogram privatised in shared memory (small n_bins) */

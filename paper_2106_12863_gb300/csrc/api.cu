@@ -276,21 +276,19 @@ static cudaError_t run_cells(int lk, const RecArgs &r, const TableArgs &ta_tab, 
 // do not). 16 bytes a bin are zeroed and read besides the outputs' 24 written,
 // so it takes records to pay for bins. Packed and straight into the outputs, us
 // (uniform; skewed):
-//   300 K bins: 200 K records 27, 29; 30, 34. 1 M 36, 40; 51, 69. 25 M 186, 278
-//   500 K: 500 K 36, 37; 44, 55. 2 M 57, 60; 63, 64    5 K: 200 K 26, 24. 500 K 30, 33
-//   600 K: 500 K 39, 37; 47, 50. 1 M 41, 40; 60, 69. 3 M 63, 66; 75, 77
-//   1 M: 1 M 48, 41; 74, 81. 4.5 M 77, 78; 102, 98. 7 M 91, 104; 130, 129
-//   1.5 M: 1 M 54, 41; 78, 74. 4.5 M 85, 78; 112, 103. 7 M 98, 103; 139, 136
-//   2.5 M: 2 M 83, 68; 94, 82. 6 M 100, 101; 138, 133. 25 M 204, 281; 369, 381
+//   5 K bins: 200 K records 25, 24; 26, 26. 400 K 25, 26; 26, 27. 20 M 193, 362; 249, 265
+//   600 K: 200 K 28, 27; 30, 30. 400 K 28, 29; 30, 31. 3 M 41, 50; 62, 66
+//   1 M: 1 M 35, 34; 46, 43. 2 M 40, 41; 56, 54. 4.5 M 53, 64; 81, 82
+//   1.5 M: 1 M 40, 34; 49, 44. 3 M 50, 49; 71, 66. 6 M 69, 82; 102, 99
+//   2.5 M: 2 M 53, 47; 69, 60. 4.5 M 68, 73; 96, 94. 20 M 157, 223; 255, 263
 // and where the output arrays no longer stay in L2 it pays sooner:
-//   3.1 M: 2.5 M 89, 80; 108, 94. 4 M 93, 102; 123, 112
-//   3.6 M: 1 M 77, 75; 97, 96. 2 M 93, 91; 105, 95. 3 M 93, 108; 116, 112. 10 M 129, 229
-//   3.9 M: 1 M 80, 87; 103, 109. 3 M 98, 126; 118, 121. 25 M 228, 548; 386, 403
+//   3.1 M: 2 M 58, 58; 71, 63. 4.5 M 73, 92; 96, 92
+//   3.6 M: 1 M 55, 52; 64, 56. 2 M 60, 70; 73, 74. 9 M 101, 190; 145, 153
+//   3.9 M: 700 K 55, 54; 62, 58. 1.5 M 60, 71; 72, 72. 20 M 178, 420; 265, 288
 bool packed_pays(uint64_t n_bins, uint64_t n) {
-    const uint64_t most = (60ull << 20) / 16;
-    if (n_bins > most) return false;
-    if (n_bins <= 600000) return n >= std::max<uint64_t>(500000, 3 * n_bins / 2);
-    return n >= std::min({9 * n_bins / 2, uint64_t(6000000), 5 * (4200000 - n_bins)});
+    if (16 * n_bins > (60ull << 20)) return false;
+    if (n_bins <= 600000) return n >= 300000;
+    return n >= std::min({11 * (n_bins - 550000) / 2, uint64_t(4500000), 3 * (4250000 - n_bins)});
 }
 // Not while the stream is captured: a graph with an allocation of its own can be
 // instantiated only once at a time.

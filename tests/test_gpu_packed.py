@@ -144,8 +144,8 @@ def test_two_threads_with_tables_of_two_sizes(strategy):
     assert sinet.sinet_device_status() == 0
 
 
-@pytest.mark.parametrize("n,n_bins", [(1_339_200, 3_932_160), (1_339_199, 3_932_160), (3_000_001, 3_600_001),
-                                      (2_700_004, 600_001), (900_000, 600_000), (899_999, 600_000), (500_000, 333_333)])
+@pytest.mark.parametrize("n,n_bins", [(953_520, 3_932_160), (953_519, 3_932_160), (1_949_999, 3_600_001),
+                                      (275_011, 600_002), (300_000, 600_000), (299_999, 600_000), (300_001, 333_333)])
 def test_packed_at_the_edges_of_the_rule(orc, n, n_bins):
     """Calls on both sides of the lines in records and bins from which packed cells are taken."""
     rng = np.random.default_rng(n)

@@ -123,9 +123,8 @@ def test_where_packed_cells_pay(plans):
     import bench
 
     pays = lambda bins, n: bool(plans.call_packed(ctypes.c_uint64(bins), ctypes.c_uint64(n)))
-    lines = {1: 500_000, 400_000: 600_000, 600_000: 900_000, 600_001: 2_700_004, 1_000_000: 4_500_000,
-             1_500_000: 6_000_000, 2_500_000: 6_000_000, 3_100_000: 5_500_000, 3_600_000: 3_000_000,
-             3_932_160: 1_339_200}
+    lines = {1: 300_000, 600_000: 300_000, 600_002: 275_011, 1_000_000: 2_475_000, 1_500_000: 4_500_000,
+             2_500_000: 4_500_000, 3_100_000: 3_450_000, 3_600_000: 1_950_000, 3_932_160: 953_520}
     for bins, line in lines.items():
         assert pays(bins, line) and not pays(bins, line - 1), bins
         assert [bench.kernels_per_step("global_atomic", n, bins) for n in (line - 1, line)] == [1, 3]
