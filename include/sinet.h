@@ -547,7 +547,7 @@ sinet_status sinet_histogram_sparse(const sinet_hist_out *in, uint64_t n_bins, u
  * partition for unsorted input over a histogram of 256 MB or more with at
  * least one record per four bins (the 32-byte cells where the partition's
  * limits are exceeded, or where its scratch does not fit the free device
- * memory at the call) or of 90 MB or more with at least 6 M records, 8 M accumulating, warp
+ * memory at the call) or of 90 MB or more with at least 6 M records, 10 M accumulating, warp
  * combining otherwise). The answer is for outputs whose rows share no memory
  * and a stream that is not captured: rows that overlap, and below 256 MB a
  * capture, take warp combining where this names the partition. No kernel runs.

@@ -230,7 +230,7 @@ static uint32_t table_smem(const sinet_prefix_table *t, int lk) {
 static const uint64_t kCellMinHistBytes = 256ull << 20;
 // Smaller ones take the partition from these sizes on (see auto_rule).
 static const uint64_t kPartMinHistBytes = 90ull << 20;
-static uint64_t part_min_records(bool accumulate) { return accumulate ? 8000000 : 6000000; }
+static uint64_t part_min_records(bool accumulate) { return accumulate ? 10000000 : 6000000; }
 
 // Hot-key cache of the warp-aggregated atomic kernel: 2^9 sets x 4 ways
 // (32 KB of shared memory per CTA).
@@ -332,13 +332,13 @@ static int auto_rule(const sinet_hist_params *p, const RecArgs &r, uint32_t cap,
     if (p->hints & SINET_HINT_TIME_SORTED) return SINET_STRAT_PRIV_TILE;
     // unsorted input over a histogram whose packed cells do not stay in L2 (see
     // packed_pays): the hot/cold partition, else (far beyond L2) the cells.
-    // Measured, us, the partition against the faster of combining and plain
-    // reductions: 20 M records over 21.6 M bins 455 / 1,074; skewed, over 8.6 M
-    // bins 286 / 352; 100 M over 86.4 M 1,588 / 6,054, skewed 1,044 / 2,163. Its
-    // fixed costs (about 80 us) lose below some 5 M records, or 8 M where there is
-    // nothing to zero (accumulating, 6 M over 3.9 M bins 170 / 153, skewed over
-    // 10.6 M 147 / 134; 8 M 189 / 194, 164 / 164), and to warp
-    // combining where bins outnumber records
+    // Measured, us, the partition against warp combining (uniform; skewed): 6 M
+    // records over 3.9 M bins 163, 166; 132, 127, over 10.6 M 217, 283; 166, 147;
+    // 13 M over 7.5 M 269, 454; 211, 227; 20 M over 21.6 M 455, 1,074; 100 M over
+    // 86.4 M 1,588, 6,054; 1,044, 2,163. Its fixed costs (about 80 us) lose below
+    // some 6 M records, or 10 M where there is nothing to zero (accumulating, 8 M
+    // over 3.9 M bins 190, 170; 142, 120, 10 M over 7.5 M 249, 325; 181, 149), and
+    // to warp combining where bins outnumber records
     const bool large = 24 * p->n_bins >= kCellMinHistBytes;
     if ((large ? r.g.n >= p->n_bins / 4
                : !capturing && 24 * p->n_bins >= kPartMinHistBytes && r.g.n >= part_min_records(p->accumulate != 0)) &&

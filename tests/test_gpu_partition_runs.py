@@ -86,7 +86,7 @@ def test_auto_without_room_for_scratch(orc, free_memory, n_bins, accumulate):
 
     table = sinet.PrefixTable(*NET)
     rng = np.random.default_rng(n_bins)
-    rec = _records(rng.integers(0, n_bins, 8_000_001), 3)
+    rec = _records(rng.integers(0, n_bins, 10_000_001), 3)
     d = to_dev(rec)
     p = sinet.HistParams(0, 1, n_bins, accumulate=accumulate)
     assert sinet.auto_strategy(table, len(rec["ts"]), p) == "partition"
@@ -106,7 +106,7 @@ def test_streams_accumulating_into_one_histogram():
     import torch
 
     table = sinet.PrefixTable(np.array([0], np.uint32), np.array([1], np.uint8))
-    n, n_bins, calls = 8_100_001, 4_000_000, 40
+    n, n_bins, calls = 10_200_001, 4_000_000, 40
     g = torch.Generator(device="cuda").manual_seed(1)
     p = sinet.HistParams(0, 1, n_bins, accumulate=True)
     assert [sinet.auto_strategy(table, k, p) for k in (n, 300_000)] == ["partition", "global_atomic"]
@@ -131,9 +131,9 @@ def test_streams_accumulating_into_one_histogram():
 
 
 def test_auto_lines_of_the_partition():
-    """From 90 MiB on: 6 M records, 8 M where the outputs are added to."""
+    """From 90 MiB on: 6 M records, 10 M where the outputs are added to."""
     table = sinet.PrefixTable(*NET)
     auto = lambda n, bins, acc: sinet.auto_strategy(table, n, sinet.HistParams(0, 1, bins, accumulate=acc))
-    for acc, line in ((False, 6_000_000), (True, 8_000_000)):
+    for acc, line in ((False, 6_000_000), (True, 10_000_000)):
         assert [auto(n, 3_932_160, acc) for n in (line - 1, line)] == ["global_atomic", "partition"]
         assert auto(line, 3_932_159, acc) == "global_atomic"
