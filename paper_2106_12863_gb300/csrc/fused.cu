@@ -103,15 +103,13 @@ __device__ __forceinline__ void watch_filter(const Classifier<LK_INTERVAL_GLOBAL
 // which uniform records over many bins would pay for nothing, and without it
 // the hottest bin of skewed records serialises its reductions. Every kRecheck-th
 // quad of a warp that goes without is combined all the same, and decides anew.
-//   AGG 1: hot keys are kept in a shared-memory cache; fewer than a fifth of a
-//          quad's updates saved, and the warp goes without (a share of what is
-//          routed, since a watch list may leave little: a fixed 32 of the 128
-//          doubled the heavy day's time behind one). (10 M records over
-//          100 K bins, packed cells: uniform 97 us, Zipf 157; always combining,
-//          into the output arrays, 159 and 199.)
+//   AGG 1: hot keys are kept in a shared-memory cache; fewer than a fifth of the
+//          quad's routed updates saved, and the warp goes without.
 //   AGG 2: a small cache that only keys which repeat within a warp enter (8 KB a
 //          CTA leave its L1); none saved, and the warp goes without (a hot bin's
-//          warps all save some). run_fused_atomic says where each is taken.
+//          warps all save some). 10 M records over 100 K bins, packed cells:
+//          uniform 85 us, skewed 133; always combining, into the output arrays,
+//          159 and 199. run_fused_atomic says where each is taken.
 enum : int { AGG_NONE = 0, AGG_CACHE = 1, AGG_REPEATS = 2 };
 constexpr uint32_t kRecheck = 16;
 constexpr uint32_t kRepeatSetBits = 7;
@@ -260,8 +258,8 @@ __device__ __forceinline__ void tile_add(uint32_t *tlo, uint32_t *thi, uint32_t 
 // takes no branch per record, and the next quad's loads overlap this one's
 // adds. With `full`, chunks are as long as the 16-bit counts allow: the whole
 // tile is flushed for each. 50 M records into 3,600 bins of 1 s, both
-// directions: 327 -> 215 us; 100 M classified records at 10 ms 439 -> 397; the
-// 400 M sorted day 2.53 -> 2.49 ms.
+// directions: 327 -> 215 us; with the counters' sums per CTA (flush_cta), 100 M
+// classified records at 10 ms 439 -> 372; the 400 M sorted day 2.53 -> 2.27-2.40 ms.
 template <int LK, bool W1>
 __global__ void __launch_bounds__(1024) k_fused_tile(RecArgs r, TableArgs t, HistArgs h, TileArgs ta,
                                                      uint32_t *status) {
@@ -737,19 +735,21 @@ cudaError_t run_fused_atomic(int lk, bool agg, const RecArgs &r, const TableArgs
                                                                    WA ? *watch : none, c.status); \
         return cudaGetLastError();                                                              \
     }
-#define SINET_ATOM2(L, WA) SINET_ATOM(L, AGG_CACHE, WA) SINET_ATOM(L, AGG_REPEATS, WA) SINET_ATOM(L, AGG_NONE, WA)
-    SINET_ATOM2(LK_INTERVAL, false)
-    SINET_ATOM2(LK_LEAF2, false)
-    SINET_ATOM2(LK_LEAF4, false)
-    SINET_ATOM2(LK_TOGGLE2, false)
-    SINET_ATOM2(LK_PML, false)
-    SINET_ATOM2(LK_INTERVAL_GLOBAL, false)
-    SINET_ATOM2(LK_CLASS_IN, false)
-    SINET_ATOM2(LK_INTERVAL, true)
-    SINET_ATOM2(LK_LEAF2, true)
-    SINET_ATOM2(LK_LEAF4, true)
-    SINET_ATOM2(LK_TOGGLE2, true)
-    SINET_ATOM2(LK_INTERVAL_GLOBAL, true)
+#define SINET_ATOM2(L) SINET_ATOM(L, AGG_CACHE, false) SINET_ATOM(L, AGG_REPEATS, false) SINET_ATOM(L, AGG_NONE, false)
+#define SINET_ATOM3(L) SINET_ATOM(L, AGG_REPEATS, true) SINET_ATOM(L, AGG_NONE, true)
+    SINET_ATOM2(LK_INTERVAL)
+    SINET_ATOM2(LK_LEAF2)
+    SINET_ATOM2(LK_LEAF4)
+    SINET_ATOM2(LK_TOGGLE2)
+    SINET_ATOM2(LK_PML)
+    SINET_ATOM2(LK_INTERVAL_GLOBAL)
+    SINET_ATOM2(LK_CLASS_IN)
+    SINET_ATOM3(LK_INTERVAL)
+    SINET_ATOM3(LK_LEAF2)
+    SINET_ATOM3(LK_LEAF4)
+    SINET_ATOM3(LK_TOGGLE2)
+    SINET_ATOM3(LK_INTERVAL_GLOBAL)
+#undef SINET_ATOM3
 #undef SINET_ATOM2
 #undef SINET_ATOM
     return cudaErrorInvalidValue;

@@ -5,7 +5,8 @@
 //              becomes a (key = d * n_bins + bin, bytes) pair, compacted with a
 //              decoupled look-back scan; per-pass digit counts are taken here.
 //   2. sort:   LSD radix sort of the pairs, 8-bit digits: per pass the tiles'
-//              digit counts, their scan, and the move (ranking by warp ballots).
+//              digit counts, their scan, and the move (ranking by warp ballots);
+//              few tiles take a pass as one kernel (kFewTiles).
 //   3. reduce: reduce-by-key over the sorted pairs (segmented scan per tile);
 //              each run's count and byte sum is scattered into the dense
 //              histogram (runs that cross a tile edge are added atomically).
