@@ -259,7 +259,7 @@ __device__ __forceinline__ void tile_add(uint32_t *tlo, uint32_t *thi, uint32_t 
 // adds. With `full`, chunks are as long as the 16-bit counts allow: the whole
 // tile is flushed for each. 50 M records into 3,600 bins of 1 s, both
 // directions: 327 -> 215 us; with the counters' sums per CTA (flush_cta), 100 M
-// classified records at 10 ms 439 -> 372; the 400 M sorted day 2.53 -> 2.27-2.40 ms.
+// classified records at 10 ms 439 -> 372; the 400 M sorted day 2.53 -> 2.27-2.47 ms.
 template <int LK, bool W1>
 __global__ void __launch_bounds__(1024) k_fused_tile(RecArgs r, TableArgs t, HistArgs h, TileArgs ta,
                                                      uint32_t *status) {
